@@ -468,12 +468,15 @@ __global__ void __launch_bounds__(32) k_trsm(const int4* __restrict__ tasks, int
 // schur_tile_epilogue.
 template <int TILE>
 struct SchurCfg {
-  static constexpr int WARPS_M = TILE == 64 ? 2 : 1;
-  static constexpr int WARPS_N = TILE == 64 ? 2 : 1;
-  static constexpr int WT = TILE / WARPS_M;       // warp tile edge: 32 or 16
+  // four warps on every tile, one per FP64 unit of an SM: a 32 x 32 tile with K = 64 is 65,536
+  // multiply-adds, 52 us on the one unit of a single warp.  64 x 64 2D Laplacian, 11 levels of
+  // 32-tiles: 0.57 ms with one warp, 0.13 ms with four and the few-tile rule of schur_cls.
+  static constexpr int WARPS_M = 2;
+  static constexpr int WARPS_N = 2;
+  static constexpr int WT = TILE / WARPS_M;       // warp tile edge: 32, 16 or 8
   static constexpr int MB = WT / 8;               // 8x8 blocks per warp edge
   static constexpr int THREADS = 32 * WARPS_M * WARPS_N;
-  static constexpr int KC = 32;                   // K chunk staged in shared memory
+  static constexpr int KC = TILE == 64 ? 32 : 64;  // K chunk staged in shared memory
   static constexpr int LDS = TILE + 8;            // padded stride (bank spread)
 };
 
@@ -960,7 +963,11 @@ static void schur_cls(int cls, bool f32, const int4* tasks, int ntasks, int* que
     // FP64 128-wide tasks run as four 64 x 64 virtual tasks of the DMMA kernel
     if (cls == kTile128) schur_f64_t<64, OWNER>(tasks, ntasks, queue, sns, mats, st, 2);
     else if (cls == kTile64) schur_f64_t<64, OWNER>(tasks, ntasks, queue, sns, mats, st);
-    else if (cls == kTile32) schur_f64_t<32, OWNER>(tasks, ntasks, queue, sns, mats, st);
+    else if (cls == kTile32 && 4 * ntasks > 3 * 152)
+      schur_f64_t<32, OWNER>(tasks, ntasks, queue, sns, mats, st);
+    // few 32-tiles: as 16 x 16 virtual tasks, which spread over the idle SMs' FP64 units (20 us
+    // a 32-tile on one SM, 5 us a 16-tile) while there are at most three of them per SM
+    else if (cls == kTile32) schur_f64_t<16, OWNER>(tasks, ntasks, queue, sns, mats, st, 2);
     else schur_f64_t<16, OWNER>(tasks, ntasks, queue, sns, mats, st);
   }
 }

@@ -523,8 +523,8 @@ int ensure_solve_ws(chol_num* f, int64_t nrhs) {
   return CHOL_OK;
 }
 
-// Work buffers of one device solve of k <= 32 right-hand sides: the work-queue counters
-// (3 per level, zeroed by the solve), y and w (n x k each), the backward partial sums (the
+// Work buffers of one device solve of k <= 32 right-hand sides: the arrival counters
+// (zeroed by the solve), y and w (n x k each), the backward partial sums (the
 // most backward tasks of a level x W x k) and, for owner assembly, the forward staging (the
 // most forward tasks of a level x kSolveRows x k; null otherwise).
 struct SolveBufs {
@@ -563,29 +563,31 @@ int enqueue_solve_seq(chol_ctx* c, const chol_num* f, int k, const double* B, in
   const bool inv = f->d_dinv != nullptr;
   const double vec = 8.0 * n * k;
   const SolveTrace tr{c, trace};
-  CK(cudaMemsetAsync(bf.sq, 0, solve_counters(S) * sizeof(int), st));
+  const int64_t counters = (int64_t)solve_counters(S);
+  CK(cudaMemsetAsync(bf.sq, 0, counters * sizeof(int), st));
   tr.begin(kProfPerm);
   chol::launch_gather_perm(B, ldb, sym->dev.perm, scale, n, k, bf.y, st);
   tr.end(kProfPerm, 2 * vec + 4.0 * n);
   for (int32_t l = 0; l < S.nlev; l++) {
-    int cnt;
+    int cnt, nsup;
     const int4* t = task_ptr(sym, chol::kTaskFwd, l, &cnt);
+    const int4* dg = task_ptr(sym, chol::kTaskPotrf, l, &nsup);
     tr.begin(kProfFwd);
-    chol::launch_fwd(t, cnt, bf.sq + 3 * l, f->d_sn, n, k, S.lvl_maxw[l], bf.y, bf.w, bf.fstage,
-                     inv, f32, st);
+    chol::launch_fwd(t, cnt, dg, nsup, f->d_sn, n, k, S.lvl_maxw[l], bf.y, bf.w, bf.fstage, counters, inv,
+                     f32, st);
     if (bf.fstage)
       chol::launch_fwd_gather(sym->dev.fg_row + S.fg_lvl[l], sym->dev.fg_ptr + S.fg_lvl[l],
                               sym->dev.fg_ent, S.fg_lvl[l + 1] - S.fg_lvl[l], n, k, bf.fstage,
                               bf.y, st);
     tr.end(kProfFwd, S.lvl_panel_bytes[l] * (f32 ? 0.5 : 1.0));
   }
-  int* arrive = bf.sq + solve_arrive_offset(S);
   for (int32_t l = S.nlev - 1; l >= 0; l--) {
-    int nb;
+    int nb, nsup;
     const int4* tb = task_ptr(sym, chol::kTaskBwd, l, &nb);
+    const int4* dg = task_ptr(sym, chol::kTaskPotrf, l, &nsup);
     tr.begin(kProfBwd);
-    chol::launch_bwd(tb, nb, bf.sq + 3 * l + 1, f->d_sn, n, k, W, S.lvl_maxw[l], bf.w, bf.part,
-                     arrive, inv, f32, st);
+    chol::launch_bwd(tb, nb, dg, nsup, S.task_off[chol::kTaskBwd][l], f->d_sn, n, k, W, S.lvl_maxw[l], bf.w, bf.part, bf.sq, counters, inv,
+                     f32, st);
     tr.end(kProfBwd, S.lvl_panel_bytes[l] * (f32 ? 0.5 : 1.0));
   }
   tr.begin(kProfPerm);
@@ -940,7 +942,7 @@ int refine_group(chol_ctx* c, std::vector<GroupItem>& g) {
 namespace chol {
 
 // Workspace, in doubles, of a device-pointer solve of k <= 32 right-hand sides: the
-// work-queue counters (3 per level), y and w (n k each), the backward partials (max tasks
+// arrival counters, y and w (n k each), the backward partials (max tasks
 // of a level x W x k) and, for owner assembly, the forward staging (max tasks of a level x
 // kSolveRows x k).
 size_t solve_scratch_doubles(const chol_num* f, int64_t k) {
@@ -959,7 +961,7 @@ int enqueue_solve_ws(chol_ctx* c, const chol_num* f, int k, const double* B, int
   const Sym& S = sym->S;
   const size_t qd = (rt::solve_counters(S) * sizeof(int) + 255) / 256 * 256 / sizeof(double);
   rt::SolveBufs bf;
-  bf.sq = reinterpret_cast<int*>(ws);  // work-queue counters, then the vectors
+  bf.sq = reinterpret_cast<int*>(ws);  // arrival counters, then the vectors
   bf.y = ws + qd;
   bf.w = bf.y + (size_t)S.n * k;
   bf.part = bf.w + (size_t)S.n * k;

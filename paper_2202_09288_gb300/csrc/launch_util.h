@@ -1,4 +1,4 @@
-// launch_util.h -- grid sizing of the task kernels.
+// launch_util.h -- grid sizing of the task kernels, and programmatic dependent launch.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -17,5 +17,34 @@ inline int task_grid(K kernel, int threads, size_t smem, int ntasks) {
   (void)smem;
   return ntasks;
 }
+
+// Launches k so that its CTAs may start while the kernel before it in the stream still runs
+// (programmatic dependent launch), as soon as every CTA of that kernel has started and called
+// pdl_launch_dependents (or, without that call, has ended).  k may read what no kernel since the last
+// ordinary launch writes; for everything else it calls pdl_wait first, which returns when the
+// kernel before has ended and its writes are visible -- and with it every earlier one, since a
+// kernel that calls pdl_wait in all its CTAs cannot end before the one before it.
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl(void (*k)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                              Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k, KArgs(args)...);
+}
+
+#ifdef __CUDACC__
+__device__ __forceinline__ void pdl_launch_dependents() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+#endif
 
 }  // namespace chol

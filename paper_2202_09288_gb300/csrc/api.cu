@@ -338,7 +338,7 @@ int enqueue_levels(chol_ctx* c, const TaskView& v, const SnDev* sns, const MatDe
     const int4* t = v.level(chol::kTaskPotrf, l, &cnt);
     if (cnt > 0) {
       prof_begin(c, kp);
-      chol::launch_potrf(t, cnt, q, sns, mats, v.max_width, f32, tau, trsm_oz ? oy : nullptr,
+      chol::launch_potrf(t, cnt, sns, mats, v.max_width, f32, tau, trsm_oz ? oy : nullptr,
                          oy_rows, st);
       prof_end(c, kp, v.flops[chol::kTaskPotrf][l], 0.0);
     }

@@ -35,10 +35,10 @@ __global__ void k_assemble(const double* __restrict__ vals, const int64_t* __res
 }
 
 // ---- diagonal-block Cholesky ---------------------------------------------------------------
-// Cost model on this part: an FP64 warp instruction occupies its SM sub-partition's FP64 unit
-// for ~64 cycles whether 1 or 32 lanes are active, a dependent DFMA chain advances one step
-// per ~64 cycles, and the library's double sqrt and reciprocal take ~690 and ~440 cycles.
-// The factorization is therefore organized so that (a) the serial per-column chain holds as
+// Cost model on this part (measured): a warp's FP64 instruction takes ~65 cycles, dependent or not;
+// an SM's FP64 unit takes one per 19 cycles from all its warps together (so eight busy warps wait
+// ~150 cycles each); the library's double sqrt and reciprocal take ~690 and ~440 cycles.  The
+// factorization is therefore organized so that (a) the serial per-column chain holds as
 // few FP64 instructions as possible and (b) the bulk of the work runs with every lane busy.
 
 // FMA in the block's precision.
@@ -49,16 +49,23 @@ __device__ __forceinline__ float fma_t(float a, float b, float c) { return fmaf(
 // With r = 1 - p y0^2, p^{-1/2} = y0 (1 - r)^{-1/2} = y0 (1 + r/2 + 3r^2/8 + O(r^3)); the seed
 // has |r| < 2^-20, so the dropped term is below 2^-58 relative, and the result is within an
 // ulp or so.  p is first scaled by an even power of two into [1, 4) with integer exponent
-// arithmetic (no FP32 overflow or underflow) and the result scaled back the same way: four
-// FP64 instructions in all.  Subnormal, infinite and NaN p take the library path.
+// arithmetic (no FP32 overflow or underflow) and the result scaled back the same way; the
+// FP32 <-> FP64 conversions are integer arithmetic too (exact, but for the seed's argument,
+// truncated to 24 bits): four FP64 instructions in all, where each conversion would be one more
+// of ~64 cycles on the serial chain.  Subnormal, infinite and NaN p take the library path.
+__device__ __forceinline__ double widen_normal(float x) {  // a positive normal float
+  const uint32_t b = __float_as_uint(x);
+  return __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
+}
 __device__ __forceinline__ double pivot_rsqrt(double p) {
   const int hi = __double2hiint(p), lo = __double2loint(p);
   const int ebits = (hi >> 20) & 0x7ff;
   if (ebits == 0 || ebits == 0x7ff) return 1.0 / sqrt(p);
   const int s = (ebits - 1023) & ~1;  // even, so that p 2^-s lies in [1, 4)
-  const double ps = __hiloint2double(hi - s * (1 << 20), lo);
-  const float y0f = rsqrtf((float)ps);
-  const double y0 = (double)y0f, c1 = (double)(0.5f * y0f), c2 = (double)(0.375f * y0f);
+  const int his = hi - s * (1 << 20);
+  const double ps = __hiloint2double(his, lo);
+  const float y0f = rsqrtf(__uint_as_float((((uint32_t)his - 0x38000000u) << 3) | ((uint32_t)lo >> 29)));
+  const double y0 = widen_normal(y0f), c1 = widen_normal(0.5f * y0f), c2 = widen_normal(0.375f * y0f);
   const double h = ps * y0;
   const double r = fma(-h, y0, 1.0);
   const double q = fma(r, c2, c1);  // y0/2 + 3 y0 r / 8
@@ -70,6 +77,11 @@ __device__ __forceinline__ float pivot_rsqrt(float p) {
   const float y0 = rsqrtf(p);
   const float r = fmaf(-p * y0, y0, 1.f);
   return fmaf(0.5f * y0, r, y0);
+}
+// p > 0 without the FP64 unit (NaN and zero of either sign are not)
+__device__ __forceinline__ bool positive(double p) {
+  const long long b = __double_as_longlong(p);
+  return b > 0 && b <= 0x7ff0000000000000ll;
 }
 
 // Threads of a POTRF CTA: warp 0 finishes the next column, the others update the trailing
@@ -93,15 +105,19 @@ __device__ __forceinline__ void build_update_table(uint16_t* tab, int n) {
 __host__ __device__ constexpr size_t update_table_bytes(int w) {
   return w > 2 ? (size_t)(w - 2) * (w - 1) / 2 * sizeof(uint16_t) : 0;
 }
-// FP64 POTRF's shared memory: the block (w^2 doubles), the update table, then (8-byte
-// aligned) the w reciprocals of the diagonal that the in-place inverse uses
-__host__ __device__ constexpr size_t potrf_rd_offset(int w) {
-  return ((size_t)w * w * sizeof(double) + update_table_bytes(w) + 7) / 8 * 8;
+
+// The mixed kernel's table follows the FP64 block of a redo, which overlays the FP32 one (leading
+// dimension 64 up to 64 columns: 64 n floats)
+__host__ __device__ constexpr size_t potrf_mixed_tab_offset(int w) {
+  return (size_t)w * w * sizeof(double) > (size_t)64 * 64 * sizeof(float)
+             ? (size_t)w * w * sizeof(double)
+             : (size_t)64 * 64 * sizeof(float);
 }
 
 // Right-looking Cholesky of the n x n block A (shared memory, column-major A[c * n + r]; only
 // the lower triangle is read or written; n <= 128) with a one-column lookahead and one barrier
-// per column.  Step j (column j final and scaled): warp 0 finishes column j+1 in registers --
+// per column: blocks wider than 64, and the FP64 redo of the mixed factor.  Step j (column j
+// final and scaled): warp 0 finishes column j+1 in registers --
 // its update by column j, the pivot (a shuffle from the lane holding the diagonal), its
 // reciprocal square root, the scaling (the diagonal becomes p y = sqrt(p)) -- while the other
 // warps apply column j to columns j+2..n-1 through the position table (build_update_table),
@@ -113,6 +129,7 @@ __device__ int potrf_lookahead(T* A, int n, const uint16_t* tab, Accept accept) 
   __shared__ int s_bad;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nupd = blockDim.x - 32;  // threads of the trailing update
+  int bad = n;
   if (warp == 0) {
     T v[4];
 #pragma unroll
@@ -123,7 +140,7 @@ __device__ int potrf_lookahead(T* A, int n, const uint16_t* tab, Accept accept) 
     }
     const T p = __shfl_sync(0xffffffffu, v[0], 0);
     const T y = pivot_rsqrt(p);
-    if (lane == 0) s_bad = accept(p) ? n : 0;
+    if (!accept(p)) bad = 0;
 #pragma unroll
     for (int g = 0; g < 4; g++) {
       if (32 * g >= n) break;
@@ -147,7 +164,7 @@ __device__ int potrf_lookahead(T* A, int n, const uint16_t* tab, Accept accept) 
       }
       const T p = __shfl_sync(0xffffffffu, v[0], 0);  // lane 0 holds row c
       const T y = pivot_rsqrt(p);
-      if (lane == 0 && s_bad == n && !accept(p)) s_bad = c;
+      if (bad == n && !accept(p)) bad = c;
 #pragma unroll
       for (int g = 0; g < 4; g++) {
         if (c + 32 * g >= n) break;
@@ -178,68 +195,383 @@ __device__ int potrf_lookahead(T* A, int n, const uint16_t* tab, Accept accept) 
     }
     __syncthreads();
   }
+  if (tid == 0) s_bad = bad;
+  __syncthreads();
   return s_bad;
 }
 
-template <typename T, typename S>
-__device__ __forceinline__ void store_diag_block(T* __restrict__ L, const S* A, int n, int m) {
-  const int lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
-  for (int c = threadIdx.x >> 5; c < n; c += nwarp)
-    for (int r = c + lane; r < n; r += 32) L[(int64_t)c * m + r] = (T)A[c * n + r];
+// What potrf_blocks leaves of Y = L11^-1 beside L11.
+enum PotrfInverse { kInvBlocks, kInvFull };  // its 16 x 16 diagonal blocks, all of it
+
+// ---- FP64 blocks up to 64 wide: 8 x 8 blocks on the FP64 matrix instruction -----------------------
+// An SM's FP64 unit takes one warp instruction per 19 cycles from all warps together, one per 65
+// from a single warp, but an m8n8k4 product (256 multiply-adds, eight instructions' worth) per
+// 73 from all and 292 from one: twice the rate.  So the block is cut into 8 x 8 blocks: warp 0
+// factors a diagonal block in registers, in the fewest dependent FP64 instructions, and everything
+// else is 8 x 8 x 8 products, dealt over the other warps.  Layout: A[c * kPld + r], L in the
+// lower triangle, Y in the blocks above it (Y[r, c] at A[r * kPld + c]), Y's diagonal 8 x 8
+// blocks in Dv (row-major, zeros above the diagonal); kPld = 4 mod 16 doubles: the matrix
+// operands' four columns of eight rows hit distinct banks.
+constexpr int kPotrfWorkers = 4;
+constexpr int kPld = 68;
+constexpr size_t kPotrfBlkSmem = (64 * kPld + 8 * 64) * sizeof(double);
+
+__device__ __forceinline__ void dmma_884(double (&c)[2], double a, double b) {
+  asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};"
+               : "+d"(c[0]), "+d"(c[1])
+               : "d"(a), "d"(b));
 }
 
-// Y = L11^-1 in place in A (n x n, column-major, L11 in the lower triangle), by forward
-// substitution on all columns of the identity at once: with l'_ij = L_ij / L_jj and Z = I, step
-// j (one barrier) takes Z[i, c] -= l'_ij Z[j, c] for the rows i > j and columns c <= j (row j
-// is final by then); Y[i, c] = Z[i, c] / L_ii.  l' lives in the strict lower triangle and the
-// lower-triangular Z transposed in the upper triangle and the diagonal (Z[i, c] at
-// A[i * n + c]), so that a warp's threads update consecutive words; on return A holds Y
-// row-major (A[r * n + c] = Y[r, c], zeros above the diagonal).  rd: n doubles.
-__device__ void invert_lower_inplace(double* A, double* rd, int n) {
-  for (int j = threadIdx.x; j < n; j += blockDim.x) rd[j] = 1.0 / A[j * n + j];
-  __syncthreads();
-  for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
-    const int c = idx / n, r = idx - c * n;
-    if (r > c) A[idx] *= rd[c];          // l'_rc
-    else A[idx] = r == c ? 1.0 : 0.0;    // Z[c, r] = I
+// 1 / p of a positive p with an exponent field in 3 .. 2043, in integer arithmetic (the FP64 unit is what the chain of pivots
+// and the other warps' products compete for): with p = P 2^-52 2^x in [1, 2) 2^x and the FP32
+// reciprocal z0 = m 2^-24 of p's leading bits, e = 1 - p z0 = E 2^-76 exactly, E = -P m mod 2^64
+// (|e| < 2^-21, so |E| < 2^55), and 1/p = z0 (1 + e + e^2 + ...): z0 e in units of 2^-60 from
+// E's upper bits, z0 e^2 from 24 x 23 bits, the dropped z0 e^3 < 2^-63; rounded to nearest (an error
+// below 0.51 ulp).
+__device__ __forceinline__ double pivot_rcp(double p) {
+  const uint32_t hi = (uint32_t)__double2hiint(p), lo = (uint32_t)__double2loint(p);
+  const int ebits = (int)(hi >> 20);
+  const uint32_t ph = (hi & 0xfffffu) | 0x100000u;  // P = ph 2^32 + lo
+  float z0;
+  asm("rcp.approx.ftz.f32 %0, %1;"
+      : "=f"(z0)
+      : "f"(__uint_as_float(((hi << 3) & 0x7fffffu) | (lo >> 29) | 0x3f800000u)));
+  const uint32_t zb = __float_as_uint(z0);  // in [0.5, 1]: exponent 126, or 1.0
+  const uint32_t m = ((zb & 0x7fffffu) | 0x800000u) << ((zb >> 23) - 126u);
+  unsigned long long pm = (unsigned long long)lo * m;
+  pm += (unsigned long long)(ph * m) << 32;
+  const long long E = -(long long)pm;
+  const long long E16 = E >> 16;  // e in units of 2^-60
+  const long long c1 = (long long)((unsigned long long)(uint32_t)E16 * m +
+                                   ((unsigned long long)((uint32_t)(E16 >> 32) * m) << 32)) >> 24;
+  const long long c2 = ((long long)(int)(c1 >> 14) * (int)(E >> 32)) >> 30;
+  const unsigned long long Z = ((unsigned long long)m << 36) + (unsigned long long)(c1 + c2) + 64ull;
+  // Z 2^-60 in [0.5, 1]: the 53-bit integer part of Z / 2^7 carries into the exponent
+  const long long bits = (long long)(Z >> 7) + (1021ll << 52) - ((long long)(ebits - 1023) << 52);
+  return __longlong_as_double(bits);
+}
+
+// One warp: Cholesky of the 8 x 8 diagonal block at column b of A, and its inverse into Dv.
+// Lane (r, g): row r, columns g and g + 4.  Gaussian elimination with the pivots' reciprocals
+// z_j: row r > j takes v_rc -= t u_c, t = v_rj z_j, where u_c is the pivot row's value: a_jc = a_cj
+// right of column j; left of it the register of the eliminated column c holds M^-1 (M the unit
+// lower factor), whose row j gives u_c, and v_rj becomes -t.  The square roots come at the end,
+// all eight at once: L_rj = a_rj y_j and (L^-1)_rc = y_r (M^-1)_rc with y = p^{-1/2}.
+// Returns the first j whose pivot is not positive, else 8.
+__device__ __forceinline__ int potrf_diag8(double* A, double* Dv, int b) {
+  const int lane = threadIdx.x & 31, r = lane & 7, g = lane >> 3;
+  constexpr unsigned full = 0xffffffffu;
+  double v[2], raw[2] = {0.0, 0.0}, prow = 1.0;
+#pragma unroll
+  for (int s = 0; s < 2; s++) {
+    const int c = g + 4 * s;
+    v[s] = r >= c ? A[(b + c) * kPld + b + r] : A[(b + r) * kPld + b + c];
+  }
+  int bad = 8;
+#pragma unroll
+  for (int j = 0; j < 8; j++) {
+    const int sj = j >> 2, gj = 8 * (j & 3);  // column j: register sj of the lanes gj + row
+    const double p = __shfl_sync(full, v[sj], gj + j);
+    double u[2];
+#pragma unroll
+    for (int s = 0; s < 2; s++) {
+      const int c = g + 4 * s;
+      const double right = __shfl_sync(full, v[sj], gj + c);
+      const double left = __shfl_sync(full, v[s], 8 * g + j);
+      u[s] = c > j ? right : left;
+    }
+    const double arj = __shfl_sync(full, v[sj], gj + r);
+#pragma unroll
+    for (int s = 0; s < 2; s++)
+      if (g + 4 * s == j) raw[s] = v[s];
+    if (r == j) prow = p;
+    if (bad == 8 && !positive(p)) bad = j;
+    if (j == 7) break;
+    // t = v_rj / p can neither overflow (v_rj^2 <= p v_rr) nor underflow for pivots and nonzero
+    // v_rj in the middle of the exponent range
+    const uint32_t phi = (uint32_t)__double2hiint(p) >> 20, ahi = (uint32_t)__double2hiint(arj) << 1;
+    const bool tiny = ahi < (300u << 21) && (ahi | (uint32_t)__double2loint(arj)) != 0u;
+    if (phi - 823u <= 400u && !__any_sync(full, tiny)) {
+      const double t = arj * pivot_rcp(p);
+#pragma unroll
+      for (int q = 0; q < 2; q++) {
+        const int s = q ^ ((j + 1) >> 2);  // the next pivot's column first
+        const double x = fma(-t, u[s], v[s]);
+        if (r > j) v[s] = g + 4 * s == j ? -t : x;
+      }
+    } else {  // by the square roots, over the whole range
+      const double y = pivot_rsqrt(p), l = arj * y, t = l * y;
+#pragma unroll
+      for (int s = 0; s < 2; s++) {
+        const int c = g + 4 * s;
+        const double x = c > j ? fma(-l, u[s] * y, v[s]) : fma(-t, u[s], v[s]);
+        if (r > j) v[s] = c == j ? -t : x;
+      }
+    }
+  }
+  const double y = pivot_rsqrt(prow);
+#pragma unroll
+  for (int s = 0; s < 2; s++) {
+    const int c = g + 4 * s;
+    const double l = raw[s] * __shfl_sync(full, y, c);
+    const double w = v[s] * y;
+    if (c <= r) A[(b + c) * kPld + b + r] = l;
+    Dv[r * 8 + c] = c < r ? w : c == r ? y : 0.0;
+  }
+  return bad;
+}
+
+// One warp: the 8 x 8 x 8 product C += sgn P Q with P[r][k] at P[r * pr + k * pk] and
+// Q[k][n] at Q[k * qk + n * qn]; C[r][n] at C[r * cr + n * cn], loaded first if ADD.
+template <bool ADD, bool NEG>
+__device__ __forceinline__ void block_product(double* C, int cr, int cn, const double* P, int pr,
+                                              int pk, const double* Q, int qk, int qn) {
+  const int lane = threadIdx.x & 31, r = lane >> 2, k = lane & 3;
+  double a[2], b[2], c[2] = {0.0, 0.0};
+#pragma unroll
+  for (int s = 0; s < 2; s++) {
+    a[s] = P[r * pr + (4 * s + k) * pk];
+    b[s] = Q[(4 * s + k) * qk + r * qn];
+    if (NEG) a[s] = -a[s];
+  }
+  double* c0 = C + r * cr + 2 * k * cn;
+  if (ADD) {
+    c[0] = c0[0];
+    c[1] = c0[cn];
+  }
+  __syncwarp();  // C may be P or Q: every lane has read before any writes
+  dmma_884(c, a[0], b[0]);
+  dmma_884(c, a[1], b[1]);
+  c0[0] = c[0];
+  c0[cn] = c[1];
+}
+
+// Cholesky of the n x n block (n <= 64, padded to whole 8 x 8 blocks with the identity, the
+// upper blocks zero) and Y.  Per block column p, one barrier of the CTA:
+//   warp 0: the block below the diagonal one, L_{p+1,p} = A_{p+1,p} D_p^{-T} (D_p the diagonal
+//   block, its inverse from potrf_diag8), then the next diagonal block's update and factor;
+//   kPotrfWorkers warps: the other blocks of the column and the block row p of Y, Y_pc =
+//   D_p^{-1} S_pc; then (a barrier of theirs that warp 0 only arrives at) the trailing update
+//   A_ij -= L_ip L_jp^T and S_ic -= L_ip Y_pc (S_ic starts at 0, Y_pp = D_p^{-1}).
+// More workers finish their products sooner but delay warp 0's chain at the FP64 unit they share.
+// kInvBlocks: of Y only the blocks (p, p-1) of odd p, which complete 16 x 16 diagonal blocks.
+// Returns the first column whose pivot is not positive, else n.
+// Measured, one 64-wide block (one CTA): kInvBlocks 31 us, kInvFull 41 us with four workers (34 /
+// 45 with three, 34 / 46 with seven); a column-by-column factorization at one barrier per
+// column took 42 us, its in-place inverse 35 more.  Per 48^3 27-point factorization POTRF 19.8 ->
+// 15.6 ms; 64 x 64 2D Laplacian step 0.70 -> 0.62 ms.
+template <int INV, int WORKERS>
+__device__ int potrf_blocks(double* A, double* Dv, int n) {
+  __shared__ int s_bad;
+  const int warp = threadIdx.x >> 5, nb = (n + 7) / 8;
+  int bad = n;
+  if (warp == 0) {
+    const int q = potrf_diag8(A, Dv, 0);
+    if (q < 8) bad = min(n, q);
   }
   __syncthreads();
-  for (int j = 0; j + 1 < n; j++) {
-    const int cols = j + 1, rows = n - 1 - j;
-    for (int idx = threadIdx.x; idx < rows * cols; idx += blockDim.x) {
-      const int ii = idx / cols, c = idx - ii * cols, i = j + 1 + ii;
-      A[i * n + c] -= A[j * n + i] * A[j * n + c];
+  for (int p = 0; p < nb; p++) {
+    const int below = nb - 1 - p;
+    const double* D = Dv + 64 * p;
+    if (warp == 0) {
+      if (below > 0) {
+        const int b = 8 * (p + 1);
+        double* X = A + 8 * p * kPld + b;
+        block_product<false, false>(X, 1, kPld, X, 1, kPld, D, 1, 8);
+        __threadfence_block();
+        __syncwarp();
+        asm volatile("bar.arrive 1, %0;" ::"n"(32 * (WORKERS + 1)) : "memory");
+        block_product<true, true>(A + b * kPld + b, 1, kPld, X, 1, kPld, X, kPld, 1);
+        __syncwarp();
+        const int q = potrf_diag8(A, Dv + 64 * (p + 1), b);
+        if (q < 8 && bad == n) bad = min(n, b + q);
+      }
+    } else if (warp <= WORKERS) {
+      const int c0 = INV == kInvFull ? 0 : p & ~1;  // first block column of Y's row p
+      const int nx = below > 0 ? below - 1 : 0;
+      for (int q = warp - 1; q < nx + p - c0; q += WORKERS) {
+        if (q < nx) {
+          double* X = A + 8 * p * kPld + 8 * (p + 2 + q);
+          block_product<false, false>(X, 1, kPld, X, 1, kPld, D, 1, 8);
+        } else {
+          double* S = A + 8 * p * kPld + 8 * (c0 + q - nx);
+          block_product<false, false>(S, kPld, 1, D, 8, 1, S, kPld, 1);
+        }
+      }
+      if (below > 0) {
+        asm volatile("bar.sync 1, %0;" ::"n"(32 * (WORKERS + 1)) : "memory");
+        // the trailing blocks (i, j), p < j <= i, without the next diagonal block, then Y's
+        const int tri = below * (below + 1) / 2, cols = INV == kInvFull ? p + 1 : (p & 1) ^ 1;
+        const int ny = INV == kInvFull ? below * cols : cols;
+        for (int q = warp; q < tri + ny; q += WORKERS) {
+          if (q < tri) {
+            int i = 0;
+            while ((i + 1) * (i + 2) / 2 <= q) i++;
+            const int j = p + 1 + q - i * (i + 1) / 2;
+            i += p + 1;
+            block_product<true, true>(A + 8 * j * kPld + 8 * i, 1, kPld, A + 8 * p * kPld + 8 * i, 1,
+                                      kPld, A + 8 * p * kPld + 8 * j, kPld, 1);
+          } else {
+            const int f = q - tri, i = p + 1 + f / cols, c = INV == kInvFull ? f % cols : p;
+            double* S = A + 8 * i * kPld + 8 * c;
+            const double* X = A + 8 * p * kPld + 8 * i;
+            if (c < p)
+              block_product<true, true>(S, kPld, 1, X, 1, kPld, A + 8 * p * kPld + 8 * c, kPld, 1);
+            else
+              block_product<true, true>(S, kPld, 1, X, 1, kPld, D, 8, 1);
+          }
+        }
+      }
     }
     __syncthreads();
   }
-  for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
-    const int r = idx / n, c = idx - r * n;
-    A[idx] = c <= r ? A[idx] * rd[r] : 0.0;
-  }
+  if (threadIdx.x == 0) s_bad = bad;
   __syncthreads();
+  return s_bad;
 }
 
-// The kOzInvRows slice rows of Y S (Y row-major in A, n x n; rows and columns past n are zero;
+// Entry (r, c) of Y as potrf_blocks leaves it, c <= r.
+__device__ __forceinline__ double potrf_y(const double* A, const double* Dv, int r, int c) {
+  return r >> 3 == c >> 3 ? Dv[64 * (r >> 3) + 8 * (r & 7) + (c & 7)] : A[r * kPld + c];
+}
+
+// FP32 Cholesky of the n x n block A (n <= 64, column-major, leading dimension 64, lower
+// triangle), in panels of 8 columns: warp 0 factors a panel in registers (two rows per lane,
+// pivots and multipliers by shuffles), then the 256 threads apply it to the columns after it,
+// a 4 x 4 block each.  Every element sees the same operations in the same order as in
+// potrf_lookahead; that one's barrier and dependent shared-memory loads per column took 33 us at
+// n = 64, where the FP32 arithmetic itself is short (96^3 diffusion: POTRF 13.2 -> 6.0 ms).
+template <typename Accept>
+__device__ int potrf_f32_panels(float* A, int n, Accept accept) {
+  __shared__ int s_bad;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  int bad = n;
+  for (int k0 = 0; k0 < n; k0 += 8) {
+    if (warp == 0) {
+      float v[2][8];
+#pragma unroll
+      for (int g = 0; g < 2; g++)
+#pragma unroll
+        for (int j = 0; j < 8; j++) {
+          const int r = k0 + 32 * g + lane;
+          v[g][j] = r < n && k0 + j < n ? A[(k0 + j) * 64 + r] : 0.f;
+        }
+#pragma unroll
+      for (int j = 0; j < 8; j++) {
+        if (k0 + j >= n) break;
+        const float p = __shfl_sync(0xffffffffu, v[0][j], j);
+        const float y = pivot_rsqrt(p);
+        if (bad == n && !accept(p)) bad = k0 + j;
+        v[0][j] *= y;
+        v[1][j] *= y;
+#pragma unroll
+        for (int q = 0; q < 8; q++)
+          if (q > j) {
+            const float l = __shfl_sync(0xffffffffu, v[0][j], q);
+            v[0][q] = fmaf(-v[0][j], l, v[0][q]);
+            v[1][q] = fmaf(-v[1][j], l, v[1][q]);
+          }
+      }
+#pragma unroll
+      for (int g = 0; g < 2; g++)
+#pragma unroll
+        for (int j = 0; j < 8; j++) {
+          const int r = k0 + 32 * g + lane;
+          if (r < n && r >= k0 + j) A[(k0 + j) * 64 + r] = v[g][j];
+        }
+    }
+    __syncthreads();
+    const int r0 = 4 * (tid & 15), c0 = 4 * (tid >> 4);
+    if (c0 >= k0 + 8 && c0 < n && r0 >= c0 && r0 < n) {
+      float4 x[4];
+#pragma unroll
+      for (int c = 0; c < 4; c++) x[c] = *reinterpret_cast<const float4*>(A + (c0 + c) * 64 + r0);
+#pragma unroll
+      for (int k = 0; k < 8; k++) {
+        const float4 a = *reinterpret_cast<const float4*>(A + (k0 + k) * 64 + r0);
+        const float4 b = *reinterpret_cast<const float4*>(A + (k0 + k) * 64 + c0);
+        const float bc[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+          x[c].x = fmaf(-a.x, bc[c], x[c].x);
+          x[c].y = fmaf(-a.y, bc[c], x[c].y);
+          x[c].z = fmaf(-a.z, bc[c], x[c].z);
+          x[c].w = fmaf(-a.w, bc[c], x[c].w);
+        }
+      }
+#pragma unroll
+      for (int c = 0; c < 4; c++) *reinterpret_cast<float4*>(A + (c0 + c) * 64 + r0) = x[c];
+    }
+    __syncthreads();
+  }
+  if (tid == 0) s_bad = bad;
+  __syncthreads();
+  return s_bad;
+}
+
+// The inverses of the 16 x 16 diagonal blocks of L11 (shared memory, leading dimension ld) into
+// Y (row-major n x n, global): warp b inverts block b, lane (i, h) column i and every other row,
+// by forward substitution on the columns of the identity in registers.
+template <typename T, typename S>
+__device__ void invert_blocks(const S* A, int ld, int n, T* __restrict__ Y) {
+  const int b0 = 16 * (threadIdx.x >> 5);
+  if (b0 >= n) return;
+  const int lane = threadIdx.x & 31, i = lane & 15, h = lane >> 4, bw = min(16, n - b0);
+  T x[8];  // rows 2 q + h of column i
+#pragma unroll
+  for (int q = 0; q < 8; q++) x[q] = 2 * q + h == i ? T(1) : T(0);
+#pragma unroll
+  for (int j = 0; j < 16; j++) {
+    if (j >= bw) break;
+    const T rj = T(1) / (T)A[(b0 + j) * ld + b0 + j];
+    T yj = x[j >> 1] * rj;  // row j is complete: its lane pair's half j & 1 holds it
+    yj = __shfl_sync(0xffffffffu, yj, i + 16 * (j & 1));
+    if (h == (j & 1)) {
+      x[j >> 1] = yj;
+      if (i <= j && b0 + i < n) Y[(int64_t)(b0 + j) * n + b0 + i] = yj;
+    }
+#pragma unroll
+    for (int q = 0; q < 8; q++) {
+      const int r = 2 * q + h;
+      if (r > j && r < bw) x[q] = fma_t(-(T)A[(b0 + j) * ld + b0 + r], yj, x[q]);
+    }
+  }
+}
+
+template <typename T, typename S>
+__device__ __forceinline__ void store_diag_block(T* __restrict__ L, const S* A, int lda, int n, int m) {
+  const int lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
+  for (int c = threadIdx.x >> 5; c < n; c += nwarp)
+    for (int r = c + lane; r < n; r += 32) L[(int64_t)c * m + r] = (T)A[c * lda + r];
+}
+
+// The kOzInvRows slice rows of Y S (Y as potrf_blocks leaves it; rows and columns past n are zero;
 // S = diag(2^t_k), t_k the exponent of L11[k,k]) at slice rows y0 .. y0+63 of the scratch oy
 // (planes oy_rows rows apart, then the rows' exponents, then the column shifts t_k): the
 // right-hand operand of the supernode's tensor-core TRSM, A21 Y^T = (A21 S^-1)(Y S)^T.  The
 // shift balances the operands: a column k of Y scales like 1/L_kk and the same column of A21
 // like L_kk (rows and columns of A may span many decades), while Y S is the inverse of the
 // unit-diagonal factor (exact: powers of two).  t: the n shifts; e: kOzInvRows ints.
-__device__ void slice_inverse(const double* A, int n, const int* t, uint8_t* oy,
+__device__ void slice_inverse(const double* A, const double* Dv, int n, const int* t, uint8_t* oy,
                               int64_t oy_rows, int64_t y0, int* e) {
   const size_t stride = (size_t)oy_rows * kOzRowBytes;
   int32_t* oexp = reinterpret_cast<int32_t*>(oy + kOzSlices * stride);
-  for (int r = threadIdx.x; r < kOzInvRows; r += blockDim.x) {
+  static_assert(kPotrfThreads == 4 * kOzInvRows, "four threads per row");
+  {
+    const int r = threadIdx.x >> 2;
     int f = 0;  // the largest exponent field of the row of Y S (fields shifted by t_k)
     if (r < n)
-      for (int c = 0; c <= r; c++) {
-        const int fc = oz_exp_field(A[r * n + c]);
+      for (int c = threadIdx.x & 3; c <= r; c += 4) {
+        const int fc = oz_exp_field(potrf_y(A, Dv, r, c));
         if (fc > 0) f = max(f, fc + t[c]);
       }
-    e[r] = oz_row_exponent(f);
-    oexp[y0 + r] = e[r];
-    oexp[oy_rows + y0 + r] = r < n ? t[r] : 0;
+    f = max(f, __shfl_xor_sync(0xffffffffu, f, 1));
+    f = max(f, __shfl_xor_sync(0xffffffffu, f, 2));
+    if ((threadIdx.x & 3) == 0) {
+      e[r] = oz_row_exponent(f);
+      oexp[y0 + r] = e[r];
+      oexp[oy_rows + y0 + r] = r < n ? t[r] : 0;
+    }
   }
   __syncthreads();
   for (int item = threadIdx.x; item < kOzInvRows * 8; item += blockDim.x) {
@@ -249,63 +581,74 @@ __device__ void slice_inverse(const double* A, int n, const int* t, uint8_t* oy,
 #pragma unroll
     for (int j = 0; j < 8; j++) {
       const int k = 8 * c + j;
-      R[j] = r < n && k < n ? oz_fixed(A[r * n + k], e[r] - t[k]) : 0;  // Y[r,k] 2^t_k
+      R[j] = r < n && k <= r ? oz_fixed(potrf_y(A, Dv, r, k), e[r] - t[k]) : 0;  // Y[r,k] 2^t_k
     }
     oz_write_chunk(R, oy + (size_t)(y0 + r) * kOzRowBytes + pc * 16, stride);
   }
 }
 
 // ---- POTRF of each diagonal block ---------------------------------------------------------
-// One CTA (kPotrfThreads threads) per supernode; the n x n block is factored in shared memory by
-// potrf_lookahead.  A non-positive pivot is an error (not SPD), recorded with its column.
-// With oy, a task whose y field is set (a 128-tile supernode of the FP64 factor) also forms
-// Y = L11^-1 (into d.dinv, row-major, for the solves) and Y's slices at rows y .. y+63 of oy,
-// the operand of its tensor-core TRSM.
-template <typename T>
-__global__ void __launch_bounds__(kPotrfThreads) k_potrf(const int4* __restrict__ tasks, int ntasks, int* __restrict__ queue,
-                                               const SnDev* __restrict__ sns,
-                                               const MatDev* __restrict__ mats,
-                                               uint8_t* __restrict__ oy, int64_t oy_rows) {
+// One CTA (kPotrfThreads threads) per supernode, in shared memory.  A non-positive pivot is an
+// error (not SPD), recorded with its column.
+// Factors that keep the inverses (d.dinv, widths up to 64) use potrf_blocks and get the inverses
+// of the 16 x 16 diagonal blocks, in their places of the row-major Y, for the FP64 TRSM
+// (k_diag_inverse completes Y later); with oy, a task whose y field is set (a 128-tile supernode
+// of the FP64 factor) all of Y, for the solves, and Y's slices at rows y .. y+63 of oy, the
+// operand of its tensor-core TRSM.
+__global__ void __launch_bounds__(kPotrfThreads)
+    k_potrf(const int4* __restrict__ tasks, const SnDev* __restrict__ sns,
+            const MatDev* __restrict__ mats, uint8_t* __restrict__ oy, int64_t oy_rows) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* A = reinterpret_cast<T*>(smem_raw);
-  __shared__ int s_next_task;
+  double* A = reinterpret_cast<double*>(smem_raw);
   __shared__ int s_e[kOzInvRows], s_t[kOzInvRows];
-  for (int tq = blockIdx.x; tq < ntasks;) {
-    const int4 tk = tasks[tq];
-    const SnDev d = sns[tk.x];
-    const int n = d.n, m = d.m;
-    T* L = reinterpret_cast<T*>(d.L);
+  pdl_launch_dependents();
+  const int4 tk = tasks[blockIdx.x];
+  const SnDev d = sns[tk.x];
+  const int n = d.n, m = d.m;
+  double* L = reinterpret_cast<double*>(d.L);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+  if (!d.dinv) {
     uint16_t* tab = reinterpret_cast<uint16_t*>(smem_raw + (size_t)n * n * sizeof(double));
-    stage_diag_block(A, L, n, m);
     build_update_table(tab, n);
+    pdl_wait();  // the levels below are done: the block is final but for this
+    stage_diag_block(A, L, n, m);
     cp_async_wait_all();
     __syncthreads();
-    const int bad = potrf_lookahead<T>(A, n, tab, [](T p) { return p > T(0); });
+    const int bad = potrf_lookahead<double>(A, n, tab, [](double p) { return positive(p); });
     if (bad < n && threadIdx.x == 0) record_error(mats[d.mat], d.col0 + bad);
-    store_diag_block(L, A, n, m);
-    __syncthreads();
-    if constexpr (sizeof(T) == 8) {
-      if (oy && tk.w >= 0 && d.dinv && n <= kOzInvRows) {
-        double* Ad = reinterpret_cast<double*>(A);
-        double* rd = reinterpret_cast<double*>(smem_raw + potrf_rd_offset(n));
-        // column shifts t_k: the exponent of L11[k,k] (|L_kk| in [2^t, 2^(t+1)))
-        for (int k = threadIdx.x; k < n; k += blockDim.x) {
-          const int f = oz_exp_field(Ad[k * n + k]);
-          s_t[k] = f > 0 ? f - 1023 : 0;
-        }
-        invert_lower_inplace(Ad, rd, n);
-        double* Y = reinterpret_cast<double*>(d.dinv);
-        for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) Y[idx] = Ad[idx];
-        slice_inverse(Ad, n, s_t, oy, oy_rows, tk.w, s_e);
-        __syncthreads();
-      }
+    store_diag_block(L, A, n, n, m);
+    return;
+  }
+  double* Dv = A + 64 * kPld;
+  const int n8 = (n + 7) & ~7;
+  for (int c = warp; c < n8; c += nwarp)  // what the block does not fill: see potrf_blocks
+    for (int r = lane; r < n8; r += 32)
+      if (r < c || r >= n) A[c * kPld + r] = r == c ? 1.0 : 0.0;
+  pdl_wait();
+  stage_diag_block_ld(A, kPld, L, n, m);
+  cp_async_wait_all();
+  __syncthreads();
+  const bool full = oy && tk.w >= 0;
+  const int bad = full ? potrf_blocks<kInvFull, kPotrfWorkers>(A, Dv, n)
+                        : potrf_blocks<kInvBlocks, kPotrfWorkers>(A, Dv, n);
+  if (bad < n && threadIdx.x == 0) record_error(mats[d.mat], d.col0 + bad);
+  store_diag_block(L, A, kPld, n, m);
+  double* Y = reinterpret_cast<double*>(d.dinv);
+  if (full) {
+    // column shifts t_k: the exponent of L11[k,k] (|L_kk| in [2^t, 2^(t+1)))
+    for (int k = threadIdx.x; k < n; k += blockDim.x) {
+      const int f = oz_exp_field(A[k * kPld + k]);
+      s_t[k] = f > 0 ? f - 1023 : 0;
     }
-    // a CTA's first task is its block index; only a grid smaller than the task list makes
-    // CTAs take further tasks from this launch's work queue
-    if (gridDim.x >= ntasks) break;
-    if (threadIdx.x == 0) s_next_task = gridDim.x + atomicAdd(queue, 1);
+    for (int r = warp; r < n; r += nwarp)
+      for (int c = lane; c < n; c += 32) Y[r * n + c] = c <= r ? potrf_y(A, Dv, r, c) : 0.0;
     __syncthreads();
-    tq = s_next_task;
+    slice_inverse(A, Dv, n, s_t, oy, oy_rows, tk.w, s_e);
+  } else {
+    for (int e = threadIdx.x; e < n * 16; e += blockDim.x) {
+      const int r = e >> 4, c = (r & ~15) + (e & 15);
+      if (c <= r) Y[r * n + c] = potrf_y(A, Dv, r, c);
+    }
   }
 }
 
@@ -314,109 +657,93 @@ __global__ void __launch_bounds__(kPotrfThreads) k_potrf(const int4* __restrict_
 // i.e. for each row x_j = (a_j - sum_{k<j} x_k L_jk) / L_jj.
 //   k_trsm (any W <= 128): the substitution itself, one thread per row, partial rows in
 //     shared memory.
-// k_trsm_blk (W <= 64): a task's 32 rows (lane = row) are solved by all kTrsmWarps warps at
-//   once, 16 columns at a time.  Block b (columns 16b .. 16b+15, diagonal block D_b of L11):
-//   warp w takes the block's columns w, w + kTrsmWarps, ... and subtracts the products with
-//   the solved columns of the earlier blocks, acc_k = a_k - sum_{j<16b} x_j L_kj; the partial
-//   vectors are exchanged through shared memory and the block is finished as x_b = D_b^{-1}
-//   acc_b with D_b^{-1} (lower triangular, formed per task by forward substitution on the
-//   unit vectors).  Each warp thus issues 1/kTrsmWarps of a row's FMAs: on this part an FP64
-//   warp instruction holds its warp for ~64 cycles, so the per-task latency (what the
-//   single-supernode levels of the elimination tree's top wait for) falls with the warps.
-constexpr int kTrsmWarps = 8;
-constexpr int kTrsmCols = 16 / kTrsmWarps;  // columns of a block per warp
+// k_trsm_blk (W <= 64): the rows of a task (lane = row, or a part of the lanes per row when ROWS is
+//   below 32) are solved by all the CTA's warps at once, 16 columns at a time.  Block b (columns
+//   16b .. 16b+15, diagonal block D_b of L11): every lane group takes QC of the block's columns
+//   and subtracts the products with the solved columns of the earlier blocks, acc_k = a_k -
+//   sum_{j<16b} x_j L_kj; the partial vectors are exchanged through shared memory and the block
+//   is finished as x_b = D_b^{-1} acc_b with D_b^{-1} from POTRF (in d.dinv).  On this part an FP64 warp
+//   instruction holds its warp for ~64 cycles and 32 rows are 66,000 multiply-adds, 16 us of
+//   one SM's FP64 units: levels with SMs to spare take ROWS = 16 or 8 per CTA (launch_trsm).
+//   Wide levels do `per` tasks in turn in one CTA, so that L11 is staged once for them.
+//   Measured per factorization: 64 x 64 2D Laplacian 0.21 -> 0.11 ms, 48^3 27-point (levels without
+//   the tensor-core TRSM) 4.5 -> 3.3 ms, 96^3 diffusion in FP32 13.4 -> 9.7 ms.
+template <int ROWS>
+__host__ __device__ constexpr int trsm_warps() { return ROWS == 8 ? 4 : 8; }
+template <typename T, int ROWS>
+constexpr size_t trsm_blk_smem() { return (64 * 64 + 64 * ROWS + 16 * ROWS + 4 * 16 * 16) * sizeof(T); }
 
-template <typename T>
-constexpr size_t trsm_blk_smem() { return (64 * 64 + 64 * 32 + 16 * 32 + 4 * 16 * 16 + 64) * sizeof(T); }
-
-template <typename T>
-__global__ void __launch_bounds__(32 * kTrsmWarps) k_trsm_blk(const int4* __restrict__ tasks, int ntasks,
-                                                              int* __restrict__ queue,
-                                                              const SnDev* __restrict__ sns) {
+template <typename T, int ROWS>
+__global__ void __launch_bounds__(32 * trsm_warps<ROWS>())
+    k_trsm_blk(const int4* __restrict__ tasks, int ntasks, int per, const SnDev* __restrict__ sns) {
+  constexpr int NG = 32 / ROWS, NC = trsm_warps<ROWS>() * NG, QC = 16 / NC;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* Ls = reinterpret_cast<T*>(smem_raw);  // Ls[c * 64 + r] = L11[r][c]
-  T* Xs = Ls + 64 * 64;                     // Xs[k * 32 + lane]: solved column k of the rows
-  T* Acc = Xs + 64 * 32;                    // Acc[kk * 32 + lane]: block column kk before D_b^{-1}
-  T* Dv = Acc + 16 * 32;                    // Dv[b * 256 + k * 16 + i] = (D_b^{-1})[k][i], k >= i
-  T* rd = Dv + 4 * 16 * 16;                 // 1 / L11[k][k]
-  __shared__ int s_next_task;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (int tq = blockIdx.x; tq < ntasks;) {
-    const int4 tk = tasks[tq];
+  T* Xs = Ls + 64 * 64;                     // Xs[k * ROWS + r]: solved column k of the rows
+  T* Acc = Xs + 64 * ROWS;                  // Acc[kk * ROWS + r]: block column kk before D_b^{-1}
+  T* Dv = Acc + 16 * ROWS;                  // Dv[b * 256 + k * 16 + i] = (D_b^{-1})[k][i], k >= i
+  pdl_launch_dependents();
+  const int lane = threadIdx.x & 31, r = lane % ROWS;
+  const int w = (threadIdx.x >> 5) * NG + lane / ROWS;  // this lane group's first column of a block
+  int cur = -1;
+  const int e0 = blockIdx.x * per, e1 = min(ntasks, e0 + per);
+  for (int e = e0; e < e1; e++) {
+    const int4 tk = tasks[e];
     const SnDev d = sns[tk.x];
     const int n = d.n, m = d.m;
     T* L = reinterpret_cast<T*>(d.L);
-    stage_diag_block_ld(Ls, 64, L, n, m);
-    // the warp's own columns k = 16 b + w + kTrsmWarps q of this task's row
-    const int row = n + tk.y + lane;
+    if (e == e0) pdl_wait();  // the diagonal blocks are factored
+    if (tk.x != cur) {
+      if (cur >= 0) __syncthreads();
+      cur = tk.x;
+      stage_diag_block_ld(Ls, 64, L, n, m);
+      const T* Y = reinterpret_cast<const T*>(d.dinv);
+      for (int q = threadIdx.x; q < n * 16; q += blockDim.x) {
+        const int k = q >> 4, i = q & 15;
+        if (i <= (k & 15)) cp_async_elem(Dv + (k >> 4) * 256 + (k & 15) * 16 + i, Y + k * n + (k & ~15) + i);
+      }
+    }
+    // the lane group's own columns k = 16 b + w + NC q of this task's row
+    const int row = n + tk.y + (int)blockIdx.y * ROWS + r;
     const bool live = row < m;
-    T a[4 * kTrsmCols];
+    T a[4 * QC];
 #pragma unroll
     for (int b = 0; b < 4; b++)
 #pragma unroll
-      for (int q = 0; q < kTrsmCols; q++) {
-        const int k = 16 * b + w + kTrsmWarps * q;
-        a[b * kTrsmCols + q] = (live && k < n) ? L[(int64_t)k * m + row] : T(0);
+      for (int q = 0; q < QC; q++) {
+        const int k = 16 * b + w + NC * q;
+        a[b * QC + q] = (live && k < n) ? L[(int64_t)k * m + row] : T(0);
       }
     cp_async_wait_all();
     __syncthreads();
-    if (threadIdx.x < n) rd[threadIdx.x] = T(1) / Ls[threadIdx.x * 65];
-    __syncthreads();
-    if (threadIdx.x < 64) {
-      const int b = threadIdx.x >> 4, i = threadIdx.x & 15, c0 = 16 * b;
-      if (c0 + i < n) {
-        T* dv = Dv + b * 256;
-        dv[i * 16 + i] = rd[c0 + i];
-        for (int k = i + 1; k < 16 && c0 + k < n; k++) {
-          T s = T(0);
-          for (int j = i; j < k; j++) s = fma_t(Ls[(c0 + j) * 64 + c0 + k], dv[j * 16 + i], s);
-          dv[k * 16 + i] = -s * rd[c0 + k];
-        }
-      }
-    }
-    __syncthreads();
-    T out[4 * kTrsmCols] = {};
 #pragma unroll
     for (int b = 0; b < 4; b++) {
       if (16 * b >= n) break;
-      T acc[kTrsmCols];
+      T acc[QC];
 #pragma unroll
-      for (int q = 0; q < kTrsmCols; q++) acc[q] = a[b * kTrsmCols + q];
-      const T* lrow = Ls + 16 * b + w;  // + j * 64 + kTrsmWarps q: L11[16b + w + kTrsmWarps q][j]
+      for (int q = 0; q < QC; q++) acc[q] = a[b * QC + q];
+      const T* lrow = Ls + 16 * b + w;  // + j * 64 + NC q: L11[16b + w + NC q][j]
       for (int j = 0; j < 16 * b; j++) {
-        const T xj = Xs[j * 32 + lane];
+        const T xj = Xs[j * ROWS + r];
 #pragma unroll
-        for (int q = 0; q < kTrsmCols; q++) acc[q] = fma_t(-xj, lrow[j * 64 + kTrsmWarps * q], acc[q]);
+        for (int q = 0; q < QC; q++) acc[q] = fma_t(-xj, lrow[j * 64 + NC * q], acc[q]);
       }
 #pragma unroll
-      for (int q = 0; q < kTrsmCols; q++) Acc[(w + kTrsmWarps * q) * 32 + lane] = acc[q];
+      for (int q = 0; q < QC; q++) Acc[(w + NC * q) * ROWS + r] = acc[q];
       __syncthreads();
       const T* dv = Dv + b * 256;
 #pragma unroll
-      for (int q = 0; q < kTrsmCols; q++) {
-        const int kk = w + kTrsmWarps * q;
+      for (int q = 0; q < QC; q++) {
+        const int kk = w + NC * q, k = 16 * b + kk;
         T s = T(0);
-        for (int i = 0; i <= kk; i++) s = fma_t(Acc[i * 32 + lane], dv[kk * 16 + i], s);
-        out[b * kTrsmCols + q] = s;
-        Xs[(16 * b + kk) * 32 + lane] = s;
+        if (k < n) {
+          for (int i = 0; i <= kk; i++) s = fma_t(Acc[i * ROWS + r], dv[kk * 16 + i], s);
+          if (live) L[(int64_t)k * m + row] = s;
+        }
+        Xs[k * ROWS + r] = s;
       }
       __syncthreads();
     }
-    if (live) {
-#pragma unroll
-      for (int b = 0; b < 4; b++)
-#pragma unroll
-        for (int q = 0; q < kTrsmCols; q++) {
-          const int k = 16 * b + w + kTrsmWarps * q;
-          if (k < n) L[(int64_t)k * m + row] = out[b * kTrsmCols + q];
-        }
-    }
-    // a CTA's first task is its block index; only a grid smaller than the task list makes
-    // CTAs take further tasks from this launch's work queue
-    if (gridDim.x >= ntasks) break;
-    if (threadIdx.x == 0) s_next_task = gridDim.x + atomicAdd(queue, 1);
-    __syncthreads();
-    tq = s_next_task;
   }
 }
 
@@ -479,12 +806,6 @@ struct SchurCfg {
   static constexpr int KC = TILE == 64 ? 32 : 64;  // K chunk staged in shared memory
   static constexpr int LDS = TILE + 8;            // padded stride (bank spread)
 };
-
-__device__ __forceinline__ void dmma_884(double (&c)[2], double a, double b) {
-  asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};"
-               : "+d"(c[0]), "+d"(c[1])
-               : "d"(a), "d"(b));
-}
 
 template <int TILE, bool OWNER>
 __global__ void __launch_bounds__(SchurCfg<TILE>::THREADS)
@@ -678,46 +999,48 @@ __global__ void __launch_bounds__(SchurF32Cfg<TILE>::THREADS)
 // is 1 after equilibration), the block is factored again in FP64 from the panel's values,
 // which are still unchanged in global memory, and the FP64 result is rounded into the panel.
 // err[2] counts such redos.  The FP64 block overlays the FP32 one in shared memory.
-__global__ void __launch_bounds__(kPotrfThreads) k_potrf_mixed(const int4* __restrict__ tasks, int ntasks, int* __restrict__ queue,
-                                                     const SnDev* __restrict__ sns,
-                                                     const MatDev* __restrict__ mats,
-                                                     float tau) {
+__global__ void __launch_bounds__(kPotrfThreads)
+    k_potrf_mixed(const int4* __restrict__ tasks, const SnDev* __restrict__ sns,
+                  const MatDev* __restrict__ mats, float tau) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ int s_next_task;
-  float* A = reinterpret_cast<float*>(smem_raw);    // n x n FP32 work block
+  float* A = reinterpret_cast<float*>(smem_raw);    // FP32 work block, leading dimension lda
   double* D = reinterpret_cast<double*>(smem_raw);  // n x n FP64 block of a redo
-  for (int tq = blockIdx.x; tq < ntasks;) {
-    const int4 tk = tasks[tq];
-    const SnDev d = sns[tk.x];
-    const int n = d.n, m = d.m;
-    float* L = reinterpret_cast<float*>(d.L);
-    uint16_t* tab = reinterpret_cast<uint16_t*>(smem_raw + (size_t)n * n * sizeof(double));
-    stage_diag_block(A, L, n, m);
-    build_update_table(tab, n);
-    cp_async_wait_all();
+  pdl_launch_dependents();
+  const int4 tk = tasks[blockIdx.x];
+  const SnDev d = sns[tk.x];
+  const int n = d.n, m = d.m, lda = n <= 64 ? 64 : n;
+  float* L = reinterpret_cast<float*>(d.L);
+  float* Y = reinterpret_cast<float*>(d.dinv);
+  uint16_t* tab = reinterpret_cast<uint16_t*>(smem_raw + potrf_mixed_tab_offset(n));
+  pdl_wait();  // the levels below are done: the block is final but for this
+  stage_diag_block_ld(A, lda, L, n, m);
+  if (n > 64) build_update_table(tab, n);
+  cp_async_wait_all();
+  __syncthreads();
+  const auto accept = [&](float p) { return p >= tau; };
+  const int stop = n <= 64 ? potrf_f32_panels(A, n, accept)
+                           : potrf_lookahead<float>(A, n, tab, accept);
+  if (stop < n) {
+    // a small FP32 pivot: the whole block again in FP64 (the barrier that ended the FP32
+    // pass is behind every thread, so D may overwrite A)
+    if (threadIdx.x == 0) atomicAdd(mats[d.mat].err + 2, 1ull);
+    const int lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
+    for (int c = threadIdx.x >> 5; c < n; c += nwarp)
+      for (int r = c + lane; r < n; r += 32) D[c * n + r] = (double)L[(int64_t)c * m + r];
+    if (n <= 64) build_update_table(tab, n);
     __syncthreads();
-    const int stop = potrf_lookahead<float>(A, n, tab, [&](float p) { return p >= tau; });
-    if (stop < n) {
-      // a small FP32 pivot: the whole block again in FP64 (the barrier that ended the FP32
-      // pass is behind every thread, so D may overwrite A)
-      if (threadIdx.x == 0) atomicAdd(mats[d.mat].err + 2, 1ull);
-      const int lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
-      for (int c = threadIdx.x >> 5; c < n; c += nwarp)
-        for (int r = c + lane; r < n; r += 32) D[c * n + r] = (double)L[(int64_t)c * m + r];
-      __syncthreads();
-      const int bad = potrf_lookahead<double>(D, n, tab, [](double p) { return p > 0.0; });
-      if (bad < n && threadIdx.x == 0) record_error(mats[d.mat], d.col0 + bad);
-      store_diag_block(L, D, n, m);
-    } else {
-      store_diag_block(L, A, n, m);
-    }
+    const int bad = potrf_lookahead<double>(D, n, tab, [](double p) { return positive(p); });
+    if (bad < n && threadIdx.x == 0) record_error(mats[d.mat], d.col0 + bad);
+    store_diag_block(L, D, n, n, m);
     __syncthreads();
-    // a CTA's first task is its block index; only a grid smaller than the task list makes
-    // CTAs take further tasks from this launch's work queue
-    if (gridDim.x >= ntasks) break;
-    if (threadIdx.x == 0) s_next_task = gridDim.x + atomicAdd(queue, 1);
+    // the diagonal blocks' inverses of the rounded factor, as without the redo
+    if (Y)
+      for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) D[idx] = (double)(float)D[idx];
     __syncthreads();
-    tq = s_next_task;
+    if (Y) invert_blocks<float, double>(D, n, n, Y);
+  } else {
+    store_diag_block(L, A, lda, n, m);
+    if (Y) invert_blocks<float, float>(A, lda, n, Y);
   }
 }
 
@@ -829,7 +1152,9 @@ void launch_assemble(const double* vals, const int64_t* amap, int64_t nnz, void*
   else k_assemble<double><<<blocks, 256, 0, st>>>(vals, amap, nnz, (double*)L);
 }
 
-static size_t potrf_smem(int w) { return potrf_rd_offset(w) + (size_t)w * sizeof(double); }
+static size_t potrf_smem(int w) {  // potrf_blocks, or the block and potrf_lookahead's table
+  return std::max((size_t)w * w * sizeof(double) + update_table_bytes(w), kPotrfBlkSmem);
+}
 
 constexpr int kDinvThreads = 256;
 template <typename P>
@@ -894,33 +1219,35 @@ void launch_diag_inverse(const int4* tasks, int ntasks, const SnDev* sns, bool f
     k_diag_inverse<double><<<ntasks, kDinvThreads, dinv_smem<double>(), st>>>(tasks, sns,
                                                                              skip_sliced);
 }
-static size_t potrf_mixed_smem(int w) {  // the FP64 block of a redo overlays the FP32 one
-  return (size_t)w * w * sizeof(double) + update_table_bytes(w);
-}
+static size_t potrf_mixed_smem(int w) { return potrf_mixed_tab_offset(w) + update_table_bytes(w); }
 static size_t trsm_smem(int w) { return ((size_t)w * w + w + (size_t)w * 32) * sizeof(double); }
 
-void launch_potrf(const int4* tasks, int ntasks, int* queue, const SnDev* sns,
-                  const MatDev* mats, int max_width, bool f32, float tau, void* oy,
-                  int64_t oy_rows, cudaStream_t st) {
+void launch_potrf(const int4* tasks, int ntasks, const SnDev* sns, const MatDev* mats,
+                  int max_width, bool f32, float tau, void* oy, int64_t oy_rows, cudaStream_t st) {
   if (ntasks <= 0) return;
-  if (f32) {
-    const size_t sm = potrf_mixed_smem(max_width);
-    k_potrf_mixed<<<task_grid(k_potrf_mixed, kPotrfThreads, sm, ntasks), kPotrfThreads, sm, st>>>(
-        tasks, ntasks, queue, sns, mats, tau);
-  } else {
-    const size_t sm = potrf_smem(max_width);
-    k_potrf<double><<<task_grid(k_potrf<double>, kPotrfThreads, sm, ntasks), kPotrfThreads, sm, st>>>(
-        tasks, ntasks, queue, sns, mats, static_cast<uint8_t*>(oy), oy_rows);
-  }
+  if (f32)
+    launch_pdl(k_potrf_mixed, ntasks, kPotrfThreads, potrf_mixed_smem(max_width), st, tasks, sns, mats,
+               tau);
+  else
+    launch_pdl(k_potrf, ntasks, kPotrfThreads, potrf_smem(max_width), st, tasks, sns, mats,
+               static_cast<uint8_t*>(oy), oy_rows);
+}
+
+template <typename T, int ROWS>
+static void trsm_blk_t(const int4* tasks, int ntasks, int per, const SnDev* sns, cudaStream_t st) {
+  launch_pdl(k_trsm_blk<T, ROWS>, dim3((ntasks + per - 1) / per, kTrsmRows / ROWS),
+             32 * trsm_warps<ROWS>(), trsm_blk_smem<T, ROWS>(), st, tasks, ntasks, per, sns);
 }
 
 template <typename T>
 static void trsm_t(const int4* tasks, int ntasks, int* queue, const SnDev* sns, int max_width,
                    cudaStream_t st) {
   if (max_width <= 64) {
-    constexpr size_t sm = trsm_blk_smem<T>();
-    k_trsm_blk<T><<<task_grid(k_trsm_blk<T>, 32 * kTrsmWarps, sm, ntasks), 32 * kTrsmWarps, sm, st>>>(
-        tasks, ntasks, queue, sns);
+    // rows per CTA: as few as keep the CTAs within one wave (152 SMs); wide levels four tasks
+    // per CTA while three CTAs per SM are left
+    if (4 * ntasks <= 152) trsm_blk_t<T, 8>(tasks, ntasks, 1, sns, st);
+    else if (2 * ntasks <= 152) trsm_blk_t<T, 16>(tasks, ntasks, 1, sns, st);
+    else trsm_blk_t<T, 32>(tasks, ntasks, ntasks >= 4 * 3 * 152 ? 4 : 1, sns, st);
     return;
   }
   const size_t sm = trsm_smem(max_width);
@@ -1002,10 +1329,14 @@ static bool set_smem(K kernel, size_t bytes) {
 int set_factor_kernel_attrs(int max_width) {
   bool ok = set_smem(k_diag_inverse<double>, dinv_smem<double>()) &&
             set_smem(k_diag_inverse<float>, dinv_smem<float>()) &&
-            set_smem(k_potrf<double>, potrf_smem(max_width)) &&
+            set_smem(k_potrf, potrf_smem(max_width)) &&
             set_smem(k_potrf_mixed, potrf_mixed_smem(max_width)) &&
-            set_smem(k_trsm_blk<double>, trsm_blk_smem<double>()) &&
-            set_smem(k_trsm_blk<float>, trsm_blk_smem<float>()) &&
+            set_smem(k_trsm_blk<double, 32>, trsm_blk_smem<double, 32>()) &&
+            set_smem(k_trsm_blk<double, 16>, trsm_blk_smem<double, 16>()) &&
+            set_smem(k_trsm_blk<double, 8>, trsm_blk_smem<double, 8>()) &&
+            set_smem(k_trsm_blk<float, 32>, trsm_blk_smem<float, 32>()) &&
+            set_smem(k_trsm_blk<float, 16>, trsm_blk_smem<float, 16>()) &&
+            set_smem(k_trsm_blk<float, 8>, trsm_blk_smem<float, 8>()) &&
             set_smem(k_trsm<double>, trsm_smem(max_width)) &&
             set_smem(k_trsm<float>, trsm_smem(max_width));
   return ok ? CHOL_OK : CHOL_E_CUDA;

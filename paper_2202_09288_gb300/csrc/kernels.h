@@ -21,9 +21,8 @@ void launch_diag_inverse(const int4* tasks, int ntasks, const SnDev* sns, bool f
                          bool skip_sliced, cudaStream_t st);
 // oy: with the FP64 factor's tensor-core TRSM, the zeroed scratch (oz_scratch_bytes(oy_rows))
 // that receives the slices of the 128-tile supernodes' Y = L11^-1 (tasks with y set); else null
-void launch_potrf(const int4* tasks, int ntasks, int* queue, const SnDev* sns,
-                  const MatDev* mats, int max_width, bool f32, float tau, void* oy,
-                  int64_t oy_rows, cudaStream_t st);
+void launch_potrf(const int4* tasks, int ntasks, const SnDev* sns, const MatDev* mats,
+                  int max_width, bool f32, float tau, void* oy, int64_t oy_rows, cudaStream_t st);
 void launch_trsm(const int4* tasks, int ntasks, int* queue, const SnDev* sns, int max_width,
                  bool f32, cudaStream_t st);
 void launch_schur(int cls, const int4* tasks, int ntasks, int* queue, const SnDev* sns,

@@ -21,13 +21,15 @@ constexpr int kMaxWidth = 128;   // hard limit on the width cap W (diagonal bloc
 // four 64 x 64 FP64 tiles).
 //
 // FP64 on bf16 tensor cores (operand splitting): a row r of L21 is scaled by 2^-e_r
-// (max |L21[r,:]| < 2^e_r) and cut into kOzSlices integer slices of 7 bits,
-//   L21[r,k] 2^-e_r = sum_p s_p[r,k] 2^(-7(p+1)),  |s_0| <= 128, |s_p| <= 64 (p > 0),
-// each exact in bf16.  Slice products are accumulated exactly in FP32 (every partial sum
-// of one diagonal p+q stays below 2^24 for K <= 128), and
-//   U[i,k] = 2^(e_i+e_k) sum_{p+q < kOzSlices} 2^(-7(p+q+2)) sum_kk s_p[i,kk] s_q[k,kk].
-// The representation error is below 2^-57 of the row maximum.
-constexpr int kOzSlices = 8;
+// (max |L21[r,:]| < 2^e_r), rounded to 55 fraction bits and cut into kOzSlices integer slices of
+// 8 bits,
+//   L21[r,k] 2^-e_r = sum_p s_p[r,k] 2^(-7-8p),  |s_p| <= 128,
+// each exact in bf16.  Slice products are accumulated exactly in FP32 (a partial sum of the
+// diagonal p+q = d is an integer of magnitude <= K (d+1) 2^14, at most 7 2^20 for K <= 64), and
+//   U[i,k] = 2^(e_i+e_k) sum_{p+q < kOzSlices} 2^(-14-8(p+q)) sum_kk s_p[i,kk] s_q[k,kk].
+// The representation error is at most 2^-56 of the row maximum.
+constexpr int kOzSlices = 7;
+constexpr int kOzPlanes = 8;      // planes of a slice scratch (the TF32 parts of 128 columns take 8)
 constexpr int kOzRowBytes = 128;  // one slice row: 64 bf16 (K <= 64), 128-byte swizzled
 constexpr int kOzInvRows = 64;    // slice rows of a diagonal-block inverse (n <= 64, zero-padded)
 enum SchurClass { kTile64 = 0, kTile32 = 1, kTile16 = 2, kTile128 = 3, kNumTileClasses = 4 };

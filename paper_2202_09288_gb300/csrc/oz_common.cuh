@@ -1,9 +1,9 @@
 // oz_common.cuh -- the operand slicing shared by the FP64 tensor-core kernels (the Schur
 // tiles' L21 rows, the TRSM's A21 rows and the rows of the diagonal-block inverses).
 //
-// A row r with exponent e_r (every |x| < 2^e_r) is the 56-bit fixed-point integer
-// x 2^(56-e_r) per entry, cut into kOzSlices balanced digits of 7 bits (|s_0| <= 128,
-// |s_p| <= 64, exact), x = 2^e_r sum_p s_p 2^(-7(p+1)) + (error < 2^(e_r-56)),
+// A row r with exponent e_r (every |x| < 2^e_r) is the integer x 2^(55-e_r) per entry, rounded to
+// nearest, cut into kOzSlices balanced digits of 8 bits (|s_p| <= 128),
+// x = 2^e_r sum_p s_p 2^(-7-8p) + (error <= 2^(e_r-56)),
 // each digit stored as bf16 (exact) in slice planes of 128-byte rows (64 entries, K <= 64)
 // whose 16-byte chunks are pre-swizzled for the tensor cores' 128-byte swizzle: the chunk of
 // columns 8c .. 8c+7 of slice row R sits at physical chunk c ^ (R & 7).
@@ -24,15 +24,16 @@ __device__ __forceinline__ uint32_t oz_f32_bits_of_int(int v) {
   return __float_as_uint(__uint_as_float(0x4B400000u + (uint32_t)v) - 12582912.0f);
 }
 
-// x 2^(56 - e) as an integer (|x| < 2^e, so |result| < 2^56), truncated toward zero below
-// 2^0 (an error below 2^(e-56)); subnormal x give 0.
+// x 2^(55 - e) as an integer (|x| < 2^e, so |result| <= 2^55), rounded to nearest (an error of at
+// most 2^(e-56)); subnormal x give 0.
 __device__ __forceinline__ long long oz_fixed(double x, int e) {
   const long long bits = __double_as_longlong(x);
   const int exb = (int)((bits >> 52) & 0x7FF);
   if (exb == 0) return 0;
   const long long mant = (bits & ((1ll << 52) - 1)) | (1ll << 52);  // x = mant 2^(exb-1075)
-  const int sh = exb - 1019 - e;
-  const long long M = sh >= 0 ? mant << sh : (sh > -64 ? mant >> -sh : 0);
+  const int sh = exb - 1020 - e;
+  const long long M =
+      sh >= 0 ? mant << sh : (sh >= -53 ? (mant + (1ll << (-sh - 1))) >> -sh : 0);
   return bits < 0 ? -M : M;
 }
 
@@ -49,32 +50,32 @@ __device__ __forceinline__ int oz_exp_field(double x) {
 // The 16-byte chunk of logical columns 8c .. 8c+7 of one row in every slice plane: R[j] are
 // the row's fixed-point integers of those columns (oz_fixed, 0 past the row's end); dst the
 // chunk's address in plane 0, planes `stride` bytes apart.
-// Digits, least significant first: d = ((R + 64) mod 128) - 64 in [-64, 63], then R = (R - d)
-// / 2^7 (exact); digit 0 takes what is left, |s_0| <= 128 because |R| < 2^56 and the lower
-// digits sum to less than 2^48 (128/127) in magnitude.  R = hi 2^28 + lo (0 <= lo < 2^28)
-// keeps the work in 32-bit integers: lo gives digits 7 .. 4 and a carry (0 or 1) into hi,
-// which gives digits 3 .. 0.
+// Digits, least significant first: d = ((R + 128) mod 256) - 128 in [-128, 127], then R = (R - d)
+// / 2^8 (exact); digit 0 takes what is left, |s_0| <= 128 because |R| <= 2^55 and the lower
+// digits sum to at most 2^47 (256/255) in magnitude.  After digit 6, R = hi 2^24 + lo (0 <= lo <
+// 2^24) keeps the work in 32-bit integers: lo gives digits 5 .. 3 and a carry (0 or 1) into hi,
+// which gives digits 2 .. 0.
 __device__ __forceinline__ void oz_write_chunk(long long (&R)[8], uint8_t* dst, size_t stride) {
-  static_assert(kOzSlices == 8, "digits 7..4 from the low 28 bits, 3..0 from the rest");
+  static_assert(kOzSlices == 7, "digit 6, digits 5..3 from the next 24 bits, 2..0 from the rest");
   int lo[8], hi[8];
-#pragma unroll
-  for (int j = 0; j < 8; j++) {
-    lo[j] = (int)(R[j] & 0x0FFFFFFFll);
-    hi[j] = (int)(R[j] >> 28);
-  }
 #pragma unroll
   for (int p = kOzSlices - 1; p >= 0; p--) {
     uint32_t h[8];
 #pragma unroll
     for (int j = 0; j < 8; j++) {
       int dg;
-      if (p >= 4) {
-        dg = ((lo[j] + 64) & 127) - 64;
-        lo[j] = (lo[j] - dg) >> 7;
-        if (p == 4) hi[j] += lo[j];  // the carry
+      if (p == 6) {
+        dg = (((int)R[j] + 128) & 255) - 128;
+        const long long r = (R[j] - dg) >> 8;
+        lo[j] = (int)(r & 0xFFFFFFll);
+        hi[j] = (int)(r >> 24);
+      } else if (p >= 3) {
+        dg = ((lo[j] + 128) & 255) - 128;
+        lo[j] = (lo[j] - dg) >> 8;
+        if (p == 3) hi[j] += lo[j];  // the carry
       } else if (p >= 1) {
-        dg = ((hi[j] + 64) & 127) - 64;
-        hi[j] = (hi[j] - dg) >> 7;
+        dg = ((hi[j] + 128) & 255) - 128;
+        hi[j] = (hi[j] - dg) >> 8;
       } else {
         dg = hi[j];
       }

@@ -4,21 +4,21 @@
 // The update U_s = L21 L21^T (Sec. 3, Listing 1: SYRK + GEMM) of a 128-tile supernode is
 // computed in two steps per level:
 //   k_oz_slice  every row r of L21 gets an exponent e_r (max_k |L21[r,k]| < 2^e_r) and
-//               kOzSlices integer slices s_p[r,k] of 7 bits with
-//               L21[r,k] = 2^e_r sum_p s_p[r,k] 2^(-7(p+1)) + (error < 2^(e_r-57)),
+//               kOzSlices integer slices s_p[r,k] of 8 bits with
+//               L21[r,k] = 2^e_r sum_p s_p[r,k] 2^(-7-8p) + (error <= 2^(e_r-56)),
 //               stored as bf16 (exact) in rows of 128 bytes, 16-byte chunks pre-swizzled
 //               for the tensor cores' 128-byte swizzle;
-//   k_schur_oz  a 128 x 128 task is done as four 128 x 32 quarters.  The 8 A slices
-//               (the task's 128 rows) and each quarter's 8 B slices (its 32 rows) are
+//   k_schur_oz  a 128 x 128 task is done as four 128 x 32 quarters.  The 7 A slices
+//               (the task's 128 rows) and each quarter's 7 B slices (its 32 rows) are
 //               brought into shared memory by bulk copies issued by a load thread, which
-//               also claims the tasks; an MMA thread issues, for every slice pair p + q < 8,
+//               also claims the tasks; an MMA thread issues, for every slice pair p + q < 7,
 //               the bf16 MMAs of D_{p+q} += S_p S_q^T into the quarter's set of tensor-memory
-//               accumulators (one per diagonal p + q, 8 x 32 columns; two sets); tasks are
+//               accumulators (one per diagonal p + q, 7 x 32 columns; two sets); tasks are
 //               claimed in runs of up to four, so that the later tiles of a row strip reuse
-//               the A slices.  Every partial sum of a diagonal is an integer below 2^22
+//               the A slices.  Every partial sum of a diagonal is an integer of at most 7 2^20
 //               (K <= 64), so FP32 accumulation is exact.  Consumer warps read a finished
 //               set (lane = tile row), release it, form U[i,k] = 2^(e_i+e_k)
-//               sum_d 2^(-7(d+2)) D_d[i,k] as an FP64 value (integer combination, one
+//               sum_d 2^(-14-8d) D_d[i,k] as an FP64 value (integer combination, one
 //               int64 -> double conversion) and add it into the ancestors with FP64
 //               reductions (or write the owner staging buffer) while the tensor cores compute
 //               the next quarter; metadata warps prepare the coming tasks' targets ahead.
@@ -52,11 +52,12 @@ constexpr int kOzN = 64;                                   // columns per half (
 constexpr uint32_t kOzASlice = kOzM * kOzRowBytes;         // 16 KB
 constexpr int kOzQ = 32;                                   // columns per quarter
 constexpr uint32_t kOzQSlice = kOzQ * kOzRowBytes;         // 4 KB: one slice of a quarter
-constexpr uint32_t kOzQBytes = kOzSlices * kOzQSlice;      // 32 KB: a quarter's B operand
-constexpr int kOzSetCols = kOzSlices * kOzQ;               // 256: TMEM columns of a set
-constexpr uint32_t kOzABytes = kOzSlices * kOzASlice;      // 128 KB
-constexpr size_t kOzSmem = 1024 + kOzABytes + 2 * kOzQBytes;  // + alignment slack
-constexpr uint32_t kOzTmemCols = 2 * kOzSetCols;          // 512: two sets of 8 diagonals
+constexpr uint32_t kOzQBytes = kOzSlices * kOzQSlice;      // 28 KB: a quarter's B operand
+constexpr int kOzSetCols = kOzSlices * kOzQ;               // 224: TMEM columns of a set
+constexpr uint32_t kOzABytes = kOzSlices * kOzASlice;      // 112 KB
+constexpr int kOzBBufs = 3;                                // quarter B buffers
+constexpr size_t kOzSmem = 1024 + kOzABytes + kOzBBufs * kOzQBytes;  // + alignment slack
+constexpr uint32_t kOzTmemCols = 512;                     // two sets of 7 diagonals (448)
 // Bound of every wait in SM clock cycles (~1 s at 2 GHz; the waits of a working launch last
 // microseconds).  Counted with clock64(), not in polls: a poll of mbarrier.try_wait may suspend
 // the thread for a hardware-defined time.
@@ -137,8 +138,8 @@ constexpr int kOzSliceLd = kOzM + 1;  // padded column stride of the staged bloc
 // Slices of the L21 rows r0 .. r0+127 of supernode s, at slice rows oz + r (rows u ..
 // roundup(u, 8) get zero slices).  The block is staged column by column through shared
 // memory (cp.async, all copies in flight); a row's exponent e_r is that of its largest entry; each
-// entry becomes the 56-bit fixed-point integer x 2^(56-e_r), cut into 8 balanced digits
-// of 7 bits (round to nearest: |s_0| <= 128, |s_p| <= 64, exact); thread t writes the
+// entry becomes the integer x 2^(55-e_r), rounded to nearest and cut into 7 balanced digits
+// of 8 bits (|s_p| <= 128, exact); thread t writes the
 // 16-byte chunk t % 8 of row t / 8 of every slice (coalesced, pre-swizzled).
 // With oy (the tensor-core TRSM's operand A21 S^-1, sliced before that TRSM), column k is
 // scaled by 2^-t_k, the shift POTRF stored with the supernode's inverse slices in oy.
@@ -213,36 +214,34 @@ __device__ __forceinline__ void oz_tmem_wait() {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-// The FP32 bits of x + 1.5 * 2^23 for an accumulator x holding an integer of magnitude below
+// The FP32 bits of x + 1.5 * 2^23 for an accumulator x holding an integer of magnitude at most
 // 2^22: 0x4B400000 + x, i.e. the integer plus a fixed offset in the low mantissa bits.
 __device__ __forceinline__ uint32_t oz_fbits(uint32_t acc) {
   return __float_as_uint(__uint_as_float(acc) + 12582912.0f);
 }
+__device__ __forceinline__ int oz_int(uint32_t acc) { return __float2int_rn(__uint_as_float(acc)); }
 
-// W = V_hi 2^20 + round(V_lo / 2^8) from the offset bits f_d = 0x4B400000 + D_d of the eight
-// diagonals (V_hi = sum_{d<4} D_d 2^(7(3-d)), V_lo = sum_{d>=4} D_d 2^(7(7-d)), |D_d| < 2^22, so
-// |W| < 2^62).  The offsets are never subtracted one by one: kOzLoBias = 128 - 0x4B400000 S
-// (S = 1 + 2^7 + 2^14 + 2^21) removes those of V_lo and adds the rounding constant before the
-// shift; the high diagonals enter modulo 2^64 (f_3 2^20 and f_2 2^27 as 32 x 32 -> 64-bit
-// multiply-adds, f_1 2^34 + f_0 2^41 in the high word alone), and kOzHiBias = -(0x4B400000
-// 2^20 S) >> 32 removes their offsets (it has no low word).  Exact since |W| < 2^63.
-constexpr unsigned long long kOzLoBias = 0xfff6850a14c00080ull;
-constexpr uint32_t kOzHiBias = 0x50a14c00u;
+// W = V_hi 2^17 + round(V_lo / 2^7) of the seven diagonals, V_hi = sum_{d<4} D_d 2^(8(3-d)),
+// V_lo = sum_{d>=4} D_d 2^(8(6-d)) (|D_d| <= (d+1) 2^20, so |W| < 2^62).  The low diagonals may
+// exceed 2^22 and come as integers (oz_int); the high ones as offset bits f_d = 0x4B400000 + D_d
+// whose offsets are never subtracted one by one: they enter modulo 2^64 (f_3 2^17 and f_2 2^25 as
+// 32 x 32 -> 64-bit multiply-adds, f_1 2^33 + f_0 2^41 in the high word alone), and kOzHiBias =
+// -(0x4B400000 2^17 (1 + 2^8 + 2^16 + 2^24)) >> 32 removes them (it has no low word).  Exact
+// since |W| < 2^63.
+constexpr uint32_t kOzHiBias = 0u - (uint32_t)((0x4B400000ull * ((1ull << 17) + (1ull << 25))) >> 32) -
+                               0x4B400000u * 2u - 0x4B400000u * 512u;
 
-__device__ __forceinline__ unsigned long long oz_low(uint32_t f4, uint32_t f5, uint32_t f6,
-                                                     uint32_t f7) {
-  unsigned long long v = (unsigned long long)f7 + kOzLoBias;
-  v = (unsigned long long)f6 * 128ull + v;
-  v = (unsigned long long)f5 * 16384ull + v;
-  v = (unsigned long long)f4 * 2097152ull + v;
-  return (unsigned long long)((long long)v >> 8);  // round(V_lo / 2^8), half up
+__device__ __forceinline__ unsigned long long oz_low(int d4, int d5, int d6) {
+  long long v = (long long)d5 * 256 + (d6 + 64);
+  v = (long long)d4 * 65536 + v;
+  return (unsigned long long)(v >> 7);  // round(V_lo / 2^7), half up
 }
 
 __device__ __forceinline__ long long oz_high(unsigned long long lo, uint32_t f0, uint32_t f1,
                                              uint32_t f2, uint32_t f3) {
-  unsigned long long w = (unsigned long long)f3 * 1048576ull + lo;
-  w = (unsigned long long)f2 * 134217728ull + w;
-  w += (unsigned long long)(f1 * 4u + f0 * 512u + kOzHiBias) << 32;
+  unsigned long long w = (unsigned long long)f3 * 131072ull + lo;
+  w = (unsigned long long)f2 * 33554432ull + w;
+  w += (unsigned long long)(f1 * 2u + f0 * 512u + kOzHiBias) << 32;
   return (long long)w;
 }
 
@@ -296,14 +295,15 @@ __device__ __forceinline__ void oz_arrive(uint32_t bar) {
 
 // A task is done as 128 x 32 quarters.  A load thread (its own warp) claims the tasks, hands
 // each one to the other roles through a ring as soon as it has claimed it, and bulk-copies
-// the task's 8 A slices once and every quarter's B slices into one of two quarter buffers;
-// an MMA thread (its own warp) issues each quarter's MMAs into one of two TMEM sets of 8
+// the task's 7 A slices once and every quarter's B slices into one of kOzBBufs quarter buffers;
+// an MMA thread (its own warp) issues each quarter's MMAs into one of two TMEM sets of 7
 // diagonals x 32 columns, slice by slice; the 16 consumer warps drain a finished set (and
 // release it) while the tensor cores compute the next quarter, then scatter; four metadata
 // warps build each task's exponents, column targets and relative rows up to two tasks ahead.
-// Barriers: a_full (a task's 8 A slices in; a task with the previous task's A rows reuses
-// them), b_full[2] (quarter B buffers in), acc_full[2] (a set's MMAs done: also frees the B
-// buffer they read, and after a task's last quarter the A slices), acc_empty[2] (a set
+// Barriers: a_full (a task's 7 A slices in; a task with the previous task's A rows reuses
+// them), a_empty (the MMAs of
+// all tasks that use an A load done), b_full[] / b_empty[] (a quarter B buffer in / read by its
+// MMAs), acc_full[2] (a set's MMAs done), acc_empty[2] (a set
 // drained), meta_full[] / meta_empty[] (a metadata buffer built / released), ring_full[]
 // (the task order).
 template <bool OWNER>
@@ -314,8 +314,9 @@ __global__ void __launch_bounds__(kOzThreads, 1)
   extern __shared__ __align__(1024) unsigned char oz_sm[];
   unsigned char* A =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(oz_sm) + 1023) & ~uintptr_t(1023));
-  unsigned char* Bq0 = A + kOzABytes;  // quarter buffers: Bq0, Bq0 + kOzQBytes
-  __shared__ __align__(8) uint64_t a_full, b_full[2], acc_full[2], acc_empty[2];
+  unsigned char* Bq0 = A + kOzABytes;  // quarter buffers: Bq0, Bq0 + kOzQBytes, ...
+  __shared__ __align__(8) uint64_t a_full, a_empty, b_full[kOzBBufs], b_empty[kOzBBufs];
+  __shared__ __align__(8) uint64_t acc_full[2], acc_empty[2];
   __shared__ __align__(8) uint64_t ring_full[kOzRing];
   __shared__ int2 ring[kOzRing];  // {task, quarters | K steps << 8} (task = ntasks: stop)
   __shared__ uint32_t tmem_base;
@@ -341,9 +342,13 @@ __global__ void __launch_bounds__(kOzThreads, 1)
   if (tid == 0) {
     s_fail = 0;
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&a_full)));
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&a_empty)));
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&never)));
-    for (int i = 0; i < 2; i++) {
+    for (int i = 0; i < kOzBBufs; i++) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&b_full[i])));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&b_empty[i])));
+    }
+    for (int i = 0; i < 2; i++) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&acc_full[i])));
       asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&acc_empty[i])),
                    "r"(kOzConsumers / 64));  // the 8 warps of the set's consumer group
@@ -367,7 +372,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
     // ---------------- loads: task claims, ring, bulk copies; one thread ----------------
     if (lane == 0) {
       long long T = 0;                       // A slice loads issued
-      long long qb = 0;                      // quarter B buffers issued (buffer = qb & 1)
+      long long qb = 0;                      // quarter B buffers issued (buffer = qb % kOzBBufs)
       long long ord = 0;                     // ring entries published
       bool ok = true;
       // Tasks are claimed in runs (g0 per CTA at first, then from the queue): four while more
@@ -415,10 +420,10 @@ __global__ void __launch_bounds__(kOzThreads, 1)
         const Job next = publish(tq);  // the next task (or the stop entry)
         const int4 t = job.t;
         const int nq = job.nq;
-        // quarter j's B slices, once the MMAs of the quarter two back (same buffer) are done
+        // quarter j's B slices, once the MMAs of the quarter before it in the buffer are done
         auto load_b = [&](int j) -> bool {
-          const int b = (int)(qb & 1);
-          if (qb >= 2 && !oz_wait(smem_u32(&acc_full[b]), (uint32_t)(((qb >> 1) - 1) & 1)))
+          const int b = (int)(qb % kOzBBufs);
+          if (qb >= kOzBBufs && !oz_wait(smem_u32(&b_empty[b]), (uint32_t)((qb / kOzBBufs - 1) & 1)))
             return false;
           const uint32_t bar = smem_u32(&b_full[b]);
           unsigned char* dst = Bq0 + b * kOzQBytes;
@@ -430,17 +435,14 @@ __global__ void __launch_bounds__(kOzThreads, 1)
           qb++;
           return true;
         };
-        // the first quarter's B goes first: its buffer is free before the A slices are
-        if (!load_b(0)) {
-          ok = false;
-          break;
-        }
+        // the first quarters' B goes first: its buffers are free before the A slices are
+        const int early = min(nq, kOzBBufs - 1);
+        for (int j = 0; j < early && ok; j++) ok = load_b(j);
+        if (!ok) break;
         // the A slices of this task (unless the previous task had the same rows), once the
-        // previous task's last quarter (the latest quarter before this task's first, qb - 2)
-        // is done: every K step reads every slice
+        // previous task's MMAs are done: every K step reads every slice
         if (!job.reuse) {
-          if (T >= 1 &&
-              !oz_wait(smem_u32(&acc_full[(qb - 2) & 1]), (uint32_t)(((qb - 2) >> 1) & 1))) {
+          if (T >= 1 && !oz_wait(smem_u32(&a_empty), (uint32_t)((T - 1) & 1))) {
             ok = false;
             break;
           }
@@ -451,7 +453,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
                          smem_u32(&a_full));
           T++;
         }
-        for (int j = 1; j < nq && ok; j++) ok = load_b(j);
+        for (int j = early; j < nq && ok; j++) ok = load_b(j);
         if (!ok) break;
         job = next;
         cur = tq;
@@ -465,20 +467,20 @@ __global__ void __launch_bounds__(kOzThreads, 1)
       // bounded waits for the copies still in flight: the last A load and the last B load of
       // each buffer
       if (T >= 1) oz_wait(smem_u32(&a_full), (uint32_t)((T - 1) & 1));
-      for (long long qq = qb - 2 < 0 ? 0 : qb - 2; qq < qb; qq++)
-        oz_wait(smem_u32(&b_full[qq & 1]), (uint32_t)((qq >> 1) & 1));
+      for (long long qq = qb - kOzBBufs < 0 ? 0 : qb - kOzBBufs; qq < qb; qq++)
+        oz_wait(smem_u32(&b_full[qq % kOzBBufs]), (uint32_t)((qq / kOzBBufs) & 1));
     }
   } else if (warp == kOzMmaWarp) {
     // ---------------- MMAs, one thread ----------------
     if (lane == 0) {
-      // N = (8 - p) x 32: the MMA of slice p against slices 0 .. 7-p of a quarter
+      // N = (7 - p) x 32: the MMA of slice p against slices 0 .. 6-p of a quarter
       uint32_t idesc[kOzSlices];
 #pragma unroll
       for (int p = 0; p < kOzSlices; p++) idesc[p] = oz_idesc((kOzSlices - p) * kOzQ);
       const uint64_t da0 = oz_desc(smem_u32(A));
-      const uint64_t db[2] = {oz_desc(smem_u32(Bq0)), oz_desc(smem_u32(Bq0 + kOzQBytes))};
+      const uint64_t db0 = oz_desc(smem_u32(Bq0));
       bool ok = true;
-      long long q = 0;  // quarters issued (TMEM set and B buffer = q & 1)
+      long long q = 0;  // quarters issued (TMEM set q & 1, B buffer q % kOzBBufs)
       long long T = 0;  // A slice loads waited for
       for (long long ord = 0; ok; ord++) {
         const int rs = (int)(ord % kOzRing);
@@ -490,9 +492,13 @@ __global__ void __launch_bounds__(kOzThreads, 1)
         if (e.x >= ntasks) break;
         const int nq = e.y & 0xff, ks = (e.y >> 8) & 0xff;
         const bool reuse = (e.y >> 16) & 1;  // the previous task's A slices
+        // the A slices are free when every MMA so far is done (one commit per A load, so that the
+        // load thread, which waits for each, is never two phases apart from this one)
+        if (!reuse && T > 0) oz_commit(smem_u32(&a_empty));
         for (int j = 0; j < nq; j++, q++) {
-          const int b = (int)(q & 1);
-          if (!oz_wait(smem_u32(&b_full[b]), (uint32_t)((q >> 1) & 1)) ||
+          const int b = (int)(q & 1), bb = (int)(q % kOzBBufs);
+          const uint64_t db = db0 + (uint64_t)((bb * kOzQBytes) >> 4);
+          if (!oz_wait(smem_u32(&b_full[bb]), (uint32_t)((q / kOzBBufs) & 1)) ||
               (q >= 2 &&  // the set was drained (quarter q - 2)
                !oz_wait(smem_u32(&acc_empty[b]), (uint32_t)(((q >> 1) - 1) & 1)))) {
             ok = false;
@@ -509,9 +515,10 @@ __global__ void __launch_bounds__(kOzThreads, 1)
 #pragma unroll
             for (int p = 0; p < kOzSlices; p++)
               oz_mma(tmem + (uint32_t)(b * kOzSetCols + p * kOzQ),
-                     da0 + (uint64_t)((p * kOzASlice) >> 4) + 2 * k, db[b] + 2 * k, idesc[p],
+                     da0 + (uint64_t)((p * kOzASlice) >> 4) + 2 * k, db + 2 * k, idesc[p],
                      (p > 0 || k > 0) ? 1u : 0u);
           oz_commit(smem_u32(&acc_full[b]));
+          oz_commit(smem_u32(&b_empty[bb]));
         }
         if (!reuse) T++;
       }
@@ -660,21 +667,20 @@ __global__ void __launch_bounds__(kOzThreads, 1)
           const bool dead = r0w >= u || gk0 >= u || r0w + 31 < gk0;
           double val[8];
           if (!dead) {
-            // the 8 diagonals of the chunk's columns -> W (exact integer) -> U = W 2^(e_i +
+            // the 7 diagonals of the chunk's columns -> W (exact integer) -> U = W 2^(e_i +
             // e_k - 55)
             const uint32_t ta =
                 tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(b * kOzSetCols + c8);
             unsigned long long w[8];
             {
-              uint32_t v[4][8];
+              uint32_t v[3][8];
 #pragma unroll
-              for (int dd = 0; dd < 4; dd++)
+              for (int dd = 0; dd < 3; dd++)
                 oz_tmem_load8(ta + (uint32_t)((4 + dd) * kOzQ), v[dd]);
               oz_tmem_wait();
 #pragma unroll
               for (int jj = 0; jj < 8; jj++)
-                w[jj] = oz_low(oz_fbits(v[0][jj]), oz_fbits(v[1][jj]), oz_fbits(v[2][jj]),
-                               oz_fbits(v[3][jj]));
+                w[jj] = oz_low(oz_int(v[0][jj]), oz_int(v[1][jj]), oz_int(v[2][jj]));
             }
             {
               uint32_t v[4][8];
@@ -757,12 +763,12 @@ __global__ void __launch_bounds__(kOzThreads, 1)
 // slices of Y S (S = diag(2^t_k), t_k the exponent of L11[k,k]) and the shifts t_k in oy; the
 // slices of A21 S^-1 come from the slicing kernel run on the panel just before.  L21 =
 // (A21 S^-1)(Y S)^T is a product of row-sliced operands of exactly the Schur tiles' form,
-// L21[i, j] = 2^(e_i + e_j) sum_{p+q<8} 2^(-7(p+q+2)) sum_k a_p[i,k] y_q[j,k], K = n <= 64, so
-// every diagonal's partial sums are integers below 2^22 (exact in FP32) and the combination is
+// L21[i, j] = 2^(e_i + e_j) sum_{p+q<7} 2^(-14-8(p+q)) sum_k a_p[i,k] y_q[j,k], K = n <= 64, so
+// every diagonal's partial sums are exact in FP32 and the combination is
 // the same integer one.  One CTA per task (128 rows of A21): one thread bulk-copies the task's
-// 8 A slices (128 KB) and Y's 8 slices (64 rows each, 64 KB), then issues, per K step and A
-// slice p, the MMAs of A_p against Y slices 0 .. 7-p in one go (N = (8-p) 64, at most 256 per
-// MMA): diagonal p + q lands at TMEM columns (p + q) 64, the 8 diagonals fill the 512 columns.
+// 7 A slices (112 KB) and Y's 7 slices (64 rows each, 56 KB), then issues, per K step and A
+// slice p, the MMAs of A_p against Y slices 0 .. 6-p in one go (N = (7-p) 64, at most 256 per
+// MMA): diagonal p + q lands at TMEM columns (p + q) 64.
 // Eight warps then read the accumulators (warp w: TMEM lanes 32 (w & 3) .., columns
 // 32 (w >> 2) ..), combine them exactly, round once to FP64 and store L21 into the panel.
 // (Forming the slices inside this kernel as well was measured slower: one CTA per SM then
@@ -770,9 +776,9 @@ __global__ void __launch_bounds__(kOzThreads, 1)
 // Waits are bounded as in the Schur tiles; a timeout is recorded in err[3] and nothing stored.
 constexpr int kToThreads = 256;
 constexpr uint32_t kToBSlice = kOzInvRows * kOzRowBytes;  // 8 KB: one slice of Y's rows
-constexpr uint32_t kToBBytes = kOzSlices * kToBSlice;      // 64 KB
+constexpr uint32_t kToBBytes = kOzSlices * kToBSlice;      // 56 KB
 constexpr size_t kToSmem = 1024 + kOzABytes + kToBBytes;   // + alignment slack
-constexpr uint32_t kToTmemCols = kOzSlices * kOzInvRows;   // 512
+constexpr uint32_t kToTmemCols = 512;                      // 7 diagonals of 64 columns
 
 __global__ void __launch_bounds__(kToThreads, 1)
     k_trsm_oz(const int4* __restrict__ tasks, const SnDev* __restrict__ sns,
@@ -864,8 +870,7 @@ __global__ void __launch_bounds__(kToThreads, 1)
       for (int j = 0; j < 8; j++) {
         const int col = col0 + j;
         if (i < rb && col < n) {
-          const unsigned long long lo =
-              oz_low(oz_fbits(v[4][j]), oz_fbits(v[5][j]), oz_fbits(v[6][j]), oz_fbits(v[7][j]));
+          const unsigned long long lo = oz_low(oz_int(v[4][j]), oz_int(v[5][j]), oz_int(v[6][j]));
           const long long W =
               oz_high(lo, oz_fbits(v[0][j]), oz_fbits(v[1][j]), oz_fbits(v[2][j]), oz_fbits(v[3][j]));
           out[(int64_t)col * m] = oz_to_double<false>(W, eA + ey[yrow + col]);
@@ -920,7 +925,7 @@ void launch_schur_oz(const int4* tasks, int ntasks, int* queue, const SnDev* sns
 }
 
 size_t oz_scratch_bytes(int64_t oz_rows) {
-  return (size_t)oz_rows * (kOzSlices * kOzRowBytes + sizeof(int32_t));
+  return (size_t)oz_rows * (kOzPlanes * kOzRowBytes + sizeof(int32_t));
 }
 
 int set_oz_kernel_attrs() {

@@ -587,10 +587,106 @@ double partition_tree(int32_t nv, const int32_t* parent, const double* work, int
   return imbalance;
 }
 
+namespace {
+
+int32_t width(const Sym* S, int32_t s) { return S->sn_start[s + 1] - S->sn_start[s]; }
+int32_t below(const Sym* S, int32_t s) { return S->sn_m[s] - width(S, s); }
+int64_t slice_rows(int64_t u) { return (u + 7) / 8 * 8; }
+
+// Groups of chunks whose updates are merged (SchurSeg): group_last[s] is the last chunk of s's
+// group (s itself without one).  A group's chunks follow one another in one separator (each
+// one's rows are the columns of the next, then the next one's rows), all in the 128-tile class,
+// all but the first a multiple of 8 wide (their rows below the group then start on a slice
+// row of 8).  The earlier chunks' rows below the group are sliced again at the last one's level:
+// a level takes groups while its slice rows, of row_bytes each, stay within the scratch of
+// the largest level without them.
+std::vector<int32_t> merge_groups(const Sym* S, const std::vector<int8_t>& cls, int most_chunks,
+                                  int64_t row_bytes) {
+  std::vector<int32_t> last(S->ns);
+  for (int32_t s = 0; s < S->ns; s++) last[s] = s;
+  std::vector<int64_t> rows(S->nlev, 0);
+  int64_t most = 0;
+  for (int32_t s = 0; s < S->ns; s++)
+    if (cls[s] == kTile128) {
+      rows[S->sn_level[s]] += slice_rows(below(S, s));
+      most = std::max(most, rows[S->sn_level[s]]);
+    }
+  const int64_t cap = (most + 128) * (kOzPlanes * kOzRowBytes + 4) / row_bytes - 128;
+  for (int32_t s = 0; s < S->ns;) {
+    int32_t e = s;
+    if (cls[s] == kTile128)
+      while (e - s + 1 < most_chunks && e + 1 < S->ns && cls[e + 1] == kTile128 &&
+             S->sn_parent[e] == e + 1 && S->sn_m[e + 1] == below(S, e) && width(S, e + 1) % 8 == 0)
+        e++;
+    for (; e > s; e--) {  // as many chunks as fit
+      int64_t& r = rows[S->sn_level[e]];
+      const int64_t extra = (e - s) * slice_rows(below(S, e));
+      if (r + extra > cap) continue;
+      r += extra;
+      for (int32_t q = s; q < e; q++) last[q] = e;
+      break;
+    }
+    s = e + 1;
+  }
+  return last;
+}
+
+void push_seg(std::vector<int32_t>& v, const SchurSeg& g) {
+  v.insert(v.end(), {g.s, g.oz, g.kind, g.first, g.w, g.g, g.nt, g.count});
+}
+
+// Level l's segment lists and the groups' slice tasks (f32: of the TF32 tiles, otherwise of the
+// FP64 ones and the plain list).
+void build_segments(Sym* S, int32_t l, const std::vector<int8_t>& cls,
+                    const std::vector<int32_t>& last, bool f32) {
+  int32_t oz = 0, plain = 0, merged = 0;
+  int64_t extra = S->lvl_ozrows[l];  // slice rows of the earlier chunks follow the level's own
+  std::vector<int32_t>& sl = S->tasks[f32 ? kTaskSliceMergeF : kTaskSliceMerge];
+  const std::vector<int32_t>& own = S->tasks[kTaskOzSlice];
+  sl.insert(sl.end(), own.begin() + 4 * S->task_off[kTaskOzSlice][l], own.end());
+  for (int32_t q = S->lvl_ptr[l]; q < S->lvl_ptr[l + 1]; q++) {
+    const int32_t s = S->lvl_sn[q];
+    if (cls[s] != kTile128) continue;
+    const int32_t u = below(S, s), nt = (u + 127) / 128;
+    SchurSeg g{s, oz, kSegAll, plain, 0, 1, nt, nt * (nt + 1) / 2};
+    if (!f32) push_seg(S->tasks[kTaskSeg], g);
+    plain += g.count;
+    g.first = merged;
+    int32_t first = s;  // of the group that ends with s
+    while (first > 0 && last[first - 1] == s) first--;
+    if (last[s] > s) {
+      g.kind = kSegInner;
+      g.w = S->sn_start[last[s] + 1] - S->sn_start[s + 1];
+      g.count = 0;
+      for (int32_t a = 0; a < nt; a++) g.count += std::min(a + 1, (g.w + 127) / 128);
+    } else if (first < s) {
+      g.kind = kSegOuter;
+      g.w = static_cast<int32_t>(extra);
+      g.g = s - first + 1;
+      if (!f32) g.count *= g.g;
+      for (int32_t c = first; c < s; c++) {
+        const int32_t w = S->sn_start[s + 1] - S->sn_start[c + 1];  // rows of c inside the group
+        for (int32_t r0 = 0; r0 < u; r0 += 128)
+          push4(sl, c, w + r0, static_cast<int32_t>(extra) - w, -1);
+        extra += slice_rows(u);
+      }
+    }
+    push_seg(S->tasks[f32 ? kTaskSegMergeF : kTaskSegMerge], g);
+    merged += g.count;
+    oz += static_cast<int32_t>(slice_rows(u));
+  }
+  (f32 ? S->lvl_mozrows_f : S->lvl_mozrows)[l] = extra;
+  if (!f32) S->lvl_segtasks[l] = plain;
+  (f32 ? S->lvl_msegtasks_f : S->lvl_msegtasks)[l] = merged;
+}
+
+}  // namespace
+
 void build_schur_tasks(Sym* S, const TilePolicy& policy) {
   S->policy = policy;
   const int kinds[] = {kTaskSchur64, kTaskSchur32, kTaskSchur16, kTaskSchur128, kTaskOzSlice,
-                       kTaskTrsmRest};
+                       kTaskTrsmRest, kTaskSeg, kTaskSegMerge, kTaskSliceMerge, kTaskSegMergeF,
+                       kTaskSliceMergeF};
   for (int k : kinds) {
     S->tasks[k].clear();
     S->task_off[k].assign(S->nlev + 1, 0);
@@ -598,6 +694,11 @@ void build_schur_tasks(Sym* S, const TilePolicy& policy) {
   }
   S->lvl_ozrows.assign(S->nlev, 0);
   S->oz_rows = 0;
+  S->lvl_mozrows.assign(S->nlev, 0);
+  S->lvl_mozrows_f.assign(S->nlev, 0);
+  S->lvl_segtasks.assign(S->nlev, 0);
+  S->lvl_msegtasks.assign(S->nlev, 0);
+  S->lvl_msegtasks_f.assign(S->nlev, 0);
   S->lvl_oyrows.assign(S->nlev, 0);
   S->lvl_trsmoz.assign(S->nlev, 0);
   S->oy_rows = 0;
@@ -656,6 +757,16 @@ void build_schur_tasks(Sym* S, const TilePolicy& policy) {
       }
     }
   }
+  std::vector<int8_t> cls1(S->ns, -1);  // the final tile classes (-1: no rows below)
+  for (int32_t s = 0; s < S->ns; s++) {
+    const int32_t u = S->sn_m[s] - (S->sn_start[s + 1] - S->sn_start[s]);
+    if (u > 0) cls1[s] = static_cast<int8_t>(whole[s] ? whole_tile_class(u) : cls0[s]);
+  }
+  // a scratch of kOzPlanes planes holds kOzSlices planes of FP64 slices, or four of the TF32 parts
+  // of up to 64 columns (wider factors keep plain tiles)
+  const std::vector<int32_t> group = merge_groups(S, cls1, kMergeChunks, kOzSlices * kOzRowBytes + 4);
+  const std::vector<int32_t> group_f =
+      merge_groups(S, cls1, S->max_width <= 64 ? kMergeChunksF32 : 1, kTfPlanes64 * kOzRowBytes);
   // pass 2: the task lists.  The 128-tile supernodes (FP64: slices on the tensor cores) of a
   // level whose 128-tile rows add up to policy.min_rows_trsm_tc also get their TRSM on the
   // tensor cores, with the slices of their diagonal blocks' inverses at 64 rows each of the
@@ -667,7 +778,7 @@ void build_schur_tasks(Sym* S, const TilePolicy& policy) {
     for (int32_t q = S->lvl_ptr[l]; q < S->lvl_ptr[l + 1]; q++) {
       const int32_t s = S->lvl_sn[q];
       const int32_t u = S->sn_m[s] - (S->sn_start[s + 1] - S->sn_start[s]);
-      if (u > 0 && (whole[s] ? whole_tile_class(u) : cls0[s]) == kTile128) rows128 += u;
+      if (cls1[s] == kTile128) rows128 += u;
     }
     const bool wide = rows128 >= policy.min_rows_trsm_tc;
     for (int32_t q = S->lvl_ptr[l]; q < S->lvl_ptr[l + 1]; q++) {
@@ -675,7 +786,7 @@ void build_schur_tasks(Sym* S, const TilePolicy& policy) {
       const int32_t w = S->sn_start[s + 1] - S->sn_start[s];
       const int32_t u = S->sn_m[s] - w;
       if (u <= 0) continue;
-      const int cls = whole[s] ? whole_tile_class(u) : cls0[s];
+      const int cls = cls1[s];
       const int T = tile_of_class(cls), k = schur_kind(cls);
       S->lvl_flops[k][l] += (double)u * (u + 1.0) * w;
       const bool tc = cls == kTile128 && wide;  // TRSM on the tensor cores
@@ -700,6 +811,8 @@ void build_schur_tasks(Sym* S, const TilePolicy& policy) {
     }
     S->lvl_ozrows[l] = ozrow;
     if (ozrow > 0) S->oz_rows = std::max(S->oz_rows, ozrow + 128);
+    build_segments(S, l, cls1, group, false);
+    build_segments(S, l, cls1, group_f, true);
     S->lvl_oyrows[l] = oyrow;
     S->oy_rows = std::max(S->oy_rows, oyrow);
     for (int k : kinds) S->task_off[k][l + 1] = (int64_t)S->tasks[k].size() / 4;

@@ -130,7 +130,8 @@ void free_devsym(chol_sym* s) {
                   d.fg_row,   d.fg_ent,   d.sn_start, d.sn_rowptr, d.sn_run0, d.run_a,
                   d.run_t,    d.run_base, d.relmap};
   for (void* p : ptrs) dev_free(c, p);
-  for (int k = 0; k < chol::kNumTaskKinds; k++) dev_free(c, d.tasks[k]);
+  for (int k = 0; k < chol::kNumTaskKinds; k++)
+    if (k != chol::kTaskBwd) dev_free(c, d.tasks[k]);  // (the forward tasks' list)
   d = DevSym();
   c->syms.erase(s);
   s->ctx = nullptr;
@@ -159,11 +160,14 @@ int ensure_uploaded(chol_ctx* c, chol_sym* s) {
     free_devsym(s);
     return rc;
   }
+  // the forward and the backward solve have the same row blocks: one list on the device
   for (int k = 0; k < chol::kNumTaskKinds; k++)
-    if ((rc = upload(c, reinterpret_cast<int32_t**>(&d.tasks[k]), S.tasks[k], &acc))) {
+    if (k != chol::kTaskBwd &&
+        (rc = upload(c, reinterpret_cast<int32_t**>(&d.tasks[k]), S.tasks[k], &acc))) {
       free_devsym(s);
       return rc;
     }
+  d.tasks[chol::kTaskBwd] = d.tasks[chol::kTaskFwd];
   // the relative map, built once per pattern on the device
   unsigned long long* miss = nullptr;
   if ((rc = upload(c, &d.sn_start, S.sn_start, &acc)) ||
@@ -312,6 +316,9 @@ TaskView sym_view(const chol_sym* sym) {
   }
   v.asm_src = sym->dev.asm_src;
   v.trsmoz = S.lvl_trsmoz.data();
+  v.segtasks = S.lvl_segtasks.data();
+  v.msegtasks = S.lvl_msegtasks.data();
+  v.msegtasks_f = S.lvl_msegtasks_f.data();
   v.nlev = S.nlev;
   v.max_width = (int)S.max_width;
   return v;
@@ -328,6 +335,10 @@ int enqueue_levels(chol_ctx* c, const TaskView& v, const SnDev* sns, const MatDe
                    int64_t oy_rows) {
   // FP64 factors with the slice scratches: 128-tile supernodes take the tensor-core TRSM
   const bool trsm_oz = oz && oy && !f32;
+  // chunks' Schur updates merged (SchurSeg), but for owner assembly
+  const int slices = owner ? chol::kTaskOzSlice : f32 ? chol::kTaskSliceMergeF : chol::kTaskSliceMerge;
+  const int segs = owner ? chol::kTaskSeg : f32 ? chol::kTaskSegMergeF : chol::kTaskSegMerge;
+  const int32_t* segtasks = owner ? v.segtasks : f32 ? v.msegtasks_f : v.msegtasks;
   cudaStream_t st = c->stream;
   CK(cudaMemsetAsync(ctr, 0, factor_counters(v.nlev) * sizeof(int), st));
   const float tau = (float)(c->opts.pivot_tau > 0 ? c->opts.pivot_tau : 1e-5);
@@ -365,7 +376,7 @@ int enqueue_levels(chol_ctx* c, const TaskView& v, const SnDev* sns, const MatDe
     // 128-tiles on the tensor cores: FP64 by bf16 slices, FP32 by TF32 hi/lo parts; their
     // operands are prepared per level after TRSM
     if (oz) {
-      t = v.level(chol::kTaskOzSlice, l, &cnt);
+      t = v.level(slices, l, &cnt);
       if (cnt > 0) {
         prof_begin(c, kProfOzSlice);
         if (f32) chol::launch_tf32_split(t, cnt, sns, v.max_width, oz, oz_rows, st);
@@ -380,10 +391,14 @@ int enqueue_levels(chol_ctx* c, const TaskView& v, const SnDev* sns, const MatDe
       const bool tcc = oz && cls == chol::kTile128;
       const int pk = prof_schur_kind(cls, f32, tcc && !f32);
       prof_begin(c, pk);
+      int nseg = 0;  // in int4
+      if (tcc) t = v.level(segs, l, &nseg);
       if (tcc && f32)
-        chol::launch_schur_tc(t, cnt, q + 2 + cls, sns, mats, owner, oz, oz_rows, c->acc_wait, st);
+        chol::launch_schur_tc(t, nseg / 2, segtasks[l], q + 2 + cls, sns, mats, owner, v.max_width, oz,
+                              oz_rows, c->acc_wait, st);
       else if (tcc)
-        chol::launch_schur_oz(t, cnt, q + 2 + cls, sns, mats, owner, oz, oz_rows, c->acc_wait, st);
+        chol::launch_schur_oz(t, nseg / 2, segtasks[l], q + 2 + cls, sns, mats, owner, oz, oz_rows,
+                              c->acc_wait, st);
       else chol::launch_schur(cls, t, cnt, q + 2 + cls, sns, mats, owner, f32, st);
       prof_end(c, pk, v.flops[kind][l], 0.0);
     }
@@ -444,7 +459,8 @@ int ensure_oz(chol_num* f, void** oz, int64_t* rows, void** oy, int64_t* oy_rows
   int rc = grow_scratch(f->ctx, &f->d_oz, &f->oz_cap, S.oz_rows, false);
   if (rc) return rc;
   *oz = f->d_oz;
-  *rows = f->oz_cap;
+  *rows = f->precision == CHOL_MIXED ? chol::tf_stride_rows(f->oz_cap, (int)S.max_width)
+                                     : chol::oz_stride_rows(f->oz_cap);
   // FP64: the slices of the 128-tile supernodes' diagonal-block inverses (tensor-core TRSM)
   if (f->precision != CHOL_MIXED && S.oy_rows > 0 && f->d_dinv) {
     if ((rc = grow_scratch(f->ctx, &f->d_oy, &f->oy_cap, S.oy_rows, true))) return rc;
@@ -679,7 +695,8 @@ size_t sym_upload_bytes(const chol_sym* sym) {
              S.csr_ptr.size() * 8 + S.csr_col.size() * 4 + S.csr_src.size() * 4 +
              S.asm_src.size() * 4 + S.fg_ptr.size() * 8 + S.fg_row.size() * 4 +
              S.fg_ent.size() * 4;
-  for (int k = 0; k < chol::kNumTaskKinds; k++) b += S.tasks[k].size() * 4;
+  for (int k = 0; k < chol::kNumTaskKinds; k++)
+    if (k != chol::kTaskBwd) b += S.tasks[k].size() * 4;
   b += (size_t)S.relmap_size * 4 + S.run_a.size() * 16 + S.sn_run0.size() * 4 +
        S.sn_start.size() * 4 + S.sn_rowptr.size() * 8;
   return b + 64 * 16;

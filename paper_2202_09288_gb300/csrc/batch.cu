@@ -40,6 +40,7 @@ struct chol_batch {
   void* d_oy = nullptr;  // FP64 tensor-core TRSM: slices of the members' inverses
   int64_t oy_rows = 0;
   std::vector<int32_t> trsmoz;  // per level: the members' tensor-core TRSM supernodes
+  std::vector<int32_t> segtasks, msegtasks, msegtasks_f;  // per level: tasks of the segment lists
   int32_t nlev = 0;
   int max_width = 0;
   // captured factorization
@@ -83,9 +84,17 @@ chol::rt::TaskView batch_view(const chol_batch* b) {
   }
   v.asm_src = b->d_asm_src;
   v.trsmoz = b->trsmoz.data();
+  v.segtasks = b->segtasks.data();
+  v.msegtasks = b->msegtasks.data();
+  v.msegtasks_f = b->msegtasks_f.data();
   v.nlev = b->nlev;
   v.max_width = b->max_width;
   return v;
+}
+
+// rows per plane of the batch's slice scratch
+int64_t stride_rows(const chol_batch* b) {
+  return b->f32 ? chol::tf_stride_rows(b->oz_rows, b->max_width) : chol::oz_stride_rows(b->oz_rows);
 }
 
 int enqueue_batch(chol_batch* b) {
@@ -94,12 +103,14 @@ int enqueue_batch(chol_batch* b) {
     if (rc) return rc;
   }
   return enqueue_levels(b->ctx, batch_view(b), b->d_sn, b->d_mat, b->f32, b->owner, b->d_ctr,
-                        b->d_oz, b->oz_rows, b->d_oy, b->oy_rows);
+                        b->d_oz, stride_rows(b), b->d_oy, b->oy_rows);
 }
 
 const int kFactorKinds[] = {chol::kTaskPotrf,    chol::kTaskTrsm,     chol::kTaskSchur64,
                             chol::kTaskSchur32,  chol::kTaskSchur16, chol::kTaskSchur128,
-                            chol::kTaskOzSlice, chol::kTaskTrsmRest, chol::kTaskAsm};
+                            chol::kTaskOzSlice, chol::kTaskTrsmRest, chol::kTaskAsm,
+                            chol::kTaskSeg, chol::kTaskSegMerge, chol::kTaskSliceMerge,
+                            chol::kTaskSegMergeF, chol::kTaskSliceMergeF};
 
 }  // namespace
 
@@ -160,6 +171,9 @@ int chol_batch_create(chol_ctx* c, int count, chol_num* const* nums, chol_batch*
   for (int i = 0; i < count; i++) oy = oy && nums[i]->d_dinv != nullptr;
   std::vector<int64_t> ozbase(count), oybase(count);
   b->trsmoz.assign(b->nlev, 0);
+  b->segtasks.assign(b->nlev, 0);
+  b->msegtasks.assign(b->nlev, 0);
+  b->msegtasks_f.assign(b->nlev, 0);
   for (int32_t l = 0; l < b->nlev; l++) {
     int64_t total = 0, ytotal = 0;
     for (int i = 0; i < count; i++) {
@@ -167,12 +181,14 @@ int chol_batch_create(chol_ctx* c, int count, chol_num* const* nums, chol_batch*
       ozbase[i] = total;
       oybase[i] = ytotal;
       if (l < S.nlev) {
-        total += S.lvl_ozrows[l];
+        total += b->owner ? S.lvl_ozrows[l] : b->f32 ? S.lvl_mozrows_f[l] : S.lvl_mozrows[l];
         ytotal += S.lvl_oyrows[l];
         b->trsmoz[l] += S.lvl_trsmoz[l];
       }
     }
-    if (oz && total > 0) b->oz_rows = std::max(b->oz_rows, total + 128);
+    if (oz && total > 0)
+      while (stride_rows(b) < total + 128)
+        b->oz_rows += std::max<int64_t>(1, (total + 128 - b->oz_rows) / 2);
     if (oy) b->oy_rows = std::max(b->oy_rows, ytotal);
     for (int k : kFactorKinds) {
       for (int i = 0; i < count; i++) {
@@ -186,7 +202,19 @@ int chol_batch_create(chol_ctx* c, int count, chol_num* const* nums, chol_batch*
                                {t[0] + base[i], t[1], t[2] + src_base[i], t[3] + src_base[i]});
           } else if (k == chol::kTaskSchur128) {  // {s, i0, k0, oz}
             b->tasks[k].insert(b->tasks[k].end(), {t[0] + base[i], t[1], t[2], t[3] + zb});
-          } else if (k == chol::kTaskOzSlice) {   // {s, r0, oz, y}
+          } else if (k == chol::kTaskSeg || k == chol::kTaskSegMerge ||
+                     k == chol::kTaskSegMergeF) {  // SchurSeg, two int4
+            if ((q - S.task_off[k][l]) % 2 == 0) {  // {s, oz, kind, first}
+              const int32_t f0 = (k == chol::kTaskSeg        ? b->segtasks
+                                  : k == chol::kTaskSegMerge ? b->msegtasks
+                                                             : b->msegtasks_f)[l];
+              b->tasks[k].insert(b->tasks[k].end(), {t[0] + base[i], t[1] + zb, t[2], t[3] + f0});
+            } else {  // {w, g, nt, count}: w is a slice row of kSegOuter
+              b->tasks[k].insert(b->tasks[k].end(),
+                                 {t[-2] == chol::kSegOuter ? t[0] + zb : t[0], t[1], t[2], t[3]});
+            }
+          } else if (k == chol::kTaskOzSlice || k == chol::kTaskSliceMerge ||
+                     k == chol::kTaskSliceMergeF) {  // {s, r0, oz, y}
             b->tasks[k].insert(b->tasks[k].end(),
                                {t[0] + base[i], t[1], t[2] + zb, t[3] >= 0 ? t[3] + yb : -1});
           } else if (k == chol::kTaskPotrf) {     // {s, first_bwd, nbwd, y or -1}
@@ -197,6 +225,9 @@ int chol_batch_create(chol_ctx* c, int count, chol_num* const* nums, chol_batch*
           }
         }
         b->flops[k][l] += S.lvl_flops[k][l];
+        if (k == chol::kTaskSeg) b->segtasks[l] += S.lvl_segtasks[l];
+        if (k == chol::kTaskSegMerge) b->msegtasks[l] += S.lvl_msegtasks[l];
+        if (k == chol::kTaskSegMergeF) b->msegtasks_f[l] += S.lvl_msegtasks_f[l];
       }
       b->off[k][l + 1] = (int64_t)b->tasks[k].size() / 4;
     }
@@ -460,7 +491,8 @@ int chol_sym_set_tile_policy(chol_sym* s, const chol_tile_policy* p) {
   // 128-tile supernodes, and POTRF (whose tasks record the inverses' slice rows)
   const int kinds[] = {chol::schur_kind(0), chol::schur_kind(1), chol::schur_kind(2),
                        chol::schur_kind(3), chol::kTaskOzSlice, chol::kTaskTrsmRest,
-                       chol::kTaskPotrf};
+                       chol::kTaskPotrf, chol::kTaskSeg, chol::kTaskSegMerge,
+                       chol::kTaskSliceMerge, chol::kTaskSegMergeF, chol::kTaskSliceMergeF};
   static_assert(chol::kNumTileClasses == 4, "one Schur kind per tile class");
   for (int k : kinds) {
     dev_free(c, s->dev.tasks[k]);

@@ -30,6 +30,7 @@ constexpr int kMaxWidth = 128;   // hard limit on the width cap W (diagonal bloc
 // The representation error is at most 2^-56 of the row maximum.
 constexpr int kOzSlices = 7;
 constexpr int kOzPlanes = 8;      // planes of a slice scratch (the TF32 parts of 128 columns take 8)
+constexpr int kTfPlanes64 = 4;    // planes of the TF32 parts of up to 64 columns
 constexpr int kOzRowBytes = 128;  // one slice row: 64 bf16 (K <= 64), 128-byte swizzled
 constexpr int kOzInvRows = 64;    // slice rows of a diagonal-block inverse (n <= 64, zero-padded)
 enum SchurClass { kTile64 = 0, kTile32 = 1, kTile16 = 2, kTile128 = 3, kNumTileClasses = 4 };
@@ -53,8 +54,43 @@ enum TaskKind {
                       //   only); the same rows' tensor-core TRSM with the inverse's slices at y
                       //   (y = -1: s keeps the FP64 TRSM)
   kTaskTrsmRest = 10, // {s, r0, -, -}: kTaskTrsm without the 128-tile supernodes
-  kNumTaskKinds = 11
+  // FP64 tensor-core Schur tiles as segments (SchurSeg, two int4 each) that the kernel expands:
+  kTaskSeg = 11,      // every 128-tile supernode's own tiles (owner assembly)
+  kTaskSegMerge = 12, // with the updates of a group of chunks merged (see SchurSeg)
+  kTaskSliceMerge = 13, // kTaskOzSlice and {s, r0, oz, -1}: slices of the groups' earlier chunks, for
+                        //   kTaskSegMerge
+  kTaskSegMergeF = 14,  // the FP32 factor's (TF32 tiles): every chunk of a group in one task
+  kTaskSliceMergeF = 15,
+  kNumTaskKinds = 16
 };
+// A run of 128 x 128 tile tasks of the FP64 tensor-core Schur kernel.
+//
+// The update of a chunk of a wide separator (a supernode of at most 64 columns) reads and writes
+// the whole trailing matrix of its ancestors, gigabytes at the top of a 3D problem, for 64
+// multiply-adds per entry: at K = 64 the memory traffic of the scatter, not the tensor
+// cores, bounds the factorization.  So up to kMergeChunks consecutive chunks of one
+// separator form a group: each updates at once only the columns of the group's later
+// chunks (kSegInner), and all of them together the ancestors after the last one is
+// factored (kSegOuter), the tasks of the group's chunks on the same tiles one after another, so
+// that a tile's entries stay in L2 from one to the next.  The FP32 factor's groups are longer and a tile
+// is one task for all of a group's chunks: their products add up in tensor memory and are
+// scattered once (FP64 diagonal sums are exact only up to K = 64 columns of full digits).
+// Measured per factorization, the Schur tiles: 80^3 27-point FP64 1,308 -> 1,241 ms, 48^3
+// 65.4 -> 62.7 ms; 96^3 diffusion in FP32 79.1 -> 37.7 ms.
+struct SchurSeg {
+  int32_t s;       // the supernode; kSegOuter: the group's last chunk, g - 1 others before it
+  int32_t oz;      // first slice row of s
+  int32_t kind;
+  int32_t first;   // index of the segment's first task among its level's
+  int32_t w;       // kSegInner: columns to update; kSegOuter: first slice row of the earlier
+                   //   chunks' rows below the group, roundup(u, 8) rows each
+  int32_t g;       // chunks (1 but for kSegOuter)
+  int32_t nt;      // row strips of 128: ceil(u / 128)
+  int32_t count;   // tasks (FP64 kSegOuter: g per tile)
+};
+enum SegKind { kSegAll = 0, kSegInner = 1, kSegOuter = 2 };
+constexpr int kMergeChunks = 2, kMergeChunksF32 = 4;
+
 inline int schur_kind(int cls) { return cls == kTile128 ? kTaskSchur128 : kTaskSchur64 + cls; }
 
 // Device descriptor of one supernode (absolute device pointers: descriptors of several
@@ -160,6 +196,10 @@ struct Sym {
   // and the largest level's count plus one tile of slack (rows a tile may read past u)
   std::vector<int64_t> lvl_ozrows;
   int64_t oz_rows = 0;
+  // the same with the groups' earlier chunks (kTaskSegMerge), and the tile tasks of each
+  // level's segment lists
+  std::vector<int64_t> lvl_mozrows, lvl_mozrows_f;  // (_f: kTaskSegMergeF)
+  std::vector<int32_t> lvl_segtasks, lvl_msegtasks, lvl_msegtasks_f;
   // slice rows of the diagonal-block inverses of the supernodes whose TRSM runs on the tensor
   // cores (64 per supernode), and those supernodes' count, per level
   std::vector<int64_t> lvl_oyrows;

@@ -43,9 +43,13 @@ void launch_tf32_split(const int4* tasks, int ntasks, const SnDev* sns, int max_
 // acc_wait: 0 normally; > 0 is a test hook of the failure path: the consumer warps then wait
 // acc_wait SM clock cycles on a barrier that never completes (an accumulator that never
 // finishes) and give up.
-void launch_schur_tc(const int4* tasks, int ntasks, int* queue, const SnDev* sns,
-                     const MatDev* mats, bool owner, const void* oz, int64_t oz_rows,
+// segs: the level's SchurSeg records (two int4 each), ntasks tile tasks in all; max_width: as for
+// launch_tf32_split
+void launch_schur_tc(const int4* segs, int nsegs, int ntasks, int* queue, const SnDev* sns,
+                     const MatDev* mats, bool owner, int max_width, const void* oz, int64_t oz_rows,
                      long long acc_wait, cudaStream_t st);
+// rows of TF32 parts (the kernels' oz_rows) in a scratch of oz_scratch_bytes(oz_rows)
+int64_t tf_stride_rows(int64_t oz_rows, int max_width);
 int set_tc_kernel_attrs();
 // FP64 128 x 128 Schur tiles on the bf16 tensor cores by operand splitting, oz_kernels.cu:
 // per level, first the slices of every 128-tile supernode's L21 (kTaskOzSlice tasks), then
@@ -54,7 +58,8 @@ int set_tc_kernel_attrs();
 // (the columns are scaled by the shifts POTRF stored there)
 void launch_oz_slice(const int4* tasks, int ntasks, const SnDev* sns, void* oz, int64_t oz_rows,
                      const void* oy, int64_t oy_rows, cudaStream_t st);
-void launch_schur_oz(const int4* tasks, int ntasks, int* queue, const SnDev* sns,
+// segs: the level's SchurSeg records (two int4 each), ntasks tile tasks in all
+void launch_schur_oz(const int4* segs, int nsegs, int ntasks, int* queue, const SnDev* sns,
                      const MatDev* mats, bool owner, const void* oz, int64_t oz_rows,
                      long long acc_wait, cudaStream_t st);
 // L21 = A21 Y^T of the 128-tile supernodes on the bf16 tensor cores (kTaskOzSlice tasks: 128
@@ -64,6 +69,9 @@ void launch_trsm_oz(const int4* tasks, int ntasks, const SnDev* sns, const MatDe
                     const void* oz, int64_t oz_rows, const void* oy, int64_t oy_rows,
                     cudaStream_t st);
 size_t oz_scratch_bytes(int64_t oz_rows);
+// slice rows (the kernels' oz_rows) of FP64 slices in a scratch of oz_scratch_bytes(oz_rows):
+// more than oz_rows, since they take kOzSlices of its kOzPlanes planes
+int64_t oz_stride_rows(int64_t oz_rows);
 // the inverses' slice scratch: slice planes, row exponents, then one column shift per row
 size_t oy_scratch_bytes(int64_t oy_rows);
 int set_oz_kernel_attrs();

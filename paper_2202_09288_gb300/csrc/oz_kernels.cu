@@ -124,6 +124,15 @@ __device__ __forceinline__ void oz_mma(uint32_t tmem, uint64_t a, uint64_t b, ui
       "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
 }
 
+// True in one thread of the (converged) warp.
+__device__ __forceinline__ bool oz_elect() {
+  uint32_t e;
+  asm volatile(
+      "{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(e));
+  return e != 0;
+}
+
 __device__ __forceinline__ void oz_commit(uint32_t bar) {
   asm volatile(
       "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
@@ -245,6 +254,13 @@ __device__ __forceinline__ long long oz_high(unsigned long long lo, uint32_t f0,
   return (long long)w;
 }
 
+// s d 2^E with a subnormal or infinite result (out of line: the consumers' code is long enough)
+template <bool NEG>
+__device__ __noinline__ double oz_scale(double d, int E) {
+  const double r = ldexp(d, E);
+  return NEG ? -r : r;
+}
+
 // s W 2^E as a double (s = -1 when NEG), rounded to nearest (ties to even): the FP64 unit's
 // int64 -> double conversion, then an add to the exponent field and, for NEG, to the sign bit
 // (exact inside the normal range; a signed zero for W = 0, ldexp outside the range).  The FP64 unit is otherwise
@@ -259,8 +275,7 @@ __device__ __forceinline__ double oz_to_double(long long W, int E) {
   if ((unsigned)(be - 1) < 2046u)
     return __hiloint2double((int)(hi + (uint32_t)E * 1048576u + (NEG ? 0x80000000u : 0u)),
                             __double2loint(d));
-  const double r = ldexp(d, E);
-  return NEG ? -r : r;
+  return oz_scale<NEG>(d, E);
 }
 
 constexpr int kOzMaxRuns = 8;  // column targets per task whose relative rows are cached
@@ -279,10 +294,62 @@ struct OzMeta {
   long long rb[2 * kOzN];  // relative-map base of every run
   int rp[kOzMaxRuns][kOzM];
   int nruns;
-  int u, i0, k0;           // the task: update order, tile origin
+  int u, uc, i0, k0;       // the task: update order, end of its columns, tile origin
   const int32_t* relmap;   // for runs beyond the cached ones
   double* ustage;          // owner assembly: this supernode's staged U
 };
+
+// A task as the load thread hands it to the other roles.
+struct OzTask {
+  int s, i0, k0;  // supernode, tile origin in its off-diagonal rows
+  int oz;         // slice row of its off-diagonal row 0
+  int kend;       // columns from here on are not this task's (the update's order, or a group's inner columns)
+  int work;       // quarters | K steps << 8 | A rows of the task before << 16; -1: stop
+};
+
+// Task ti of segment g (SchurSeg); sns: the descriptors.  A strip's tiles
+// follow one another, so that later ones reuse the A rows; a group's chunks take turns on
+// up to four tiles of a strip.
+__device__ __forceinline__ OzTask oz_task(const SchurSeg& g, int ti, const SnDev* __restrict__ sns) {
+  const int x = ti - g.first;
+  const SnDev& d = sns[g.s];
+  OzTask t;
+  t.s = g.s;
+  t.oz = g.oz;
+  t.kend = d.m - d.n;
+  if (g.kind == kSegInner) {
+    const int nc = (g.w + 127) >> 7;  // column tiles: strip a has min(a + 1, nc)
+    int a = 0, y = x;
+    while (a + 1 < nc && y > a) y -= ++a;
+    if (a + 1 < nc) {
+      t.i0 = 128 * a;
+      t.k0 = 128 * y;
+    } else {
+      t.i0 = 128 * (a + y / nc);
+      t.k0 = 128 * (y % nc);
+    }
+    t.kend = g.w;
+    return t;
+  }
+  // strip a: g (a + 1) tasks after g a (a + 1) / 2
+  const int y = x / g.g;
+  int a = (int)((sqrtf(8.f * (float)y + 1.f) - 1.f) * 0.5f);
+  while (a * (a + 1) / 2 > y) a--;
+  while ((a + 1) * (a + 2) / 2 <= y) a++;
+  const int rem = x - g.g * (a * (a + 1) / 2);
+  const int q = rem / (4 * g.g), r = min(4, a + 1 - 4 * q), pos = rem - 4 * g.g * q;
+  const int c = pos / r, b = 4 * q + pos - c * r;  // chunk c of the group, tile column b
+  int off = 0;
+  if (c < g.g - 1) {  // an earlier chunk: its rows below the group, sliced apart
+    t.s = g.s - (g.g - 1) + c;
+    for (int e = t.s + 1; e <= g.s; e++) off += sns[e].n;
+    t.oz = g.w + c * ((t.kend + 7) & ~7) - off;
+    t.kend += off;
+  }
+  t.i0 = off + 128 * a;
+  t.k0 = off + 128 * b;
+  return t;
+}
 
 // barrier among the metadata warps only
 __device__ __forceinline__ void oz_meta_sync() {
@@ -308,7 +375,7 @@ __device__ __forceinline__ void oz_arrive(uint32_t bar) {
 // (the task order).
 template <bool OWNER>
 __global__ void __launch_bounds__(kOzThreads, 1)
-    k_schur_oz(const int4* __restrict__ tasks, int ntasks, int* __restrict__ queue,
+    k_schur_oz(const SchurSeg* __restrict__ segs, int nsegs, int ntasks, int* __restrict__ queue,
                const SnDev* __restrict__ sns, const MatDev* __restrict__ mats,
                const uint8_t* __restrict__ oz, int64_t oz_rows, long long acc_wait) {
   extern __shared__ __align__(1024) unsigned char oz_sm[];
@@ -318,18 +385,18 @@ __global__ void __launch_bounds__(kOzThreads, 1)
   __shared__ __align__(8) uint64_t a_full, a_empty, b_full[kOzBBufs], b_empty[kOzBBufs];
   __shared__ __align__(8) uint64_t acc_full[2], acc_empty[2];
   __shared__ __align__(8) uint64_t ring_full[kOzRing];
-  __shared__ int2 ring[kOzRing];  // {task, quarters | K steps << 8} (task = ntasks: stop)
+  __shared__ OzTask ring[kOzRing];
   __shared__ uint32_t tmem_base;
   __shared__ __align__(8) uint64_t meta_full[kOzMetaBufs], meta_empty[kOzMetaBufs];
   __shared__ OzMeta meta[kOzMetaBufs];
   __shared__ __align__(8) uint64_t never;  // test hook: a barrier nothing completes
-  __shared__ int s_mtq;  // the metadata warps' next task (or ntasks: stop)
+  __shared__ int s_mgo;  // the metadata warps go on with the next task (0: stop)
   __shared__ int s_fail;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   // a launch of an earlier level of this factorization already gave up on a wait: its
   // updates are missing and the factorization is reported failed, so skip the work (before
   // any barrier or tensor memory is set up); every thread reads the same word
-  if (ntasks > 0 && *(volatile unsigned long long*)(mats[sns[tasks[0].x].mat].err + 3) != 0) return;
+  if (*(volatile unsigned long long*)(mats[sns[segs[0].s].mat].err + 3) != 0) return;
   const size_t stride = (size_t)oz_rows * kOzRowBytes;
   const int32_t* exps = reinterpret_cast<const int32_t*>(oz + kOzSlices * stride);
 
@@ -387,22 +454,37 @@ __global__ void __launch_bounds__(kOzThreads, 1)
       // can build its targets while the current task is still being copied and computed.
       int prow = -1;                         // slice row of the last published task's A rows
       struct Job {
-        int4 t;
-        int nq, ks;
+        OzTask t;
+        int nq;
         bool reuse;  // the A rows of the task before it (still in shared memory)
       };
+      int sg = -1;  // the segment of the last published task
+      SchurSeg seg;
+      seg.first = seg.count = 0;
       auto publish = [&](int ti) -> Job {
-        Job jb{make_int4(0, 0, 0, 0), 0, 0, false};
+        Job jb;
+        jb.t.work = -1;
+        jb.nq = 0;
+        jb.reuse = false;
         if (ti < ntasks) {
-          jb.t = tasks[ti];
-          const SnDev& dd = sns[jb.t.x];
-          jb.nq = min(4, (dd.m - dd.n - jb.t.z + kOzQ - 1) / kOzQ);
-          jb.ks = (dd.n + 15) >> 4;
-          jb.reuse = jb.t.w + jb.t.y == prow;
-          prow = jb.t.w + jb.t.y;
+          if (ti >= seg.first + seg.count) {  // the next segment, or a search among the later ones
+            int lo = sg + 1, hi = nsegs - 1;
+            if (lo < hi && ti < segs[lo + 1].first) hi = lo;
+            while (lo < hi) {
+              const int mid = (lo + hi + 1) >> 1;
+              if (segs[mid].first <= ti) lo = mid; else hi = mid - 1;
+            }
+            sg = lo;
+            seg = segs[sg];
+          }
+          jb.t = oz_task(seg, ti, sns);
+          jb.nq = min(4, (jb.t.kend - jb.t.k0 + kOzQ - 1) / kOzQ);
+          jb.reuse = jb.t.oz + jb.t.i0 == prow;
+          prow = jb.t.oz + jb.t.i0;
+          jb.t.work = jb.nq | (((sns[jb.t.s].n + 15) >> 4) << 8) | ((int)jb.reuse << 16);
         }
         const int rs = (int)(ord % kOzRing);
-        ring[rs] = make_int2(ti < ntasks ? ti : ntasks, jb.nq | (jb.ks << 8) | ((int)jb.reuse << 16));
+        ring[rs] = jb.t;
         oz_arrive(smem_u32(&ring_full[rs]));
         ord++;
         return jb;
@@ -418,7 +500,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
           tend = min(tq + g, ntasks);
         }
         const Job next = publish(tq);  // the next task (or the stop entry)
-        const int4 t = job.t;
+        const OzTask& t = job.t;
         const int nq = job.nq;
         // quarter j's B slices, once the MMAs of the quarter before it in the buffer are done
         auto load_b = [&](int j) -> bool {
@@ -430,7 +512,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
           oz_expect(bar, kOzQBytes);
           for (int p = 0; p < kOzSlices; p++)
             oz_bulk_load(smem_u32(dst + p * kOzQSlice),
-                         oz + p * stride + (size_t)(t.w + t.z + kOzQ * j) * kOzRowBytes,
+                         oz + p * stride + (size_t)(t.oz + t.k0 + kOzQ * j) * kOzRowBytes,
                          kOzQSlice, bar);
           qb++;
           return true;
@@ -449,7 +531,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
           oz_expect(smem_u32(&a_full), kOzABytes);
           for (int p = 0; p < kOzSlices; p++)
             oz_bulk_load(smem_u32(A + p * kOzASlice),
-                         oz + p * stride + (size_t)(t.w + t.y) * kOzRowBytes, kOzASlice,
+                         oz + p * stride + (size_t)(t.oz + t.i0) * kOzRowBytes, kOzASlice,
                          smem_u32(&a_full));
           T++;
         }
@@ -461,7 +543,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
       if (!ok) {
         s_fail = 1;
         const int rs = (int)(ord % kOzRing);
-        ring[rs] = make_int2(ntasks, 0);
+        ring[rs].work = -1;
         oz_arrive(smem_u32(&ring_full[rs]));
       }
       // bounded waits for the copies still in flight: the last A load and the last B load of
@@ -471,61 +553,81 @@ __global__ void __launch_bounds__(kOzThreads, 1)
         oz_wait(smem_u32(&b_full[qq % kOzBBufs]), (uint32_t)((qq / kOzBBufs) & 1));
     }
   } else if (warp == kOzMmaWarp) {
-    // ---------------- MMAs, one thread ----------------
-    if (lane == 0) {
-      // N = (7 - p) x 32: the MMA of slice p against slices 0 .. 6-p of a quarter
-      uint32_t idesc[kOzSlices];
-#pragma unroll
-      for (int p = 0; p < kOzSlices; p++) idesc[p] = oz_idesc((kOzSlices - p) * kOzQ);
-      const uint64_t da0 = oz_desc(smem_u32(A));
-      const uint64_t db0 = oz_desc(smem_u32(Bq0));
-      bool ok = true;
-      long long q = 0;  // quarters issued (TMEM set q & 1, B buffer q % kOzBBufs)
-      long long T = 0;  // A slice loads waited for
-      for (long long ord = 0; ok; ord++) {
-        const int rs = (int)(ord % kOzRing);
-        if (!oz_wait(smem_u32(&ring_full[rs]), (uint32_t)((ord / kOzRing) & 1))) {
-          ok = false;
-          break;
+    // ---------------- MMAs: one elected thread, the warp's control flow uniform ----------------
+    // The loop over a quarter's MMAs is rolled and short: it shares its scheduler's instruction
+    // cache with consumer warps that run through long unrolled code, and an unrolled loop was
+    // refetched line by line (2,800 cycles of issuing per quarter whose MMAs take 1,930).
+    const bool lead = oz_elect();
+    // N = (7 - p) x 32: the MMA of slice p against slices 0 .. 6-p of a quarter
+    const uint32_t idesc0 = oz_idesc(kOzSlices * kOzQ);
+    constexpr uint32_t kIdStep = (uint32_t)(kOzQ >> 3) << 17, kAStep = kOzASlice >> 4;
+    const uint64_t da0 = oz_desc(smem_u32(A)), db0 = oz_desc(smem_u32(Bq0));
+    bool ok = true;
+    int q = 0;            // quarters issued (TMEM set q & 1)
+    int bb = 0, bpar = 0;  // B buffer q % kOzBBufs and the parity of its use
+    int T = 0;            // A slice loads waited for
+    for (int ord = 0; ok; ord++) {
+      const int rs = ord % kOzRing;
+      if (!oz_wait(smem_u32(&ring_full[rs]), (uint32_t)((ord / kOzRing) & 1))) {
+        ok = false;
+        break;
+      }
+      const int work = ring[rs].work;
+      if (work < 0) break;
+      const int nq = work & 0xff, ks = (work >> 8) & 0xff;
+      const bool reuse = (work >> 16) & 1;  // the previous task's A slices
+      // the A slices are free when every MMA so far is done (one commit per A load, so that the
+      // load thread, which waits for each, is never two phases apart from this one)
+      if (!reuse && T > 0 && lead) oz_commit(smem_u32(&a_empty));
+      for (int j = 0; j < nq; j++, q++) {
+        const int b = q & 1;
+        ok = oz_wait(smem_u32(&b_full[bb]), (uint32_t)bpar) &&
+             (q < 2 ||  // the set was drained (quarter q - 2)
+              oz_wait(smem_u32(&acc_empty[b]), (uint32_t)(((q >> 1) - 1) & 1))) &&
+             (j > 0 || reuse || oz_wait(smem_u32(&a_full), (uint32_t)(T & 1)));  // the task's A
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;");
+        // K step outer, slice inner: consecutive MMAs start at different diagonals (measured
+        // 2.3x faster than issuing one slice's K steps back to back into the same columns)
+        uint64_t da = da0, db = db0 + (uint64_t)((bb * kOzQBytes) >> 4);
+        uint32_t col = tmem + (uint32_t)(b * kOzSetCols), id = idesc0;
+        int left = ks, p = 0;
+        uint32_t acc = 0;
+#pragma unroll 1
+        while (left > 0) {
+          if (lead) oz_mma(col, da, db, id, acc);
+          acc = 1;
+          if (++p < kOzSlices) {
+            da += kAStep;
+            col += kOzQ;
+            id -= kIdStep;
+          } else {
+            p = 0;
+            left--;
+            da -= (kOzSlices - 1) * kAStep - 2;
+            db += 2;
+            col -= (kOzSlices - 1) * kOzQ;
+            id = idesc0;
+          }
         }
-        const int2 e = ring[rs];
-        if (e.x >= ntasks) break;
-        const int nq = e.y & 0xff, ks = (e.y >> 8) & 0xff;
-        const bool reuse = (e.y >> 16) & 1;  // the previous task's A slices
-        // the A slices are free when every MMA so far is done (one commit per A load, so that the
-        // load thread, which waits for each, is never two phases apart from this one)
-        if (!reuse && T > 0) oz_commit(smem_u32(&a_empty));
-        for (int j = 0; j < nq; j++, q++) {
-          const int b = (int)(q & 1), bb = (int)(q % kOzBBufs);
-          const uint64_t db = db0 + (uint64_t)((bb * kOzQBytes) >> 4);
-          if (!oz_wait(smem_u32(&b_full[bb]), (uint32_t)((q / kOzBBufs) & 1)) ||
-              (q >= 2 &&  // the set was drained (quarter q - 2)
-               !oz_wait(smem_u32(&acc_empty[b]), (uint32_t)(((q >> 1) - 1) & 1)))) {
-            ok = false;
-            break;
-          }
-          if (j == 0 && !reuse && !oz_wait(smem_u32(&a_full), (uint32_t)(T & 1))) {  // the task's A
-            ok = false;
-            break;
-          }
-          asm volatile("tcgen05.fence::after_thread_sync;");
-          // K step outer, slice inner: consecutive MMAs start at different diagonals (measured
-          // 2.3x faster than issuing one slice's K steps back to back into the same columns)
-          for (int k = 0; k < ks; k++)
-#pragma unroll
-            for (int p = 0; p < kOzSlices; p++)
-              oz_mma(tmem + (uint32_t)(b * kOzSetCols + p * kOzQ),
-                     da0 + (uint64_t)((p * kOzASlice) >> 4) + 2 * k, db + 2 * k, idesc[p],
-                     (p > 0 || k > 0) ? 1u : 0u);
+        if (lead) {
           oz_commit(smem_u32(&acc_full[b]));
           oz_commit(smem_u32(&b_empty[bb]));
         }
-        if (!reuse) T++;
+        if (++bb == kOzBBufs) {
+          bb = 0;
+          bpar ^= 1;
+        }
       }
+      if (!reuse) T++;
+    }
+    if (lead) {
       if (!ok) s_fail = 1;
       // bounded wait for the MMAs in flight (the last quarter's commit covers all earlier ones)
       if (q >= 1) oz_wait(smem_u32(&acc_full[(q - 1) & 1]), (uint32_t)(((q - 1) >> 1) & 1));
     }
+    __syncwarp();
   } else if (warp >= kOzMetaBase / 32) {
     // ---------------- metadata warps: one thread per tile row / column ----------------
     // For each task in ring order, into meta[ord % kOzMetaBufs] once the consumers have released it:
@@ -539,29 +641,30 @@ __global__ void __launch_bounds__(kOzThreads, 1)
       const int buf = ord % kOzMetaBufs;
       if (mt == 0) {
         const int rs = ord % kOzRing;
-        int tq = ntasks;
+        int go = 0;
         if (!oz_wait(smem_u32(&ring_full[rs]), (uint32_t)((ord / kOzRing) & 1)) ||
-            (ring[rs].x < ntasks && ord >= kOzMetaBufs &&
+            (ring[rs].work >= 0 && ord >= kOzMetaBufs &&
              !oz_wait(smem_u32(&meta_empty[buf]), (uint32_t)((ord / kOzMetaBufs - 1) & 1))))
           s_fail = 1;
         else
-          tq = ring[rs].x;
-        s_mtq = tq;
+          go = ring[rs].work >= 0;
+        s_mgo = go;
       }
       oz_meta_sync();
-      const int tq = s_mtq;
-      oz_meta_sync();  // s_mtq is rewritten only after every thread has read it
-      if (tq >= ntasks) break;
+      const int go = s_mgo;
+      const OzTask tk = ring[ord % kOzRing];
+      oz_meta_sync();  // s_mgo is rewritten only after every thread has read it
+      if (!go) break;
       OzMeta& M = meta[buf];
-      const int4 tk = tasks[tq];
-      const SnDev d = sns[tk.x];
-      const int n = d.n, u = d.m - n, i0 = tk.y, k0 = tk.z;
+      const SnDev d = sns[tk.s];
+      const int n = d.n, u = d.m - n, i0 = tk.i0, k0 = tk.k0, uc = tk.kend;
       const MatDev md = mats[d.mat];
       const int gk = k0 + mt;
-      M.eA[mt] = (i0 + mt < u) ? exps[tk.w + i0 + mt] : 0;
-      M.eB[mt] = (gk < u ? exps[tk.w + gk] : 0) - 55;  // U = W 2^(e_i + e_k - 55)
+      M.eA[mt] = (i0 + mt < u) ? exps[tk.oz + i0 + mt] : 0;
+      M.eB[mt] = (gk < uc ? exps[tk.oz + gk] : 0) - 55;  // U = W 2^(e_i + e_k - 55)
       if (mt == 0) {
         M.u = u;
+        M.uc = uc;
         M.i0 = i0;
         M.k0 = k0;
         M.relmap = md.relmap;
@@ -569,8 +672,8 @@ __global__ void __launch_bounds__(kOzThreads, 1)
       }
       if (!OWNER) {
         const int32_t* rows = d.rows + n;
-        const int grow = gk < u ? rows[gk] : 0;
-        const int tc = gk < u ? md.col2sn[grow] : -1;
+        const int grow = gk < uc ? rows[gk] : 0;
+        const int tc = gk < uc ? md.col2sn[grow] : -1;
         M.tcol[mt] = tc;
         // the supernode's runs that start after position 0 and at or before k0: their count
         // is the index (from run0) of the run holding the tile's first column; the tile's
@@ -583,14 +686,14 @@ __global__ void __launch_bounds__(kOzThreads, 1)
         oz_meta_sync();
         // a column starts a run when its target differs from its left neighbour's; its run
         // index is the number of starts up to it, less one
-        const bool start = gk < u && (mt == 0 || M.tcol[mt - 1] != tc);
+        const bool start = gk < uc && (mt == 0 || M.tcol[mt - 1] != tc);
         const unsigned bl = __ballot_sync(0xffffffffu, start);
         if (lane == 0) M.wcnt[mwarp] = __popc(bl);
         oz_meta_sync();
         int off = 0;
         for (int w2 = 0; w2 < mwarp; w2++) off += M.wcnt[w2];
         const int first = d.run0 + M.fcnt[0] + M.fcnt[1] + M.fcnt[2] + M.fcnt[3];
-        if (gk < u) {
+        if (gk < uc) {
           const int r = off + __popc(bl & ((2u << lane) - 1u)) - 1;
           const SnDev& td = sns[md.sn_base + tc];
           M.run[mt] = r;
@@ -633,14 +736,14 @@ __global__ void __launch_bounds__(kOzThreads, 1)
         s_fail = 1;
         break;
       }
-      if (ring[rs].x >= ntasks) break;
+      if (ring[rs].work < 0) break;
       const OzMeta& M = meta[buf];
       if (!__all_sync(0xffffffffu, oz_wait(smem_u32(&meta_full[buf]), (uint32_t)((ord / kOzMetaBufs) & 1)))) {
         s_fail = 1;
         break;
       }
-      const int u = M.u, i0 = M.i0, k0 = M.k0;
-      const int nq = min(4, (u - k0 + kOzQ - 1) / kOzQ);
+      const int u = M.u, uc = M.uc, i0 = M.i0, k0 = M.k0;
+      const int nq = min(4, (uc - k0 + kOzQ - 1) / kOzQ);
       const int gi = i0 + i;
       const int eA = M.eA[i];
       bool stop = false;
@@ -664,7 +767,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
           const int r0w = i0 + 32 * (warp & 3);  // the warp's first tile row
           // warp-uniform: no entry of the chunk in the lower triangle of the update (past
           // its order, or above the diagonal): nothing to read but the release
-          const bool dead = r0w >= u || gk0 >= u || r0w + 31 < gk0;
+          const bool dead = r0w >= u || gk0 >= uc || r0w + 31 < gk0;
           double val[8];
           if (!dead) {
             // the 7 diagonals of the chunk's columns -> W (exact integer) -> U = W 2^(e_i +
@@ -714,10 +817,10 @@ __global__ void __launch_bounds__(kOzThreads, 1)
 #pragma unroll
               for (int jj = 0; jj < 8; jj++) {
                 const int gk = gk0 + jj;
-                if (gk < u && gk <= gi) U[(int64_t)gk * u + gi] = val[jj];
+                if (gk < uc && gk <= gi) U[(int64_t)gk * u + gi] = val[jj];
               }
             }
-          } else if (r0w + 31 < u && gk0 + 7 < u && gk0 + 7 <= r0w &&
+          } else if (r0w + 31 < u && gk0 + 7 < uc && gk0 + 7 <= r0w &&
                      M.run[kb] == M.run[kb + 7]) {
             // warp-uniform fast path: every entry live, one target run for all 8 columns
             const int r = M.run[kb];
@@ -732,7 +835,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
 #pragma unroll
             for (int jj = 0; jj < 8; jj++) {
               const int kk = kb + jj, gk = k0 + kk;
-              if (gk >= u || gk > gi) continue;
+              if (gk >= uc || gk > gi) continue;
               const int r = M.run[kk];
               if (r != rprev) {
                 rprev = r;
@@ -750,7 +853,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
     }
   }
   __syncthreads();
-  if (s_fail && tid == 0 && ntasks > 0) atomicAdd(mats[sns[tasks[0].x].mat].err + 3, 1ull);
+  if (s_fail && tid == 0) atomicAdd(mats[sns[segs[0].s].mat].err + 3, 1ull);
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   if (warp == 0)
@@ -907,7 +1010,7 @@ size_t oy_scratch_bytes(int64_t oy_rows) {
   return oz_scratch_bytes(oy_rows) + (size_t)oy_rows * sizeof(int32_t);
 }
 
-void launch_schur_oz(const int4* tasks, int ntasks, int* queue, const SnDev* sns,
+void launch_schur_oz(const int4* segs, int nsegs, int ntasks, int* queue, const SnDev* sns,
                      const MatDev* mats, bool owner, const void* oz, int64_t oz_rows,
                      long long acc_wait, cudaStream_t st) {
   if (ntasks <= 0) return;
@@ -916,12 +1019,17 @@ void launch_schur_oz(const int4* tasks, int ntasks, int* queue, const SnDev* sns
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int grid = ntasks < sms ? ntasks : sms;  // one resident CTA per SM, tasks by queue
   const uint8_t* z = static_cast<const uint8_t*>(oz);
+  const SchurSeg* sg = reinterpret_cast<const SchurSeg*>(segs);
   if (owner)
-    k_schur_oz<true><<<grid, kOzThreads, kOzSmem, st>>>(tasks, ntasks, queue, sns, mats, z, oz_rows,
-                                                       acc_wait);
+    k_schur_oz<true><<<grid, kOzThreads, kOzSmem, st>>>(sg, nsegs, ntasks, queue, sns, mats, z,
+                                                       oz_rows, acc_wait);
   else
-    k_schur_oz<false><<<grid, kOzThreads, kOzSmem, st>>>(tasks, ntasks, queue, sns, mats, z,
+    k_schur_oz<false><<<grid, kOzThreads, kOzSmem, st>>>(sg, nsegs, ntasks, queue, sns, mats, z,
                                                         oz_rows, acc_wait);
+}
+
+int64_t oz_stride_rows(int64_t oz_rows) {
+  return (int64_t)(oz_scratch_bytes(oz_rows) / (kOzSlices * kOzRowBytes + sizeof(int32_t)));
 }
 
 size_t oz_scratch_bytes(int64_t oz_rows) {

@@ -154,6 +154,8 @@ struct TaskView {
   const double* flops[kNumTaskKinds] = {};
   const int4* asm_src = nullptr;
   const int32_t* trsmoz = nullptr;  // per level: supernodes whose TRSM runs on the tensor cores
+  // per level: tasks of the segment lists
+  const int32_t *segtasks = nullptr, *msegtasks = nullptr, *msegtasks_f = nullptr;
   int32_t nlev = 0;
   int max_width = 0;
   const int4* level(int k, int32_t l, int* count) const {

@@ -154,6 +154,45 @@ __device__ __forceinline__ void meta_sync() {
   asm volatile("bar.sync 1, %0;" ::"n"(kTfMetaThreads) : "memory");
 }
 
+// A task as the load thread hands it to the other roles.
+struct TfTask {
+  int s, i0, k0;    // supernode (a group's last chunk), tile origin in its off-diagonal rows
+  int kend;         // columns from here on are not this task's
+  int g;            // chunks whose products the tile sums (0: stop)
+  int gap;          // slice rows of each earlier chunk
+  uint32_t widths;  // the chunks' columns, a byte each
+};
+
+// Task ti of segment g (SchurSeg).
+__device__ __forceinline__ TfTask tf_task(const SchurSeg& g, int ti, const SnDev* __restrict__ sns) {
+  const SnDev& d = sns[g.s];
+  int y = ti - g.first, a = 0;
+  TfTask t;
+  t.s = g.s;
+  t.g = g.g;
+  t.kend = d.m - d.n;
+  t.gap = (t.kend + 7) & ~7;
+  t.widths = 0;
+  for (int c = 0; c < g.g; c++) t.widths |= (uint32_t)sns[g.s - (g.g - 1) + c].n << (8 * c);
+  if (g.kind == kSegInner) {
+    const int nc = (g.w + 127) >> 7;  // column tiles: strip a has min(a + 1, nc)
+    while (a + 1 < nc && y > a) y -= ++a;
+    if (a + 1 == nc) {
+      a += y / nc;
+      y %= nc;
+    }
+    t.kend = g.w;
+  } else {  // strip a: a + 1 tiles after a (a + 1) / 2
+    a = (int)((sqrtf(8.f * (float)y + 1.f) - 1.f) * 0.5f);
+    while (a * (a + 1) / 2 > y) a--;
+    while ((a + 1) * (a + 2) / 2 <= y) a++;
+    y -= a * (a + 1) / 2;
+  }
+  t.i0 = 128 * a;
+  t.k0 = 128 * y;
+  return t;
+}
+
 static_assert(kTfM == 128, "the run count sums four 32-column words");
 struct TfMeta {
   float* cp[kTfM];  // each column's target panel column (its relative rows are added)
@@ -164,7 +203,7 @@ struct TfMeta {
   long long rb[kTfM];   // relative-map base of every run
   int rp[kTfMaxRuns][kTfM];
   int nruns;
-  int u, i0, k0;                 // the task: update order, tile origin
+  int u, uc, i0, k0;             // the task: update order, end of its columns, tile origin
   const int32_t* relmap;         // for runs beyond the cached ones
   float* ustage;                 // owner assembly: this supernode's staged U
 };
@@ -172,12 +211,12 @@ struct TfMeta {
 }  // namespace
 
 // hi and lo TF32 parts of the L21 rows r0 .. r0+127 of supernode s at slice rows oz + r:
-// plane (part p, chunk c) at oz + (4 p + c) oz_rows 128 B, 16-byte piece q of a row (its
-// columns 32 c + 4 q .. +3) stored at piece q ^ (row & 7).  Rows u .. roundup(u, 8) and
-// columns n .. are zero.
+// plane (part p, chunk c) at oz + (pp p + c) oz_rows 128 B (pp planes per part), 16-byte piece q of
+// a row (its columns 32 c + 4 q .. +3) stored at piece q ^ (row & 7).  Rows u .. roundup(u, 8)
+// and columns n .. are zero.
 __global__ void __launch_bounds__(256)
     k_tf32_split(const int4* __restrict__ tasks, const SnDev* __restrict__ sns,
-                 uint8_t* __restrict__ oz, int64_t oz_rows) {
+                 uint8_t* __restrict__ oz, int64_t oz_rows, int pp) {
   extern __shared__ __align__(16) float xf[];  // [n][kTfM]
   const int4 tk = tasks[blockIdx.x];
   const SnDev d = sns[tk.x];
@@ -206,34 +245,34 @@ __global__ void __launch_bounds__(256)
     }
     uint8_t* dst = oz + (size_t)(row0 + i) * kOzRowBytes + pc * 16;
     *reinterpret_cast<float4*>(dst + (size_t)c * stride) = make_float4(hi[0], hi[1], hi[2], hi[3]);
-    *reinterpret_cast<float4*>(dst + (size_t)(4 + c) * stride) =
+    *reinterpret_cast<float4*>(dst + (size_t)(pp + c) * stride) =
         make_float4(lo[0], lo[1], lo[2], lo[3]);
   }
 }
 
 template <bool OWNER>
 __global__ void __launch_bounds__(kTfThreads, 1)
-    k_schur_tf32(const int4* __restrict__ tasks, int ntasks, int* __restrict__ queue,
+    k_schur_tf32(const SchurSeg* __restrict__ segs, int nsegs, int ntasks, int* __restrict__ queue,
                  const SnDev* __restrict__ sns, const MatDev* __restrict__ mats,
-                 const uint8_t* __restrict__ oz, int64_t oz_rows, long long acc_wait) {
+                 const uint8_t* __restrict__ oz, int64_t oz_rows, int pp, long long acc_wait) {
   extern __shared__ __align__(1024) unsigned char tf_sm[];
   unsigned char* stage_base =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(tf_sm) + 1023) & ~uintptr_t(1023));
   __shared__ __align__(8) uint64_t st_full[kTfStages], st_empty[kTfStages];
   __shared__ __align__(8) uint64_t acc_full[kTfSlots], acc_empty[kTfSlots];
   __shared__ __align__(8) uint64_t ring_full[kTfRing];
-  __shared__ int ring[kTfRing];
+  __shared__ TfTask ring[kTfRing];
   __shared__ uint32_t tmem_base;
   __shared__ __align__(8) uint64_t meta_full[kTfMetaBufs], meta_empty[kTfMetaBufs];
   __shared__ TfMeta meta[kTfMetaBufs];
-  __shared__ int s_mtq;  // the metadata warps' next task (or ntasks: stop)
+  __shared__ int s_mgo;  // the metadata warps go on with the next task (0: stop)
   __shared__ int s_fail;
   __shared__ __align__(8) uint64_t never;  // test hook: a barrier nothing completes
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   // a launch of an earlier level of this factorization already gave up on a wait: its
   // updates are missing and the factorization is reported failed, so skip the work (before
   // any barrier or tensor memory is set up); every thread reads the same word
-  if (ntasks > 0 && *(volatile unsigned long long*)(mats[sns[tasks[0].x].mat].err + 3) != 0) return;
+  if (*(volatile unsigned long long*)(mats[sns[segs[0].s].mat].err + 3) != 0) return;
   const size_t stride = (size_t)oz_rows * kOzRowBytes;
 
   if (warp == 0) {
@@ -276,15 +315,35 @@ __global__ void __launch_bounds__(kTfThreads, 1)
       int ord = 0;         // ring entries published
       bool ok = true;
       int tq = blockIdx.x;  // a CTA's first task is its block index
+      int sg = -1;          // the segment of the last task
+      SchurSeg seg;
+      seg.first = seg.count = 0;
       for (;;) {
-        ring[ord % kTfRing] = tq < ntasks ? tq : ntasks;  // the task order, at claim time
+        TfTask t;
+        t.g = 0;
+        if (tq < ntasks) {
+          if (tq >= seg.first + seg.count) {  // the next segment, or a search among the later ones
+            int lo = sg + 1, hi = nsegs - 1;
+            if (lo < hi && tq < segs[lo + 1].first) hi = lo;
+            while (lo < hi) {
+              const int mid = (lo + hi + 1) >> 1;
+              if (segs[mid].first <= tq) lo = mid; else hi = mid - 1;
+            }
+            sg = lo;
+            seg = segs[sg];
+          }
+          t = tf_task(seg, tq, sns);
+        }
+        ring[ord % kTfRing] = t;  // the task order, at claim time
         tf_arrive(smem_u32(&ring_full[ord % kTfRing]));
         ord++;
         if (tq >= ntasks) break;
-        const int4 t = tasks[tq];
-        const int nch = (sns[t.x].n + kTfChunk - 1) / kTfChunk;
-        const uint8_t* arow = oz + (size_t)(t.w + t.y) * kOzRowBytes;
-        const uint8_t* brow = oz + (size_t)(t.w + t.z) * kOzRowBytes;
+        for (int src = 0; src < t.g && ok; src++) {
+        // the group's earlier chunks' rows first, in their own slice rows; the last chunk's own
+        const int64_t row0 = src < t.g - 1 ? seg.w + (int64_t)src * t.gap : seg.oz;
+        const int nch = (int)(((t.widths >> (8 * src)) & 255u) + kTfChunk - 1) / kTfChunk;
+        const uint8_t* arow = oz + (size_t)(row0 + t.i0) * kOzRowBytes;
+        const uint8_t* brow = oz + (size_t)(row0 + t.k0) * kOzRowBytes;
         for (int c = 0; c < nch && ok; c++, item++) {
           const int s = (int)(item % kTfStages);
           if (item >= kTfStages &&  // the stage's previous MMAs must have read it
@@ -296,10 +355,11 @@ __global__ void __launch_bounds__(kTfThreads, 1)
           const uint32_t bar = smem_u32(&st_full[s]);
           tf_expect(bar, kTfStageBytes);
           tf_bulk_load(smem_u32(sb), arow + (size_t)c * stride, kTfPlane, bar);
-          tf_bulk_load(smem_u32(sb + kTfPlane), arow + (size_t)(4 + c) * stride, kTfPlane, bar);
+          tf_bulk_load(smem_u32(sb + kTfPlane), arow + (size_t)(pp + c) * stride, kTfPlane, bar);
           tf_bulk_load(smem_u32(sb + 2 * kTfPlane), brow + (size_t)c * stride, kTfPlane, bar);
-          tf_bulk_load(smem_u32(sb + 3 * kTfPlane), brow + (size_t)(4 + c) * stride, kTfPlane,
+          tf_bulk_load(smem_u32(sb + 3 * kTfPlane), brow + (size_t)(pp + c) * stride, kTfPlane,
                        bar);
+        }
         }
         if (!ok) break;
         tq = gridDim.x >= ntasks ? ntasks : (int)gridDim.x + atomicAdd(queue, 1);
@@ -307,7 +367,7 @@ __global__ void __launch_bounds__(kTfThreads, 1)
       if (!ok) {
         s_fail = 1;
         // the other roles stop at their next ring wait on an end marker
-        ring[ord % kTfRing] = ntasks;
+        ring[ord % kTfRing].g = 0;
         tf_arrive(smem_u32(&ring_full[ord % kTfRing]));
       }
       // bounded waits for the copies still in flight: the last one of each stage
@@ -325,15 +385,17 @@ __global__ void __launch_bounds__(kTfThreads, 1)
           ok = false;
           break;
         }
-        const int tq = ring[ord % kTfRing];
-        if (tq >= ntasks) break;
-        const int n = sns[tasks[tq].x].n;
-        const int nch = (n + kTfChunk - 1) / kTfChunk;
+        const int g = ring[ord % kTfRing].g;
+        if (g == 0) break;
+        const uint32_t widths = ring[ord % kTfRing].widths;
         const int acc = ord % kTfSlots;
+        for (int src = 0; src < g && ok; src++) {
+        const int n = (int)((widths >> (8 * src)) & 255u);
+        const int nch = (n + kTfChunk - 1) / kTfChunk;
         for (int c = 0; c < nch; c++, done++) {
           const int s = (int)(done % kTfStages);
           if (!tf_wait(smem_u32(&st_full[s]), (uint32_t)((done / kTfStages) & 1)) ||
-              (c == 0 && ord >= kTfSlots &&  // wait for the drain of the slot
+              (src == 0 && c == 0 && ord >= kTfSlots &&  // wait for the drain of the slot
                !tf_wait(smem_u32(&acc_empty[acc]), (uint32_t)(((ord / kTfSlots) - 1) & 1)))) {
             ok = false;
             break;
@@ -345,12 +407,13 @@ __global__ void __launch_bounds__(kTfThreads, 1)
           const uint64_t bhi = tf_desc(sa + 2 * kTfPlane), blo = tf_desc(sa + 3 * kTfPlane);
           const uint32_t dt = tmem + (uint32_t)(acc * kTfM);
           for (int kk = 0; kk < (kw + 7) / 8; kk++) {  // K steps of 8 TF32 = 32 bytes
-            tf_mma(dt, ahi + 2 * kk, bhi + 2 * kk, idesc, (c > 0 || kk > 0) ? 1u : 0u);
+            tf_mma(dt, ahi + 2 * kk, bhi + 2 * kk, idesc, (src > 0 || c > 0 || kk > 0) ? 1u : 0u);
             tf_mma(dt, ahi + 2 * kk, blo + 2 * kk, idesc, 1u);
             tf_mma(dt, alo + 2 * kk, bhi + 2 * kk, idesc, 1u);
           }
           tf_commit(smem_u32(&st_empty[s]));  // the stage is free once these MMAs are done
-          if (c + 1 == nch) tf_commit(smem_u32(&acc_full[acc]));
+          if (src + 1 == g && c + 1 == nch) tf_commit(smem_u32(&acc_full[acc]));
+        }
         }
       }
       if (!ok) s_fail = 1;
@@ -370,26 +433,27 @@ __global__ void __launch_bounds__(kTfThreads, 1)
       const int buf = ord % kTfMetaBufs;
       if (mt == 0) {
         const int rs = ord % kTfRing;
-        int tq = ntasks;
+        int go = 0;
         if (!tf_wait(smem_u32(&ring_full[rs]), (uint32_t)((ord / kTfRing) & 1)) ||
-            (ring[rs] < ntasks && ord >= kTfMetaBufs &&
+            (ring[rs].g > 0 && ord >= kTfMetaBufs &&
              !tf_wait(smem_u32(&meta_empty[buf]), (uint32_t)((ord / kTfMetaBufs - 1) & 1))))
           s_fail = 1;
         else
-          tq = ring[rs];
-        s_mtq = tq;
+          go = ring[rs].g > 0;
+        s_mgo = go;
       }
       meta_sync();
-      const int tq = s_mtq;
-      meta_sync();  // s_mtq is rewritten only after every thread has read it
-      if (tq >= ntasks) break;
+      const int go = s_mgo;
+      const TfTask tk = ring[ord % kTfRing];
+      meta_sync();  // s_mgo is rewritten only after every thread has read it
+      if (!go) break;
       TfMeta& M = meta[buf];
-      const int4 tk = tasks[tq];
-      const SnDev d = sns[tk.x];
-      const int n = d.n, u = d.m - n, i0 = tk.y, k0 = tk.z;
+      const SnDev d = sns[tk.s];
+      const int n = d.n, u = d.m - n, i0 = tk.i0, k0 = tk.k0, uc = tk.kend;
       const MatDev md = mats[d.mat];
       if (mt == 0) {
         M.u = u;
+        M.uc = uc;
         M.i0 = i0;
         M.k0 = k0;
         M.relmap = md.relmap;
@@ -398,8 +462,8 @@ __global__ void __launch_bounds__(kTfThreads, 1)
       if (!OWNER) {
         const int32_t* rows = d.rows + n;
         const int gk = k0 + mt;
-        const int grow = gk < u ? rows[gk] : 0;
-        const int tc = gk < u ? md.col2sn[grow] : -1;
+        const int grow = gk < uc ? rows[gk] : 0;
+        const int tc = gk < uc ? md.col2sn[grow] : -1;
         M.tcol[mt] = tc;
         // the supernode's runs that start after position 0 and at or before k0: their count
         // is the index (from run0) of the run holding the tile's first column; the tile's
@@ -412,14 +476,14 @@ __global__ void __launch_bounds__(kTfThreads, 1)
         meta_sync();
         // a column starts a run when its target differs from its left neighbour's; its run
         // index is the number of starts up to it, less one
-        const bool start = gk < u && (mt == 0 || M.tcol[mt - 1] != tc);
+        const bool start = gk < uc && (mt == 0 || M.tcol[mt - 1] != tc);
         const unsigned bl = __ballot_sync(0xffffffffu, start);
         if (lane == 0) M.wcnt[mwarp] = __popc(bl);
         meta_sync();
         int off = 0;
         for (int w2 = 0; w2 < mwarp; w2++) off += M.wcnt[w2];
         const int first = d.run0 + M.fcnt[0] + M.fcnt[1] + M.fcnt[2] + M.fcnt[3];
-        if (gk < u) {
+        if (gk < uc) {
           const int r = off + __popc(bl & ((2u << lane) - 1u)) - 1;
           const SnDev& td = sns[md.sn_base + tc];
           M.run[mt] = r;
@@ -453,7 +517,7 @@ __global__ void __launch_bounds__(kTfThreads, 1)
         s_fail = 1;
         break;
       }
-      if (ring[rs] >= ntasks) break;
+      if (ring[rs].g == 0) break;
       const TfMeta& M = meta[buf];
       const int acc = ord % kTfSlots;
       if (!__all_sync(0xffffffffu, tf_wait(smem_u32(&meta_full[buf]), (uint32_t)((ord / kTfMetaBufs) & 1)) &&
@@ -465,7 +529,7 @@ __global__ void __launch_bounds__(kTfThreads, 1)
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;");
-      const int u = M.u, i0 = M.i0, k0 = M.k0;
+      const int u = M.u, uc = M.uc, i0 = M.i0, k0 = M.k0;
       const int i = 32 * (warp & 3) + lane;  // this thread's tile row
       const int c0 = 32 * (warp >> 2);       // and its 32 columns
       uint32_t v[32];
@@ -480,7 +544,7 @@ __global__ void __launch_bounds__(kTfThreads, 1)
 #pragma unroll
           for (int j = 0; j < 32; j++) {
             const int gk = k0 + c0 + j;
-            if (gk < u && gk <= gi) U[(int64_t)gk * u + gi] = __uint_as_float(v[j]);
+            if (gk < uc && gk <= gi) U[(int64_t)gk * u + gi] = __uint_as_float(v[j]);
           }
         } else {
           // the relative row changes only with the run, which is the same for every lane
@@ -488,7 +552,7 @@ __global__ void __launch_bounds__(kTfThreads, 1)
 #pragma unroll
           for (int j = 0; j < 32; j++) {
             const int kk = c0 + j, gk = k0 + kk;
-            if (gk >= u || gk > gi) continue;
+            if (gk >= uc || gk > gi) continue;
             const int r = M.run[kk];
             if (r != rprev) {
               rprev = r;
@@ -503,7 +567,7 @@ __global__ void __launch_bounds__(kTfThreads, 1)
     }
   }
   __syncthreads();
-  if (s_fail && tid == 0 && ntasks > 0) atomicAdd(mats[sns[tasks[0].x].mat].err + 3, 1ull);
+  if (s_fail && tid == 0) atomicAdd(mats[sns[segs[0].s].mat].err + 3, 1ull);
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   if (warp == 0)
@@ -511,16 +575,23 @@ __global__ void __launch_bounds__(kTfThreads, 1)
                  "r"(kTfSlots * kTfM));
 }
 
+// Planes per part of a factor (or batch) of this width.
+static int tf_planes(int max_width) { return max_width <= 64 ? kTfPlanes64 / 2 : kOzPlanes / 2; }
+int64_t tf_stride_rows(int64_t oz_rows, int max_width) {
+  return (int64_t)(oz_scratch_bytes(oz_rows) / (2 * tf_planes(max_width) * kOzRowBytes));
+}
+
 void launch_tf32_split(const int4* tasks, int ntasks, const SnDev* sns, int max_width, void* oz,
                        int64_t oz_rows, cudaStream_t st) {
   if (ntasks <= 0) return;
   k_tf32_split<<<ntasks, 256, (size_t)max_width * kTfM * sizeof(float), st>>>(
-      tasks, sns, static_cast<uint8_t*>(oz), oz_rows);
+      tasks, sns, static_cast<uint8_t*>(oz), oz_rows, tf_planes(max_width));
 }
 
-void launch_schur_tc(const int4* tasks, int ntasks, int* queue, const SnDev* sns,
-                     const MatDev* mats, bool owner, const void* oz, int64_t oz_rows,
+void launch_schur_tc(const int4* segments, int nsegs, int ntasks, int* queue, const SnDev* sns,
+                     const MatDev* mats, bool owner, int max_width, const void* oz, int64_t oz_rows,
                      long long acc_wait, cudaStream_t st) {
+  const SchurSeg* segs = reinterpret_cast<const SchurSeg*>(segments);
   if (ntasks <= 0) return;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
@@ -528,11 +599,11 @@ void launch_schur_tc(const int4* tasks, int ntasks, int* queue, const SnDev* sns
   const int grid = ntasks < sms ? ntasks : sms;  // one resident CTA per SM, tasks by queue
   const uint8_t* z = static_cast<const uint8_t*>(oz);
   if (owner)
-    k_schur_tf32<true><<<grid, kTfThreads, kTfSmem, st>>>(tasks, ntasks, queue, sns, mats, z,
-                                                         oz_rows, acc_wait);
+    k_schur_tf32<true><<<grid, kTfThreads, kTfSmem, st>>>(segs, nsegs, ntasks, queue, sns, mats, z,
+                                                         oz_rows, tf_planes(max_width), acc_wait);
   else
-    k_schur_tf32<false><<<grid, kTfThreads, kTfSmem, st>>>(tasks, ntasks, queue, sns, mats, z,
-                                                          oz_rows, acc_wait);
+    k_schur_tf32<false><<<grid, kTfThreads, kTfSmem, st>>>(segs, nsegs, ntasks, queue, sns, mats, z,
+                                                          oz_rows, tf_planes(max_width), acc_wait);
 }
 
 int set_tc_kernel_attrs() {

@@ -75,7 +75,7 @@ def test_scaled_blocks(torch, span):
 @pytest.mark.parametrize("precision", [P.CHOL_FP64, P.CHOL_MIXED])
 def test_bad_pivot_column(torch, col, precision):
     a = inputs.uniform(3, 8, 64 * 64).reshape(64, 64)
-    a = a @ a.T + 64 * np.eye(64)
+    a = a @ a.T + np.eye(64)
     L = np.linalg.cholesky(a)
     a[col, col] -= 1.05 * L[col, col] ** 2  # pivot col becomes -0.05 of itself
     A = inputs.from_dense(a)

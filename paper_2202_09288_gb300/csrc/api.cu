@@ -406,7 +406,7 @@ int enqueue_levels(chol_ctx* c, const TaskView& v, const SnDev* sns, const MatDe
       t = v.level(chol::kTaskAsm, l, &cnt);
       if (cnt > 0) {
         prof_begin(c, kProfAsmOwner);
-        chol::launch_assemble_owner(t, cnt, q + 2 + chol::kNumTileClasses, v.asm_src, sns, mats, f32, st);
+        chol::launch_assemble_owner(t, cnt, v.asm_src, sns, mats, f32, st);
         prof_end(c, kProfAsmOwner, 0.0, 0.0);
       }
     }

@@ -27,8 +27,8 @@ void launch_trsm(const int4* tasks, int ntasks, int* queue, const SnDev* sns, in
                  bool f32, cudaStream_t st);
 void launch_schur(int cls, const int4* tasks, int ntasks, int* queue, const SnDev* sns,
                   const MatDev* mats, bool owner, bool f32, cudaStream_t st);
-void launch_assemble_owner(const int4* groups, int ngroups, int* queue, const int4* srcs,
-                           const SnDev* sns, const MatDev* mats, bool f32, cudaStream_t st);
+void launch_assemble_owner(const int4* groups, int ngroups, const int4* srcs, const SnDev* sns,
+                           const MatDev* mats, bool f32, cudaStream_t st);
 int set_factor_kernel_attrs(int max_width);
 // The relative map of a pattern (MatDev::relmap), one CTA per supernode; misses counted.
 void launch_build_relmap(int32_t ns, const int32_t* sn_start, const int64_t* sn_rowptr,

@@ -159,6 +159,7 @@ __global__ void __launch_bounds__(kOzSliceThreads)
   extern __shared__ __align__(16) double xs[];  // [n][kOzSliceLd]
   __shared__ int s_e[kOzM], s_t[kOzInvRows];
   const int4 tk = tasks[blockIdx.x];
+  pdl_wait();
   if (oy && tk.w < 0) return;  // A21 slices only for the tensor-core TRSM's supernodes
   const SnDev d = sns[tk.x];
   const int n = d.n, m = d.m, u = m - n;
@@ -393,6 +394,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
   __shared__ int s_mgo;  // the metadata warps go on with the next task (0: stop)
   __shared__ int s_fail;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  pdl_wait();
   // a launch of an earlier level of this factorization already gave up on a wait: its
   // updates are missing and the factorization is reported failed, so skip the work (before
   // any barrier or tensor memory is set up); every thread reads the same word
@@ -896,6 +898,7 @@ __global__ void __launch_bounds__(kToThreads, 1)
   __shared__ int s_fail;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int4 tk = tasks[blockIdx.x];
+  pdl_wait();
   if (tk.w < 0) return;  // the supernode keeps the FP64 TRSM
   const SnDev d = sns[tk.x];
   unsigned long long* err = mats[d.mat].err;
@@ -994,16 +997,15 @@ void launch_trsm_oz(const int4* tasks, int ntasks, const SnDev* sns, const MatDe
                     const void* oz, int64_t oz_rows, const void* oy, int64_t oy_rows,
                     cudaStream_t st) {
   if (ntasks <= 0) return;
-  k_trsm_oz<<<ntasks, kToThreads, kToSmem, st>>>(tasks, sns, mats,
-                                                 static_cast<const uint8_t*>(oz), oz_rows,
-                                                 static_cast<const uint8_t*>(oy), oy_rows);
+  launch_pdl(k_trsm_oz, ntasks, kToThreads, kToSmem, st, tasks, sns, mats,
+             static_cast<const uint8_t*>(oz), oz_rows, static_cast<const uint8_t*>(oy), oy_rows);
 }
 
 void launch_oz_slice(const int4* tasks, int ntasks, const SnDev* sns, void* oz, int64_t oz_rows,
                      const void* oy, int64_t oy_rows, cudaStream_t st) {
   if (ntasks <= 0) return;
-  k_oz_slice<<<ntasks, kOzSliceThreads, (size_t)64 * kOzSliceLd * sizeof(double), st>>>(
-      tasks, sns, static_cast<uint8_t*>(oz), oz_rows, static_cast<const uint8_t*>(oy), oy_rows);
+  launch_pdl(k_oz_slice, ntasks, kOzSliceThreads, (size_t)64 * kOzSliceLd * sizeof(double), st, tasks,
+             sns, static_cast<uint8_t*>(oz), oz_rows, static_cast<const uint8_t*>(oy), oy_rows);
 }
 
 size_t oy_scratch_bytes(int64_t oy_rows) {
@@ -1021,11 +1023,11 @@ void launch_schur_oz(const int4* segs, int nsegs, int ntasks, int* queue, const 
   const uint8_t* z = static_cast<const uint8_t*>(oz);
   const SchurSeg* sg = reinterpret_cast<const SchurSeg*>(segs);
   if (owner)
-    k_schur_oz<true><<<grid, kOzThreads, kOzSmem, st>>>(sg, nsegs, ntasks, queue, sns, mats, z,
-                                                       oz_rows, acc_wait);
+    launch_pdl(k_schur_oz<true>, grid, kOzThreads, kOzSmem, st, sg, nsegs, ntasks, queue, sns, mats, z,
+               oz_rows, acc_wait);
   else
-    k_schur_oz<false><<<grid, kOzThreads, kOzSmem, st>>>(sg, nsegs, ntasks, queue, sns, mats, z,
-                                                        oz_rows, acc_wait);
+    launch_pdl(k_schur_oz<false>, grid, kOzThreads, kOzSmem, st, sg, nsegs, ntasks, queue, sns, mats,
+               z, oz_rows, acc_wait);
 }
 
 int64_t oz_stride_rows(int64_t oz_rows) {

@@ -219,6 +219,7 @@ __global__ void __launch_bounds__(256)
                  uint8_t* __restrict__ oz, int64_t oz_rows, int pp) {
   extern __shared__ __align__(16) float xf[];  // [n][kTfM]
   const int4 tk = tasks[blockIdx.x];
+  pdl_wait();
   const SnDev d = sns[tk.x];
   const int n = d.n, m = d.m, u = m - n;
   const int r0 = tk.y;
@@ -269,6 +270,7 @@ __global__ void __launch_bounds__(kTfThreads, 1)
   __shared__ int s_fail;
   __shared__ __align__(8) uint64_t never;  // test hook: a barrier nothing completes
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  pdl_wait();
   // a launch of an earlier level of this factorization already gave up on a wait: its
   // updates are missing and the factorization is reported failed, so skip the work (before
   // any barrier or tensor memory is set up); every thread reads the same word
@@ -584,8 +586,8 @@ int64_t tf_stride_rows(int64_t oz_rows, int max_width) {
 void launch_tf32_split(const int4* tasks, int ntasks, const SnDev* sns, int max_width, void* oz,
                        int64_t oz_rows, cudaStream_t st) {
   if (ntasks <= 0) return;
-  k_tf32_split<<<ntasks, 256, (size_t)max_width * kTfM * sizeof(float), st>>>(
-      tasks, sns, static_cast<uint8_t*>(oz), oz_rows, tf_planes(max_width));
+  launch_pdl(k_tf32_split, ntasks, 256, (size_t)max_width * kTfM * sizeof(float), st, tasks, sns,
+             static_cast<uint8_t*>(oz), oz_rows, tf_planes(max_width));
 }
 
 void launch_schur_tc(const int4* segments, int nsegs, int ntasks, int* queue, const SnDev* sns,
@@ -599,11 +601,11 @@ void launch_schur_tc(const int4* segments, int nsegs, int ntasks, int* queue, co
   const int grid = ntasks < sms ? ntasks : sms;  // one resident CTA per SM, tasks by queue
   const uint8_t* z = static_cast<const uint8_t*>(oz);
   if (owner)
-    k_schur_tf32<true><<<grid, kTfThreads, kTfSmem, st>>>(segs, nsegs, ntasks, queue, sns, mats, z,
-                                                         oz_rows, tf_planes(max_width), acc_wait);
+    launch_pdl(k_schur_tf32<true>, grid, kTfThreads, kTfSmem, st, segs, nsegs, ntasks, queue, sns, mats,
+               z, oz_rows, tf_planes(max_width), acc_wait);
   else
-    k_schur_tf32<false><<<grid, kTfThreads, kTfSmem, st>>>(segs, nsegs, ntasks, queue, sns, mats, z,
-                                                          oz_rows, tf_planes(max_width), acc_wait);
+    launch_pdl(k_schur_tf32<false>, grid, kTfThreads, kTfSmem, st, segs, nsegs, ntasks, queue, sns,
+               mats, z, oz_rows, tf_planes(max_width), acc_wait);
 }
 
 int set_tc_kernel_attrs() {

@@ -643,7 +643,11 @@ void build_segments(Sym* S, int32_t l, const std::vector<int8_t>& cls,
   int64_t extra = S->lvl_ozrows[l];  // slice rows of the earlier chunks follow the level's own
   std::vector<int32_t>& sl = S->tasks[f32 ? kTaskSliceMergeF : kTaskSliceMerge];
   const std::vector<int32_t>& own = S->tasks[kTaskOzSlice];
+  const size_t own0 = sl.size();
   sl.insert(sl.end(), own.begin() + 4 * S->task_off[kTaskOzSlice][l], own.end());
+  if (!f32)  // the last chunks of groups share the exponents of the chunk before (w = -2)
+    for (size_t q = own0; q < sl.size(); q += 4)
+      sl[q + 3] = sl[q] > 0 && last[sl[q] - 1] == sl[q] ? -2 : -1;
   for (int32_t q = S->lvl_ptr[l]; q < S->lvl_ptr[l + 1]; q++) {
     const int32_t s = S->lvl_sn[q];
     if (cls[s] != kTile128) continue;
@@ -663,11 +667,10 @@ void build_segments(Sym* S, int32_t l, const std::vector<int8_t>& cls,
       g.kind = kSegOuter;
       g.w = static_cast<int32_t>(extra);
       g.g = s - first + 1;
-      if (!f32) g.count *= g.g;
       for (int32_t c = first; c < s; c++) {
         const int32_t w = S->sn_start[s + 1] - S->sn_start[c + 1];  // rows of c inside the group
         for (int32_t r0 = 0; r0 < u; r0 += 128)
-          push4(sl, c, w + r0, static_cast<int32_t>(extra) - w, -1);
+          push4(sl, c, w + r0, static_cast<int32_t>(extra) - w, f32 ? -1 : -3);
         extra += slice_rows(u);
       }
     }

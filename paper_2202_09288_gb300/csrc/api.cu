@@ -396,9 +396,11 @@ int enqueue_levels(chol_ctx* c, const TaskView& v, const SnDev* sns, const MatDe
       if (tcc && f32)
         chol::launch_schur_tc(t, nseg / 2, segtasks[l], q + 2 + cls, sns, mats, owner, v.max_width, oz,
                               oz_rows, c->acc_wait, st);
-      else if (tcc)
-        chol::launch_schur_oz(t, nseg / 2, segtasks[l], q + 2 + cls, sns, mats, owner, oz, oz_rows,
-                              c->acc_wait, st);
+      else if (tcc) {
+        const int rc = chol::launch_schur_oz(t, nseg / 2, segtasks[l], q + 2 + cls, sns, mats, owner, oz,
+                                             oz_rows, c->acc_wait, st);
+        if (rc != CHOL_OK) return rc;
+      }
       else chol::launch_schur(cls, t, cnt, q + 2 + cls, sns, mats, owner, f32, st);
       prof_end(c, pk, v.flops[kind][l], 0.0);
     }

@@ -216,7 +216,7 @@ int chol_batch_create(chol_ctx* c, int count, chol_num* const* nums, chol_batch*
           } else if (k == chol::kTaskOzSlice || k == chol::kTaskSliceMerge ||
                      k == chol::kTaskSliceMergeF) {  // {s, r0, oz, y}
             b->tasks[k].insert(b->tasks[k].end(),
-                               {t[0] + base[i], t[1], t[2] + zb, t[3] >= 0 ? t[3] + yb : -1});
+                               {t[0] + base[i], t[1], t[2] + zb, t[3] >= 0 ? t[3] + yb : t[3]});
           } else if (k == chol::kTaskPotrf) {     // {s, first_bwd, nbwd, y or -1}
             b->tasks[k].insert(b->tasks[k].end(),
                                {t[0] + base[i], t[1], t[2], t[3] >= 0 ? t[3] + yb : -1});

@@ -57,8 +57,9 @@ enum TaskKind {
   // FP64 tensor-core Schur tiles as segments (SchurSeg, two int4 each) that the kernel expands:
   kTaskSeg = 11,      // every 128-tile supernode's own tiles (owner assembly)
   kTaskSegMerge = 12, // with the updates of a group of chunks merged (see SchurSeg)
-  kTaskSliceMerge = 13, // kTaskOzSlice and {s, r0, oz, -1}: slices of the groups' earlier chunks, for
-                        //   kTaskSegMerge
+  kTaskSliceMerge = 13, // kTaskOzSlice and the slices of the groups' earlier chunks, for
+                        //   kTaskSegMerge: {s, r0, oz, e}, e = -2 / -3: row exponents shared with the
+                        //   chunk before / after s
   kTaskSegMergeF = 14,  // the FP32 factor's (TF32 tiles): every chunk of a group in one task
   kTaskSliceMergeF = 15,
   kNumTaskKinds = 16
@@ -71,12 +72,13 @@ enum TaskKind {
 // cores, bounds the factorization.  So up to kMergeChunks consecutive chunks of one
 // separator form a group: each updates at once only the columns of the group's later
 // chunks (kSegInner), and all of them together the ancestors after the last one is
-// factored (kSegOuter), the tasks of the group's chunks on the same tiles one after another, so
-// that a tile's entries stay in L2 from one to the next.  The FP32 factor's groups are longer and a tile
-// is one task for all of a group's chunks: their products add up in tensor memory and are
-// scattered once (FP64 diagonal sums are exact only up to K = 64 columns of full digits).
-// Measured per factorization, the Schur tiles: 80^3 27-point FP64 1,308 -> 1,241 ms, 48^3
-// 65.4 -> 62.7 ms; 96^3 diffusion in FP32 79.1 -> 37.7 ms.
+// factored (kSegOuter), a tile in one task for all of a group's chunks: their products add up in tensor
+// memory and are scattered once.  FP64 groups have two chunks: the diagonal sums of 8-bit digits are
+// exact in FP32 up to K = 128 columns (7 2^21 < 2^24), with one exponent per row for both chunks.
+// The FP32 factor's have up to four.  (Two tasks per tile on levels of at most 76 tiles, half of the
+// SMs, took as long as one.)
+// Measured per factorization, the Schur tiles: 80^3 27-point FP64 1,308 -> 936 ms, 48^3
+// 65.4 -> 49.4 ms; 96^3 diffusion in FP32 79.1 -> 37.7 ms.
 struct SchurSeg {
   int32_t s;       // the supernode; kSegOuter: the group's last chunk, g - 1 others before it
   int32_t oz;      // first slice row of s
@@ -86,7 +88,7 @@ struct SchurSeg {
                    //   chunks' rows below the group, roundup(u, 8) rows each
   int32_t g;       // chunks (1 but for kSegOuter)
   int32_t nt;      // row strips of 128: ceil(u / 128)
-  int32_t count;   // tasks (FP64 kSegOuter: g per tile)
+  int32_t count;   // tasks
 };
 enum SegKind { kSegAll = 0, kSegInner = 1, kSegOuter = 2 };
 constexpr int kMergeChunks = 2, kMergeChunksF32 = 4;

@@ -59,9 +59,9 @@ int set_tc_kernel_attrs();
 void launch_oz_slice(const int4* tasks, int ntasks, const SnDev* sns, void* oz, int64_t oz_rows,
                      const void* oy, int64_t oy_rows, cudaStream_t st);
 // segs: the level's SchurSeg records (two int4 each), ntasks tile tasks in all
-void launch_schur_oz(const int4* segs, int nsegs, int ntasks, int* queue, const SnDev* sns,
-                     const MatDev* mats, bool owner, const void* oz, int64_t oz_rows,
-                     long long acc_wait, cudaStream_t st);
+int launch_schur_oz(const int4* segs, int nsegs, int ntasks, int* queue, const SnDev* sns,
+                    const MatDev* mats, bool owner, const void* oz, int64_t oz_rows,
+                    long long acc_wait, cudaStream_t st);
 // L21 = A21 Y^T of the 128-tile supernodes on the bf16 tensor cores (kTaskOzSlice tasks: 128
 // rows each): A21's slices from launch_oz_slice with oy on the panel before this launch, Y's
 // slices from launch_potrf (oy); writes L21 into the panels.

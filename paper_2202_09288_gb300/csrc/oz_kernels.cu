@@ -6,25 +6,30 @@
 //   k_oz_slice  every row r of L21 gets an exponent e_r (max_k |L21[r,k]| < 2^e_r) and
 //               kOzSlices integer slices s_p[r,k] of 8 bits with
 //               L21[r,k] = 2^e_r sum_p s_p[r,k] 2^(-7-8p) + (error <= 2^(e_r-56)),
-//               stored as bf16 (exact) in rows of 128 bytes, 16-byte chunks pre-swizzled
-//               for the tensor cores' 128-byte swizzle;
-//   k_schur_oz  a 128 x 128 task is done as four 128 x 32 quarters.  The 7 A slices
-//               (the task's 128 rows) and each quarter's 7 B slices (its 32 rows) are
-//               brought into shared memory by bulk copies issued by a load thread, which
+//               stored as bf16 (exact) in units of 32 columns, rows of 64 bytes whose 16-byte
+//               chunks are pre-swizzled for the tensor cores' 64-byte swizzle;
+//   k_schur_oz  a 128 x 128 task is done as four 128 x 32 quarters.  The units of the task's 128 A
+//               rows and of each quarter's 32 B rows (7 slices each) are brought into
+//               shared memory by tiled TMA copies issued by a load thread, which
 //               also claims the tasks; an MMA thread issues, for every slice pair p + q < 7,
 //               the bf16 MMAs of D_{p+q} += S_p S_q^T into the quarter's set of tensor-memory
-//               accumulators (one per diagonal p + q, 7 x 32 columns; two sets); tasks are
-//               claimed in runs of up to four, so that the later tiles of a row strip reuse
-//               the A slices.  Every partial sum of a diagonal is an integer of at most 7 2^20
-//               (K <= 64), so FP32 accumulation is exact.  Consumer warps read a finished
+//               accumulators (one per diagonal p + q, 7 x 32 columns; two sets).  K is the
+//               supernode's columns (<= 64) or those of two merged chunks (<= 128): every partial
+//               sum of a diagonal is an integer of at most 7 2^21, so FP32 accumulation is exact.
+//               Consumer warps read a finished
 //               set (lane = tile row), release it, form U[i,k] = 2^(e_i+e_k)
 //               sum_d 2^(-14-8d) D_d[i,k] as an FP64 value (integer combination, one
 //               int64 -> double conversion) and add it into the ancestors with FP64
 //               reductions (or write the owner staging buffer) while the tensor cores compute
-//               the next quarter; metadata warps prepare the coming tasks' targets ahead.
+//               the next quarter; metadata warps prepare the next task's targets ahead.
+// What bounds it (80^3 27-point, 23,400 cycles per K = 128 tile): the MMAs (15,400 alone, 16,800 as the
+// MMA thread issues them, 17,500 with the copies, 19,900 with the conversions) and the latency of the
+// copies while the reductions fill the L2 (the rest).  In tiles of K = 64 with one chunk per task
+// the same work took 32,800.
 // Every wait is bounded in time (kOzWaitCycles SM clock cycles, about a second): then the
 // kernel records a timeout in err[3],
 // waits (bounded) for its copies and MMAs in flight, frees its tensor memory and returns.
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -48,16 +53,23 @@ constexpr int kOzMetaBase = kOzConsumers + 64;             // first metadata thr
 constexpr int kOzThreads = kOzMetaBase + kOzMetaThreads;
 constexpr int kOzRing = 16;
 constexpr int kOzM = 128;                                  // tile rows (UMMA M)
-constexpr int kOzN = 64;                                   // columns per half (UMMA N)
-constexpr uint32_t kOzASlice = kOzM * kOzRowBytes;         // 16 KB
+constexpr uint32_t kOzASlice = kOzM * kOzRowBytes;         // 16 KB (TRSM)
+constexpr uint32_t kOzABytes = kOzSlices * kOzASlice;      // 112 KB (TRSM)
+// Schur tiles: operands in units of 32 columns of K (64-byte rows)
 constexpr int kOzQ = 32;                                   // columns per quarter
-constexpr uint32_t kOzQSlice = kOzQ * kOzRowBytes;         // 4 KB: one slice of a quarter
-constexpr uint32_t kOzQBytes = kOzSlices * kOzQSlice;      // 28 KB: a quarter's B operand
+constexpr int kOzUnitRow = 64;                             // bytes of a row's unit
+constexpr uint32_t kOzUASlice = kOzM * kOzUnitRow;         // 8 KB
+constexpr uint32_t kOzUBSlice = kOzQ * kOzUnitRow;         // 2 KB
+constexpr uint32_t kOzUA = kOzSlices * kOzUASlice;         // 56 KB: a unit of A
+constexpr uint32_t kOzUB = kOzSlices * kOzUBSlice;         // 14 KB: a unit of a quarter's B
+constexpr int kOzABufs = 3, kOzBBufs = 3;
 constexpr int kOzSetCols = kOzSlices * kOzQ;               // 224: TMEM columns of a set
-constexpr uint32_t kOzABytes = kOzSlices * kOzASlice;      // 112 KB
-constexpr int kOzBBufs = 3;                                // quarter B buffers
-constexpr size_t kOzSmem = 1024 + kOzABytes + kOzBBufs * kOzQBytes;  // + alignment slack
+constexpr size_t kOzSmem = 512 + kOzABufs * kOzUA + kOzBBufs * kOzUB;  // + alignment slack
 constexpr uint32_t kOzTmemCols = 512;                     // two sets of 7 diagonals (448)
+static_assert(kOzABufs == 3, "the load thread's replacement looks at three buffers");
+// A step as the load thread describes it: A buffer, K steps of 16 (1 or 2), first and last of its
+// quarter, stop.
+constexpr int kStepK = 2, kStepFirst = 4, kStepLast = 5, kStepStop = 6;
 // Bound of every wait in SM clock cycles (~1 s at 2 GHz; the waits of a working launch last
 // microseconds).  Counted with clock64(), not in polls: a poll of mbarrier.try_wait may suspend
 // the thread for a hardware-defined time.
@@ -79,6 +91,12 @@ __device__ __forceinline__ uint64_t oz_desc(uint32_t addr) {
   return d;
 }
 
+// The same with the 64-byte swizzle: 8-row groups 512 bytes apart.
+__device__ __forceinline__ uint64_t oz_desc64(uint32_t addr) {
+  return (uint64_t)((addr >> 4) & 0x3FFF) | (uint64_t)(16 >> 4) << 16 | (uint64_t)(512 >> 4) << 32 |
+         (uint64_t)1 << 46 | (uint64_t)4 << 61;
+}
+
 // Instruction descriptor of kind::f16: FP32 accumulator, bf16 A and B (format 1), both
 // K-major, N >> 3 at bit 17, M >> 4 at bit 24.
 __device__ __forceinline__ uint32_t oz_idesc(int N) {
@@ -88,7 +106,7 @@ __device__ __forceinline__ uint32_t oz_idesc(int N) {
 
 __device__ __forceinline__ bool oz_wait(uint32_t bar, uint32_t parity,
                                         long long limit = kOzWaitCycles) {
-  const long long t0 = clock64();
+  long long t0 = 0;
   for (;;) {
     uint32_t ok;
     asm volatile(
@@ -98,8 +116,21 @@ __device__ __forceinline__ bool oz_wait(uint32_t bar, uint32_t parity,
         : "r"(bar), "r"(parity)
         : "memory");
     if (ok) return true;
-    if (clock64() - t0 > limit) return false;
+    if (t0 == 0) t0 = clock64();
+    else if (clock64() - t0 > limit) return false;
   }
+}
+
+// Whether the phase is complete, without waiting.
+__device__ __forceinline__ bool oz_test(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+      " selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok;
 }
 
 __device__ __forceinline__ void oz_expect(uint32_t bar, uint32_t bytes) {
@@ -113,6 +144,16 @@ __device__ __forceinline__ void oz_bulk_load(uint32_t dst, const void* src, uint
       "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::
           "r"(dst),
       "l"(src), "r"(bytes), "r"(bar)
+      : "memory");
+}
+
+// Tiled copy of a unit: all slices of the 8-row groups from g8 on, half h (see oz_unit_map).
+__device__ __forceinline__ void oz_unit_load(uint32_t dst, const CUtensorMap* map, int g8, int h,
+                                             uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], "
+      "[%1, {%2, %3, %4, %2}], [%5];" ::"r"(dst),
+      "l"(map), "r"(0), "r"(g8), "r"(h), "r"(bar)
       : "memory");
 }
 
@@ -151,13 +192,19 @@ constexpr int kOzSliceLd = kOzM + 1;  // padded column stride of the staged bloc
 // of 8 bits (|s_p| <= 128, exact); thread t writes the
 // 16-byte chunk t % 8 of row t / 8 of every slice (coalesced, pre-swizzled).
 // With oy (the tensor-core TRSM's operand A21 S^-1, sliced before that TRSM), column k is
-// scaled by 2^-t_k, the shift POTRF stored with the supernode's inverse slices in oy.
+// scaled by 2^-t_k, the shift POTRF stored with the supernode's inverse slices in oy, and the planes
+// have rows of 128 bytes.  Without it (the Schur tiles) plane p is two planes of 64-byte rows, its
+// columns 0 .. 31 and 32 .. 63, swizzled by 64 bytes: 16-byte chunk c of slice row R sits at chunk c ^
+// ((R >> 1) & 3).  A task with w = -2 or -3 is one of two merged chunks whose rows get one exponent
+// (their products are summed in tensor memory): w = -2, the chunk before s is the other, w =
+// -3 the one after it; the other's largest exponents are read straight from its panel (a second pass
+// over it, 80^3 27-point: the level's slicing 62 -> 67.5 ms, of 1,434).
 __global__ void __launch_bounds__(kOzSliceThreads)
     k_oz_slice(const int4* __restrict__ tasks, const SnDev* __restrict__ sns,
                uint8_t* __restrict__ oz, int64_t oz_rows, const uint8_t* __restrict__ oy,
                int64_t oy_rows) {
   extern __shared__ __align__(16) double xs[];  // [n][kOzSliceLd]
-  __shared__ int s_e[kOzM], s_t[kOzInvRows];
+  __shared__ int s_e[kOzM], s_t[kOzInvRows], s_f[kOzSliceThreads];
   const int4 tk = tasks[blockIdx.x];
   pdl_wait();
   if (oy && tk.w < 0) return;  // A21 slices only for the tensor-core TRSM's supernodes
@@ -176,16 +223,31 @@ __global__ void __launch_bounds__(kOzSliceThreads)
            : nullptr;
     s_t[threadIdx.x] = shift && threadIdx.x < n ? shift[threadIdx.x] : 0;
   }
+  int fmax = 0;  // largest exponent field of the other chunk's row, half of its columns
+  static_assert(kMergeChunks == 2, "a merged chunk has one other");
+  if (!oy && tk.w <= -2) {
+    const SnDev o = sns[tk.w == -2 ? tk.x - 1 : tk.x + 1];
+    const int i = threadIdx.x & (kOzM - 1);
+    if (i < u - r0) {
+      const int off = tk.w == -2 ? r0 + n : r0 - o.n;  // row r0 of s among the other's rows below
+      const double* P = reinterpret_cast<const double*>(o.L) + o.n + off + i;
+#pragma unroll 8
+      for (int k = threadIdx.x / kOzM; k < o.n; k += kOzSliceThreads / kOzM)
+        fmax = max(fmax, oz_exp_field(P[(int64_t)k * o.m]));
+    }
+  }
+  s_f[threadIdx.x] = fmax;
   cp_async_wait_all();
   __syncthreads();
   const int64_t row0 = tk.z + (int64_t)r0;
   const size_t stride = (size_t)oz_rows * kOzRowBytes;
+  static_assert(kOzSliceThreads == 2 * kOzM, "two threads a row");
   if (threadIdx.x < kOzM) {
     const int i = threadIdx.x;
     // the largest entry's exponent field by integer comparison (the FP64 unit is slow):
     // max |x| = f 2^e with f in [0.5, 1) has e = field - 1022 (0 for rows of zeros and
     // subnormals, whose slices are zero)
-    int emax = 0;  // of the row scaled by 2^-t_k (exponent fields shifted by -t_k)
+    int emax = max(s_f[i], s_f[i + kOzM]);  // of the row scaled by 2^-t_k (exponent fields shifted by -t_k)
     for (int k = 0; k < n; k++) {
       const int f = oz_exp_field(xs[k * kOzSliceLd + i]);
       if (f > 0) emax = max(emax, f - s_t[k]);
@@ -198,7 +260,10 @@ __global__ void __launch_bounds__(kOzSliceThreads)
   for (int item = threadIdx.x; item < kOzM * 8; item += kOzSliceThreads) {
     const int i = item >> 3, pc = item & 7;  // row, physical 16-byte chunk
     if (i >= rows) continue;
-    const int c = pc ^ (int)((row0 + i) & 7);  // logical chunk: columns 8c .. 8c+7
+    const int R7 = (int)((row0 + i) & 7);
+    const int c = pc ^ (oy ? R7 : R7 >> 1);  // logical chunk: columns 8c .. 8c+7
+    uint8_t* dst = oy ? oz + (size_t)(row0 + i) * kOzRowBytes + pc * 16
+                      : oz + ((size_t)(pc >> 2) * oz_rows + row0 + i) * kOzUnitRow + (pc & 3) * 16;
     const int e = s_e[i];
     long long R[8];
 #pragma unroll
@@ -206,7 +271,7 @@ __global__ void __launch_bounds__(kOzSliceThreads)
       const int k = 8 * c + j;
       R[j] = k < n ? oz_fixed(xs[k * kOzSliceLd + i], e + s_t[k]) : 0;  // x 2^-t_k
     }
-    oz_write_chunk(R, oz + (size_t)(row0 + i) * kOzRowBytes + pc * 16, stride);
+    oz_write_chunk(R, dst, stride);
   }
 }
 
@@ -232,27 +297,22 @@ __device__ __forceinline__ uint32_t oz_fbits(uint32_t acc) {
 __device__ __forceinline__ int oz_int(uint32_t acc) { return __float2int_rn(__uint_as_float(acc)); }
 
 // W = V_hi 2^17 + round(V_lo / 2^7) of the seven diagonals, V_hi = sum_{d<4} D_d 2^(8(3-d)),
-// V_lo = sum_{d>=4} D_d 2^(8(6-d)) (|D_d| <= (d+1) 2^20, so |W| < 2^62).  The low diagonals may
-// exceed 2^22 and come as integers (oz_int); the high ones as offset bits f_d = 0x4B400000 + D_d
-// whose offsets are never subtracted one by one: they enter modulo 2^64 (f_3 2^17 and f_2 2^25 as
-// 32 x 32 -> 64-bit multiply-adds, f_1 2^33 + f_0 2^41 in the high word alone), and kOzHiBias =
-// -(0x4B400000 2^17 (1 + 2^8 + 2^16 + 2^24)) >> 32 removes them (it has no low word).  Exact
-// since |W| < 2^63.
-constexpr uint32_t kOzHiBias = 0u - (uint32_t)((0x4B400000ull * ((1ull << 17) + (1ull << 25))) >> 32) -
-                               0x4B400000u * 2u - 0x4B400000u * 512u;
+// V_lo = sum_{d>=4} D_d 2^(8(6-d)) (|D_d| <= (d+1) 2^21 at K = 128, so |W| < 1.01 2^62).  Diagonals 2
+// to 6 may exceed 2^22 and come as integers (oz_int), d_3 2^17 and d_2 2^25 as 32 x 32 -> 64-bit
+// multiply-adds; 0 and 1 as offset bits f_d = 0x4B400000 + D_d, whose offsets are not subtracted one
+// by one: f_1 2^33 + f_0 2^41 are in the high word alone, and kOzHiBias removes them (modulo 2^32).
+constexpr uint32_t kOzHiBias = 0u - 0x4B400000u * 2u - 0x4B400000u * 512u;
 
-__device__ __forceinline__ unsigned long long oz_low(int d4, int d5, int d6) {
+__device__ __forceinline__ long long oz_low(int d4, int d5, int d6) {
   long long v = (long long)d5 * 256 + (d6 + 64);
   v = (long long)d4 * 65536 + v;
-  return (unsigned long long)(v >> 7);  // round(V_lo / 2^7), half up
+  return v >> 7;  // round(V_lo / 2^7), half up
 }
 
-__device__ __forceinline__ long long oz_high(unsigned long long lo, uint32_t f0, uint32_t f1,
-                                             uint32_t f2, uint32_t f3) {
-  unsigned long long w = (unsigned long long)f3 * 131072ull + lo;
-  w = (unsigned long long)f2 * 33554432ull + w;
-  w += (unsigned long long)(f1 * 2u + f0 * 512u + kOzHiBias) << 32;
-  return (long long)w;
+__device__ __forceinline__ long long oz_high(long long lo, uint32_t f0, uint32_t f1, int d2, int d3) {
+  long long w = (long long)d3 * 131072 + lo;
+  w = (long long)d2 * 33554432 + w;
+  return (long long)((unsigned long long)w + ((unsigned long long)(f1 * 2u + f0 * 512u + kOzHiBias) << 32));
 }
 
 // s d 2^E with a subnormal or infinite result (out of line: the consumers' code is long enough)
@@ -280,75 +340,67 @@ __device__ __forceinline__ double oz_to_double(long long W, int E) {
 }
 
 constexpr int kOzMaxRuns = 8;  // column targets per task whose relative rows are cached
-constexpr int kOzMetaBufs = 3;  // metadata buffers: the metadata warps run up to two tasks ahead
+constexpr int kOzMetaBufs = 2;  // metadata buffers: the metadata warps run up to one task ahead
 
-// Per-task metadata, in kOzMetaBufs buffers: the metadata warps build the next tasks' copies
+// Per-task metadata, in kOzMetaBufs buffers: the metadata warps build the next task's copy
 // while the consumers scatter with the current one.
-static_assert(2 * kOzN == 128, "the run count sums four 32-column words");
 struct OzMeta {
-  double* cp[2 * kOzN];  // each column's target panel column (its relative rows are added)
-  int eA[kOzM], eB[2 * kOzN];  // row exponents e_i; column exponents e_k - 55
-  int tcol[2 * kOzN], run[2 * kOzN];
-  int run_start[2 * kOzN + 1];
-  int wcnt[2 * kOzN / 32];  // run starts per 32 columns
-  int fcnt[kOzMetaThreads / 32];  // the supernode's runs before the tile, per warp
-  long long rb[2 * kOzN];  // relative-map base of every run
-  int rp[kOzMaxRuns][kOzM];
-  int nruns;
+  double* cp[kOzM];  // each column's target panel column (its relative rows are added)
+  long long rb[kOzM];  // relative-map base of every run
+  int eA[kOzM], eB[kOzM];  // row exponents e_i; column exponents e_k - 55
+  int rp[kOzMaxRuns][kOzM];  // relative rows (while building, rp[0]: each column's target)
+  uint8_t run[kOzM];
   int u, uc, i0, k0;       // the task: update order, end of its columns, tile origin
   const int32_t* relmap;   // for runs beyond the cached ones
   double* ustage;          // owner assembly: this supernode's staged U
+};
+// ... and what only its construction needs
+static_assert(kOzM == 128, "the run count sums four 32-column words; a run index fits a byte");
+struct OzMetaWork {
+  uint8_t run_start[kOzM];
+  int wcnt[kOzM / 32];  // run starts per 32 columns
+  int fcnt[kOzMetaThreads / 32];  // the supernode's runs before the tile, per warp
 };
 
 // A task as the load thread hands it to the other roles.
 struct OzTask {
   int s, i0, k0;  // supernode, tile origin in its off-diagonal rows
   int oz;         // slice row of its off-diagonal row 0
+  int oz0;        // a merged chunk before it (n0 > 0): slice row of the same row
   int kend;       // columns from here on are not this task's (the update's order, or a group's inner columns)
-  int work;       // quarters | K steps << 8 | A rows of the task before << 16; -1: stop
+  int n0, n;      // K: columns of the chunk before (0: none) and of s; n < 0: stop
 };
 
 // Task ti of segment g (SchurSeg); sns: the descriptors.  A strip's tiles
-// follow one another, so that later ones reuse the A rows; a group's chunks take turns on
-// up to four tiles of a strip.
+// follow one another, so that later ones reuse the A rows.
 __device__ __forceinline__ OzTask oz_task(const SchurSeg& g, int ti, const SnDev* __restrict__ sns) {
-  const int x = ti - g.first;
   const SnDev& d = sns[g.s];
+  int y = ti - g.first, a = 0;
   OzTask t;
   t.s = g.s;
   t.oz = g.oz;
+  t.oz0 = g.w;
+  t.n = d.n;
+  t.n0 = 0;
   t.kend = d.m - d.n;
   if (g.kind == kSegInner) {
     const int nc = (g.w + 127) >> 7;  // column tiles: strip a has min(a + 1, nc)
-    int a = 0, y = x;
     while (a + 1 < nc && y > a) y -= ++a;
-    if (a + 1 < nc) {
-      t.i0 = 128 * a;
-      t.k0 = 128 * y;
-    } else {
-      t.i0 = 128 * (a + y / nc);
-      t.k0 = 128 * (y % nc);
+    if (a + 1 == nc) {
+      a += y / nc;
+      y %= nc;
     }
     t.kend = g.w;
-    return t;
+  } else {
+    if (g.kind == kSegOuter) t.n0 = sns[g.s - 1].n;
+    // strip a: a + 1 tiles after a (a + 1) / 2
+    a = (int)((sqrtf(8.f * (float)y + 1.f) - 1.f) * 0.5f);
+    while (a * (a + 1) / 2 > y) a--;
+    while ((a + 1) * (a + 2) / 2 <= y) a++;
+    y -= a * (a + 1) / 2;
   }
-  // strip a: g (a + 1) tasks after g a (a + 1) / 2
-  const int y = x / g.g;
-  int a = (int)((sqrtf(8.f * (float)y + 1.f) - 1.f) * 0.5f);
-  while (a * (a + 1) / 2 > y) a--;
-  while ((a + 1) * (a + 2) / 2 <= y) a++;
-  const int rem = x - g.g * (a * (a + 1) / 2);
-  const int q = rem / (4 * g.g), r = min(4, a + 1 - 4 * q), pos = rem - 4 * g.g * q;
-  const int c = pos / r, b = 4 * q + pos - c * r;  // chunk c of the group, tile column b
-  int off = 0;
-  if (c < g.g - 1) {  // an earlier chunk: its rows below the group, sliced apart
-    t.s = g.s - (g.g - 1) + c;
-    for (int e = t.s + 1; e <= g.s; e++) off += sns[e].n;
-    t.oz = g.w + c * ((t.kend + 7) & ~7) - off;
-    t.kend += off;
-  }
-  t.i0 = off + 128 * a;
-  t.k0 = off + 128 * b;
+  t.i0 = 128 * a;
+  t.k0 = 128 * y;
   return t;
 }
 
@@ -361,35 +413,40 @@ __device__ __forceinline__ void oz_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
-// A task is done as 128 x 32 quarters.  A load thread (its own warp) claims the tasks, hands
-// each one to the other roles through a ring as soon as it has claimed it, and bulk-copies
-// the task's 7 A slices once and every quarter's B slices into one of kOzBBufs quarter buffers;
-// an MMA thread (its own warp) issues each quarter's MMAs into one of two TMEM sets of 7
+// A task is done as 128 x 32 quarters, a quarter in steps of one unit of K (32 columns).  A load
+// thread (its own warp) claims the tasks, hands each one to the other roles through a ring as soon
+// as it has claimed it, and bulk-copies per step the quarter's B slices of the unit into one of
+// kOzBBufs buffers and the unit's A slices into one of kOzABufs, unless they are still there: the
+// units of K = 128 (4 x 56 KB) do not fit, so successive quarters take them in alternating
+// directions and the buffer used longest ago is replaced, one unit of four per quarter; at K = 64
+// every unit stays for a whole strip of tiles.  An MMA thread (its own warp) issues each
+// step's MMAs into one of two TMEM sets of 7
 // diagonals x 32 columns, slice by slice; the 16 consumer warps drain a finished set (and
 // release it) while the tensor cores compute the next quarter, then scatter; four metadata
-// warps build each task's exponents, column targets and relative rows up to two tasks ahead.
-// Barriers: a_full (a task's 7 A slices in; a task with the previous task's A rows reuses
-// them), a_empty (the MMAs of
-// all tasks that use an A load done), b_full[] / b_empty[] (a quarter B buffer in / read by its
-// MMAs), acc_full[2] (a set's MMAs done), acc_empty[2] (a set
+// warps build each task's exponents, column targets and relative rows one task ahead.
+// Barriers: b_full[] / b_empty[] (a step's B, and its A if that was copied for it, in / the step's
+// MMAs done, which also frees its A buffer), acc_full[2] (a set's MMAs done), acc_empty[2] (a set
 // drained), meta_full[] / meta_empty[] (a metadata buffer built / released), ring_full[]
 // (the task order).
 template <bool OWNER>
 __global__ void __launch_bounds__(kOzThreads, 1)
     k_schur_oz(const SchurSeg* __restrict__ segs, int nsegs, int ntasks, int* __restrict__ queue,
                const SnDev* __restrict__ sns, const MatDev* __restrict__ mats,
-               const uint8_t* __restrict__ oz, int64_t oz_rows, long long acc_wait) {
-  extern __shared__ __align__(1024) unsigned char oz_sm[];
+               const uint8_t* __restrict__ oz, int64_t oz_rows, long long acc_wait,
+               const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b) {
+  extern __shared__ __align__(512) unsigned char oz_sm[];
   unsigned char* A =
-      reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(oz_sm) + 1023) & ~uintptr_t(1023));
-  unsigned char* Bq0 = A + kOzABytes;  // quarter buffers: Bq0, Bq0 + kOzQBytes, ...
-  __shared__ __align__(8) uint64_t a_full, a_empty, b_full[kOzBBufs], b_empty[kOzBBufs];
+      reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(oz_sm) + 511) & ~uintptr_t(511));
+  unsigned char* Bq0 = A + kOzABufs * kOzUA;
+  __shared__ __align__(8) uint64_t b_full[kOzBBufs], b_empty[kOzBBufs];
+  __shared__ int step[kOzBBufs];  // the step in a B buffer: see kStep...
   __shared__ __align__(8) uint64_t acc_full[2], acc_empty[2];
   __shared__ __align__(8) uint64_t ring_full[kOzRing];
   __shared__ OzTask ring[kOzRing];
   __shared__ uint32_t tmem_base;
   __shared__ __align__(8) uint64_t meta_full[kOzMetaBufs], meta_empty[kOzMetaBufs];
   __shared__ OzMeta meta[kOzMetaBufs];
+  __shared__ OzMetaWork mw;
   __shared__ __align__(8) uint64_t never;  // test hook: a barrier nothing completes
   __shared__ int s_mgo;  // the metadata warps go on with the next task (0: stop)
   __shared__ int s_fail;
@@ -410,8 +467,6 @@ __global__ void __launch_bounds__(kOzThreads, 1)
   }
   if (tid == 0) {
     s_fail = 0;
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&a_full)));
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&a_empty)));
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&never)));
     for (int i = 0; i < kOzBBufs; i++) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&b_full[i])));
@@ -440,9 +495,12 @@ __global__ void __launch_bounds__(kOzThreads, 1)
   if (warp == kOzLoadWarp) {
     // ---------------- loads: task claims, ring, bulk copies; one thread ----------------
     if (lane == 0) {
-      long long T = 0;                       // A slice loads issued
-      long long qb = 0;                      // quarter B buffers issued (buffer = qb % kOzBBufs)
-      long long ord = 0;                     // ring entries published
+      int st = 0;                            // steps issued (B buffer st % kOzBBufs)
+      // the A buffers: the unit in each (slice row, half) and the last step that reads it
+      int arow[kOzABufs] = {-1, -1, -1}, ahalf[kOzABufs] = {0, 0, 0};
+      int alast[kOzABufs] = {-3, -2, -1};
+      bool down = false;                     // the next quarter takes its units from the last on
+      int ord = 0;                           // ring entries published
       bool ok = true;
       // Tasks are claimed in runs (g0 per CTA at first, then from the queue): four while more
       // than 16 per CTA remain, then two while more than 4 do, then singles: the tasks of a
@@ -454,20 +512,12 @@ __global__ void __launch_bounds__(kOzThreads, 1)
       // The ring runs one task ahead of the copies: a task is published (and the next one
       // claimed) before the current task's copies are issued, so that the metadata warps
       // can build its targets while the current task is still being copied and computed.
-      int prow = -1;                         // slice row of the last published task's A rows
-      struct Job {
-        OzTask t;
-        int nq;
-        bool reuse;  // the A rows of the task before it (still in shared memory)
-      };
       int sg = -1;  // the segment of the last published task
       SchurSeg seg;
       seg.first = seg.count = 0;
-      auto publish = [&](int ti) -> Job {
-        Job jb;
-        jb.t.work = -1;
-        jb.nq = 0;
-        jb.reuse = false;
+      auto publish = [&](int ti) -> OzTask {
+        OzTask t;
+        t.n = -1;
         if (ti < ntasks) {
           if (ti >= seg.first + seg.count) {  // the next segment, or a search among the later ones
             int lo = sg + 1, hi = nsegs - 1;
@@ -479,20 +529,21 @@ __global__ void __launch_bounds__(kOzThreads, 1)
             sg = lo;
             seg = segs[sg];
           }
-          jb.t = oz_task(seg, ti, sns);
-          jb.nq = min(4, (jb.t.kend - jb.t.k0 + kOzQ - 1) / kOzQ);
-          jb.reuse = jb.t.oz + jb.t.i0 == prow;
-          prow = jb.t.oz + jb.t.i0;
-          jb.t.work = jb.nq | (((sns[jb.t.s].n + 15) >> 4) << 8) | ((int)jb.reuse << 16);
+          t = oz_task(seg, ti, sns);
         }
-        const int rs = (int)(ord % kOzRing);
-        ring[rs] = jb.t;
+        const int rs = ord % kOzRing;
+        ring[rs] = t;
         oz_arrive(smem_u32(&ring_full[rs]));
         ord++;
-        return jb;
+        return t;
+      };
+      // the B buffer of the next step, once the MMAs of the step before it there are done
+      auto b_wait = [&]() -> bool {
+        return st < kOzBBufs ||
+               oz_wait(smem_u32(&b_empty[st % kOzBBufs]), (uint32_t)((st / kOzBBufs - 1) & 1));
       };
       int cur = tq;
-      Job job = publish(cur);
+      OzTask t = publish(cur);
       while (cur < ntasks) {
         if (++tq >= tend) {  // the run is done: claim the next one
           const int g = tq < ntasks - 16 * (int)gridDim.x ? 4
@@ -501,133 +552,151 @@ __global__ void __launch_bounds__(kOzThreads, 1)
                                              : g0 * (int)gridDim.x + atomicAdd(queue, g);
           tend = min(tq + g, ntasks);
         }
-        const Job next = publish(tq);  // the next task (or the stop entry)
-        const OzTask& t = job.t;
-        const int nq = job.nq;
-        // quarter j's B slices, once the MMAs of the quarter before it in the buffer are done
-        auto load_b = [&](int j) -> bool {
-          const int b = (int)(qb % kOzBBufs);
-          if (qb >= kOzBBufs && !oz_wait(smem_u32(&b_empty[b]), (uint32_t)((qb / kOzBBufs - 1) & 1)))
-            return false;
-          const uint32_t bar = smem_u32(&b_full[b]);
-          unsigned char* dst = Bq0 + b * kOzQBytes;
-          oz_expect(bar, kOzQBytes);
-          for (int p = 0; p < kOzSlices; p++)
-            oz_bulk_load(smem_u32(dst + p * kOzQSlice),
-                         oz + p * stride + (size_t)(t.oz + t.k0 + kOzQ * j) * kOzRowBytes,
-                         kOzQSlice, bar);
-          qb++;
-          return true;
-        };
-        // the first quarters' B goes first: its buffers are free before the A slices are
-        const int early = min(nq, kOzBBufs - 1);
-        for (int j = 0; j < early && ok; j++) ok = load_b(j);
-        if (!ok) break;
-        // the A slices of this task (unless the previous task had the same rows), once the
-        // previous task's MMAs are done: every K step reads every slice
-        if (!job.reuse) {
-          if (T >= 1 && !oz_wait(smem_u32(&a_empty), (uint32_t)((T - 1) & 1))) {
-            ok = false;
-            break;
+        const OzTask next = publish(tq);  // the next task (or the stop entry)
+        const int nq = min(4, (t.kend - t.k0 + kOzQ - 1) / kOzQ);
+        const int z0 = (t.n0 + 31) >> 5, nz = z0 + ((t.n + 31) >> 5);  // units
+        for (int j = 0; j < nq && ok; j++, down = !down)
+          for (int zz = 0; zz < nz; zz++, st++) {
+            const int z = down ? nz - 1 - zz : zz;
+            const int row = z < z0 ? t.oz0 : t.oz, h = z < z0 ? z : z - z0;
+            const int left = (z < z0 ? t.n0 : t.n) - 32 * h;
+            ok = b_wait();
+            if (!ok) break;
+            int ab = 0;
+            bool hit = false;
+#pragma unroll
+            for (int i = 0; i < kOzABufs; i++)
+              if (arow[i] == row + t.i0 && ahalf[i] == h) {
+                ab = i;
+                hit = true;
+              }
+            if (!hit) {  // replace the unit used longest ago, once its last MMAs are done
+#pragma unroll
+              for (int i = 1; i < kOzABufs; i++)
+                if (alast[i] < (ab == 0 ? alast[0] : alast[1])) ab = i;
+            }
+            const int b = st % kOzBBufs;
+            const uint32_t bar = smem_u32(&b_full[b]);
+            if (!hit) {
+              const int last = ab == 0 ? alast[0] : (ab == 1 ? alast[1] : alast[2]);
+              // (steps up to st - kOzBBufs are done: the wait for the B buffer)
+              if (last > st - kOzBBufs && last >= 0 &&
+                  !oz_wait(smem_u32(&b_empty[last % kOzBBufs]), (uint32_t)((last / kOzBBufs) & 1))) {
+                ok = false;
+                break;
+              }
+            }
+#pragma unroll
+            for (int i = 0; i < kOzABufs; i++)
+              if (ab == i) {
+                arow[i] = row + t.i0;
+                ahalf[i] = h;
+                alast[i] = st;
+              }
+            step[b] = ab | (left > 16 ? 2 : 1) << kStepK | (zz == 0 ? 1 << kStepFirst : 0) |
+                      (zz == nz - 1 ? 1 << kStepLast : 0);
+            // a unit of A counts on its first step's barrier: the later steps that find it come after
+            oz_expect(bar, hit ? kOzUB : kOzUA + kOzUB);
+            oz_unit_load(smem_u32(Bq0 + b * kOzUB), &map_b, (row + t.k0 + kOzQ * j) >> 3, h, bar);
+            if (!hit) oz_unit_load(smem_u32(A + ab * kOzUA), &map_a, (row + t.i0) >> 3, h, bar);
           }
-          oz_expect(smem_u32(&a_full), kOzABytes);
-          for (int p = 0; p < kOzSlices; p++)
-            oz_bulk_load(smem_u32(A + p * kOzASlice),
-                         oz + p * stride + (size_t)(t.oz + t.i0) * kOzRowBytes, kOzASlice,
-                         smem_u32(&a_full));
-          T++;
-        }
-        for (int j = early; j < nq && ok; j++) ok = load_b(j);
         if (!ok) break;
-        job = next;
+        t = next;
         cur = tq;
+      }
+      if (ok && b_wait()) {  // the stop step
+        step[st % kOzBBufs] = 1 << kStepStop;
+        oz_arrive(smem_u32(&b_full[st % kOzBBufs]));
+        st++;
+      } else {
+        ok = false;
       }
       if (!ok) {
         s_fail = 1;
-        const int rs = (int)(ord % kOzRing);
-        ring[rs].work = -1;
+        const int rs = ord % kOzRing;
+        ring[rs].n = -1;
         oz_arrive(smem_u32(&ring_full[rs]));
       }
-      // bounded waits for the copies still in flight: the last A load and the last B load of
-      // each buffer
-      if (T >= 1) oz_wait(smem_u32(&a_full), (uint32_t)((T - 1) & 1));
-      for (long long qq = qb - kOzBBufs < 0 ? 0 : qb - kOzBBufs; qq < qb; qq++)
-        oz_wait(smem_u32(&b_full[qq % kOzBBufs]), (uint32_t)((qq / kOzBBufs) & 1));
+      // bounded waits for the copies still in flight: the last steps'
+      for (int q = max(0, st - kOzBBufs); q < st; q++)
+        oz_wait(smem_u32(&b_full[q % kOzBBufs]), (uint32_t)((q / kOzBBufs) & 1));
     }
   } else if (warp == kOzMmaWarp) {
-    // ---------------- MMAs: one elected thread, the warp's control flow uniform ----------------
-    // The loop over a quarter's MMAs is rolled and short: it shares its scheduler's instruction
+    // ---------------- MMAs: one elected thread ----------------
+    // The loop over a step's MMAs is rolled and short: it shares its scheduler's instruction
     // cache with consumer warps that run through long unrolled code, and an unrolled loop was
     // refetched line by line (2,800 cycles of issuing per quarter whose MMAs take 1,930).
-    const bool lead = oz_elect();
-    // N = (7 - p) x 32: the MMA of slice p against slices 0 .. 6-p of a quarter
-    const uint32_t idesc0 = oz_idesc(kOzSlices * kOzQ);
-    constexpr uint32_t kIdStep = (uint32_t)(kOzQ >> 3) << 17, kAStep = kOzASlice >> 4;
-    const uint64_t da0 = oz_desc(smem_u32(A)), db0 = oz_desc(smem_u32(Bq0));
-    bool ok = true;
-    int q = 0;            // quarters issued (TMEM set q & 1)
-    int bb = 0, bpar = 0;  // B buffer q % kOzBBufs and the parity of its use
-    int T = 0;            // A slice loads waited for
-    for (int ord = 0; ok; ord++) {
-      const int rs = ord % kOzRing;
-      if (!oz_wait(smem_u32(&ring_full[rs]), (uint32_t)((ord / kOzRing) & 1))) {
-        ok = false;
-        break;
-      }
-      const int work = ring[rs].work;
-      if (work < 0) break;
-      const int nq = work & 0xff, ks = (work >> 8) & 0xff;
-      const bool reuse = (work >> 16) & 1;  // the previous task's A slices
-      // the A slices are free when every MMA so far is done (one commit per A load, so that the
-      // load thread, which waits for each, is never two phases apart from this one)
-      if (!reuse && T > 0 && lead) oz_commit(smem_u32(&a_empty));
-      for (int j = 0; j < nq; j++, q++) {
-        const int b = q & 1;
-        ok = oz_wait(smem_u32(&b_full[bb]), (uint32_t)bpar) &&
-             (q < 2 ||  // the set was drained (quarter q - 2)
-              oz_wait(smem_u32(&acc_empty[b]), (uint32_t)(((q >> 1) - 1) & 1))) &&
-             (j > 0 || reuse || oz_wait(smem_u32(&a_full), (uint32_t)(T & 1)));  // the task's A
-        ok = __all_sync(0xffffffffu, ok);
+    if (oz_elect()) {
+      // N = (7 - p) x 32: the MMA of slice p against slices 0 .. 6-p of a quarter
+      const uint32_t idesc0 = oz_idesc(kOzSlices * kOzQ);
+      constexpr uint32_t kIdStep = (uint32_t)(kOzQ >> 3) << 17, kAStep = kOzUASlice >> 4;
+      const uint64_t da0 = oz_desc64(smem_u32(A)), db0 = oz_desc64(smem_u32(Bq0));
+      bool ok = true;
+      int q = 0;            // quarters issued (TMEM set q & 1)
+      int bb = 0, bpar = 0;  // the step's B buffer and the parity of its use
+      int st = 0;           // steps issued
+      bool ready = false, drained = false;  // the next step is in / its set drained
+      int snext = 0;
+      uint32_t acc = 0;
+      for (;; st++) {
+        ok = ready || oz_wait(smem_u32(&b_full[bb]), (uint32_t)bpar);
         if (!ok) break;
+        const int s = ready ? snext : *(volatile int*)&step[bb];
+        if (s >> kStepStop & 1) break;
+        const int ab = s & ((1 << kStepK) - 1), b = q & 1;
+        if (s >> kStepFirst & 1) {
+          // the set was drained (quarter q - 2)
+          ok = q < 2 || drained || oz_wait(smem_u32(&acc_empty[b]), (uint32_t)(((q >> 1) - 1) & 1));
+          if (!ok) break;
+          acc = 0;
+        }
         asm volatile("tcgen05.fence::after_thread_sync;");
         // K step outer, slice inner: consecutive MMAs start at different diagonals (measured
-        // 2.3x faster than issuing one slice's K steps back to back into the same columns)
-        uint64_t da = da0, db = db0 + (uint64_t)((bb * kOzQBytes) >> 4);
+        // 2.3x faster than issuing one slice's K steps back to back into the same columns).  The second
+        // K step takes the slices from the last to the first: the largest MMAs (N = 160 to 224) then end a
+        // step and, queued, keep the tensor cores busy over the commit and the next step's waits.
+        uint64_t da = da0 + (uint64_t)((ab * kOzUA) >> 4), db = db0 + (uint64_t)((bb * kOzUB) >> 4);
         uint32_t col = tmem + (uint32_t)(b * kOzSetCols), id = idesc0;
-        int left = ks, p = 0;
-        uint32_t acc = 0;
 #pragma unroll 1
-        while (left > 0) {
-          if (lead) oz_mma(col, da, db, id, acc);
+        for (int p = 0; p < kOzSlices; p++) {
+          oz_mma(col, da, db, id, acc);
           acc = 1;
-          if (++p < kOzSlices) {
-            da += kAStep;
-            col += kOzQ;
-            id -= kIdStep;
-          } else {
-            p = 0;
-            left--;
-            da -= (kOzSlices - 1) * kAStep - 2;
-            db += 2;
-            col -= (kOzSlices - 1) * kOzQ;
-            id = idesc0;
+          da += kAStep;
+          col += kOzQ;
+          id -= kIdStep;
+        }
+        // the next step's waits, if they are over, while these MMAs run
+        const int nb = bb + 1 == kOzBBufs ? 0 : bb + 1, npar = nb == 0 ? bpar ^ 1 : bpar;
+        ready = oz_test(smem_u32(&b_full[nb]), (uint32_t)npar);
+        drained = false;
+        if (ready) {
+          snext = *(volatile int*)&step[nb];
+          drained = (s >> kStepLast & 1) && q >= 1 &&
+                    oz_test(smem_u32(&acc_empty[b ^ 1]), (uint32_t)(((q + 1) >> 1) - 1) & 1);
+        }
+        if ((s >> kStepK & 3) == 2) {
+          da += 2;
+          db += 2;
+#pragma unroll 1
+          for (int p = 0; p < kOzSlices; p++) {
+            da -= kAStep;
+            col -= kOzQ;
+            id += kIdStep;
+            oz_mma(col, da, db, id, 1u);
           }
         }
-        if (lead) {
+        if (s >> kStepLast & 1) {
           oz_commit(smem_u32(&acc_full[b]));
-          oz_commit(smem_u32(&b_empty[bb]));
+          q++;
         }
-        if (++bb == kOzBBufs) {
-          bb = 0;
-          bpar ^= 1;
-        }
+        oz_commit(smem_u32(&b_empty[bb]));
+        bb = nb;
+        bpar = npar;
       }
-      if (!reuse) T++;
-    }
-    if (lead) {
       if (!ok) s_fail = 1;
-      // bounded wait for the MMAs in flight (the last quarter's commit covers all earlier ones)
-      if (q >= 1) oz_wait(smem_u32(&acc_full[(q - 1) & 1]), (uint32_t)(((q - 1) >> 1) & 1));
+      // bounded wait for the MMAs in flight (the last step's commit covers all earlier ones)
+      if (st >= 1)
+        oz_wait(smem_u32(&b_empty[(st - 1) % kOzBBufs]), (uint32_t)(((st - 1) / kOzBBufs) & 1));
     }
     __syncwarp();
   } else if (warp >= kOzMetaBase / 32) {
@@ -645,11 +714,11 @@ __global__ void __launch_bounds__(kOzThreads, 1)
         const int rs = ord % kOzRing;
         int go = 0;
         if (!oz_wait(smem_u32(&ring_full[rs]), (uint32_t)((ord / kOzRing) & 1)) ||
-            (ring[rs].work >= 0 && ord >= kOzMetaBufs &&
+            (ring[rs].n >= 0 && ord >= kOzMetaBufs &&
              !oz_wait(smem_u32(&meta_empty[buf]), (uint32_t)((ord / kOzMetaBufs - 1) & 1))))
           s_fail = 1;
         else
-          go = ring[rs].work >= 0;
+          go = ring[rs].n >= 0;
         s_mgo = go;
       }
       oz_meta_sync();
@@ -662,6 +731,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
       const int n = d.n, u = d.m - n, i0 = tk.i0, k0 = tk.k0, uc = tk.kend;
       const MatDev md = mats[d.mat];
       const int gk = k0 + mt;
+      // (merged chunks have the same exponents)
       M.eA[mt] = (i0 + mt < u) ? exps[tk.oz + i0 + mt] : 0;
       M.eB[mt] = (gk < uc ? exps[tk.oz + gk] : 0) - 55;  // U = W 2^(e_i + e_k - 55)
       if (mt == 0) {
@@ -676,7 +746,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
         const int32_t* rows = d.rows + n;
         const int grow = gk < uc ? rows[gk] : 0;
         const int tc = gk < uc ? md.col2sn[grow] : -1;
-        M.tcol[mt] = tc;
+        M.rp[0][mt] = tc;
         // the supernode's runs that start after position 0 and at or before k0: their count
         // is the index (from run0) of the run holding the tile's first column; the tile's
         // runs are that run and the ones after it, in order (runs split where the target
@@ -684,36 +754,35 @@ __global__ void __launch_bounds__(kOzThreads, 1)
         int before = 0;
         for (int t = 1 + mt; t < d.nrun; t += kOzMetaThreads) before += md.run_a[d.run0 + t] <= k0 ? 1 : 0;
         before = __reduce_add_sync(0xffffffffu, before);
-        if (lane == 0) M.fcnt[mwarp] = before;
+        if (lane == 0) mw.fcnt[mwarp] = before;
         oz_meta_sync();
         // a column starts a run when its target differs from its left neighbour's; its run
         // index is the number of starts up to it, less one
-        const bool start = gk < uc && (mt == 0 || M.tcol[mt - 1] != tc);
+        const bool start = gk < uc && (mt == 0 || M.rp[0][mt - 1] != tc);
         const unsigned bl = __ballot_sync(0xffffffffu, start);
-        if (lane == 0) M.wcnt[mwarp] = __popc(bl);
+        if (lane == 0) mw.wcnt[mwarp] = __popc(bl);
         oz_meta_sync();
         int off = 0;
-        for (int w2 = 0; w2 < mwarp; w2++) off += M.wcnt[w2];
-        const int first = d.run0 + M.fcnt[0] + M.fcnt[1] + M.fcnt[2] + M.fcnt[3];
+        for (int w2 = 0; w2 < mwarp; w2++) off += mw.wcnt[w2];
+        const int first = d.run0 + mw.fcnt[0] + mw.fcnt[1] + mw.fcnt[2] + mw.fcnt[3];
         if (gk < uc) {
           const int r = off + __popc(bl & ((2u << lane) - 1u)) - 1;
           const SnDev& td = sns[md.sn_base + tc];
-          M.run[mt] = r;
+          M.run[mt] = (uint8_t)r;
           M.cp[mt] = reinterpret_cast<double*>(td.L) + (int64_t)(grow - td.col0) * td.m;
           if (start) {  // the run's first column fetches its map base
-            M.run_start[r] = mt;
+            mw.run_start[r] = (uint8_t)mt;
             M.rb[r] = md.run_base[first + r];
           }
         }
-        if (mt == 0) M.nruns = M.wcnt[0] + M.wcnt[1] + M.wcnt[2] + M.wcnt[3];
         oz_meta_sync();
         // relative rows of the cached runs: this thread's tile row in each, all loads in flight
         static_assert(kOzMetaThreads == kOzM, "one metadata thread per tile row");
-        const int nrc = min(M.nruns, kOzMaxRuns), g = i0 + mt;
+        const int nrc = min(mw.wcnt[0] + mw.wcnt[1] + mw.wcnt[2] + mw.wcnt[3], kOzMaxRuns), g = i0 + mt;
         int rpv[kOzMaxRuns];
 #pragma unroll
         for (int r = 0; r < kOzMaxRuns; r++)
-          rpv[r] = (r < nrc && g < u && g >= k0 + M.run_start[r]) ? md.relmap[M.rb[r] + g] : -1;
+          rpv[r] = (r < nrc && g < u && g >= k0 + mw.run_start[r]) ? md.relmap[M.rb[r] + g] : -1;
 #pragma unroll
         for (int r = 0; r < kOzMaxRuns; r++)
           if (r < nrc) M.rp[r][mt] = rpv[r];
@@ -738,7 +807,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
         s_fail = 1;
         break;
       }
-      if (ring[rs].work < 0) break;
+      if (ring[rs].n < 0) break;
       const OzMeta& M = meta[buf];
       if (!__all_sync(0xffffffffu, oz_wait(smem_u32(&meta_full[buf]), (uint32_t)((ord / kOzMetaBufs) & 1)))) {
         s_fail = 1;
@@ -776,7 +845,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
             // e_k - 55)
             const uint32_t ta =
                 tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(b * kOzSetCols + c8);
-            unsigned long long w[8];
+            long long w[8];
             {
               uint32_t v[3][8];
 #pragma unroll
@@ -794,9 +863,8 @@ __global__ void __launch_bounds__(kOzThreads, 1)
               oz_tmem_wait();
 #pragma unroll
               for (int jj = 0; jj < 8; jj++)
-                w[jj] = (unsigned long long)oz_high(w[jj], oz_fbits(v[0][jj]),
-                                                    oz_fbits(v[1][jj]), oz_fbits(v[2][jj]),
-                                                    oz_fbits(v[3][jj]));
+                w[jj] = oz_high(w[jj], oz_fbits(v[0][jj]), oz_fbits(v[1][jj]), oz_int(v[2][jj]),
+                                oz_int(v[3][jj]));
             }
             if (c == 1) {  // the warp's last reads of this set
               asm volatile("tcgen05.fence::before_thread_sync;");
@@ -805,7 +873,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
             }
 #pragma unroll
             for (int jj = 0; jj < 8; jj++)  // -U for the atomics, U for the staging buffer
-              val[jj] = oz_to_double<!OWNER>((long long)w[jj], eA + M.eB[kb + jj]);
+              val[jj] = oz_to_double<!OWNER>(w[jj], eA + M.eB[kb + jj]);
           } else if (c == 1) {
             asm volatile("tcgen05.fence::before_thread_sync;");
             __syncwarp();
@@ -976,9 +1044,9 @@ __global__ void __launch_bounds__(kToThreads, 1)
       for (int j = 0; j < 8; j++) {
         const int col = col0 + j;
         if (i < rb && col < n) {
-          const unsigned long long lo = oz_low(oz_int(v[4][j]), oz_int(v[5][j]), oz_int(v[6][j]));
+          const long long lo = oz_low(oz_int(v[4][j]), oz_int(v[5][j]), oz_int(v[6][j]));
           const long long W =
-              oz_high(lo, oz_fbits(v[0][j]), oz_fbits(v[1][j]), oz_fbits(v[2][j]), oz_fbits(v[3][j]));
+              oz_high(lo, oz_fbits(v[0][j]), oz_fbits(v[1][j]), oz_int(v[2][j]), oz_int(v[3][j]));
           out[(int64_t)col * m] = oz_to_double<false>(W, eA + ey[yrow + col]);
         }
       }
@@ -1012,22 +1080,48 @@ size_t oy_scratch_bytes(int64_t oy_rows) {
   return oz_scratch_bytes(oy_rows) + (size_t)oy_rows * sizeof(int32_t);
 }
 
-void launch_schur_oz(const int4* segs, int nsegs, int ntasks, int* queue, const SnDev* sns,
-                     const MatDev* mats, bool owner, const void* oz, int64_t oz_rows,
-                     long long acc_wait, cudaStream_t st) {
-  if (ntasks <= 0) return;
+// The slices as units for tiled copies: dimensions {8 rows of a unit (512 bytes, as FP64 elements), groups
+// of 8 rows, halves of K, slices}, boxes of `rows` rows and all slices.  One copy per unit: with bulk copies
+// (one per slice and unit, 144 a tile at K = 128) the load thread's issuing bounded the kernel.
+static decltype(&cuTensorMapEncodeTiled) tensor_map_encode() {
+  static const auto fn = [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult r;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &r) !=
+            cudaSuccess ||
+        r != cudaDriverEntryPointSuccess)
+      p = nullptr;
+    return reinterpret_cast<decltype(&cuTensorMapEncodeTiled)>(p);
+  }();
+  return fn;
+}
+static bool oz_unit_map(CUtensorMap* map, const void* oz, int64_t oz_rows, int rows) {
+  const cuuint64_t dim[4] = {64, (cuuint64_t)(oz_rows / 8), 2, kOzSlices};
+  const cuuint64_t stride[3] = {8 * kOzUnitRow, (cuuint64_t)oz_rows * kOzUnitRow,
+                                (cuuint64_t)oz_rows * kOzRowBytes};
+  const cuuint32_t box[4] = {64, (cuuint32_t)(rows / 8), 1, kOzSlices}, one[4] = {1, 1, 1, 1};
+  const auto fn = tensor_map_encode();
+  return fn && fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 4, const_cast<void*>(oz), dim, stride, box, one,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+int launch_schur_oz(const int4* segs, int nsegs, int ntasks, int* queue, const SnDev* sns,
+                    const MatDev* mats, bool owner, const void* oz, int64_t oz_rows,
+                    long long acc_wait, cudaStream_t st) {
+  if (ntasks <= 0) return CHOL_OK;
+  CUtensorMap map_a, map_b;
+  if (!oz_unit_map(&map_a, oz, oz_rows, kOzM) || !oz_unit_map(&map_b, oz, oz_rows, kOzQ))
+    return CHOL_E_CUDA;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int grid = ntasks < sms ? ntasks : sms;  // one resident CTA per SM, tasks by queue
   const uint8_t* z = static_cast<const uint8_t*>(oz);
   const SchurSeg* sg = reinterpret_cast<const SchurSeg*>(segs);
-  if (owner)
-    launch_pdl(k_schur_oz<true>, grid, kOzThreads, kOzSmem, st, sg, nsegs, ntasks, queue, sns, mats, z,
-               oz_rows, acc_wait);
-  else
-    launch_pdl(k_schur_oz<false>, grid, kOzThreads, kOzSmem, st, sg, nsegs, ntasks, queue, sns, mats,
-               z, oz_rows, acc_wait);
+  launch_pdl(owner ? k_schur_oz<true> : k_schur_oz<false>, grid, kOzThreads, kOzSmem, st, sg, nsegs, ntasks,
+             queue, sns, mats, z, oz_rows, acc_wait, map_a, map_b);
+  return CHOL_OK;
 }
 
 int64_t oz_stride_rows(int64_t oz_rows) {
@@ -1039,6 +1133,7 @@ size_t oz_scratch_bytes(int64_t oz_rows) {
 }
 
 int set_oz_kernel_attrs() {
+  if (!tensor_map_encode()) return CHOL_E_CUDA;
   if (cudaFuncSetAttribute(k_oz_slice, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)(64 * kOzSliceLd * sizeof(double))) != cudaSuccess ||
       cudaFuncSetAttribute(k_schur_oz<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -42,7 +42,7 @@ METRIC = "factor GFLOP/s + % FP64 peak; served solves/s and p99 latency at resid
 NOMINAL_FP64_OVER_BF16 = 1.25 / 2250.0  # nominal dense FP64 / BF16 rates of a GB300
 FALLBACK_BF16_TFLOPS = 1900.0
 FP32_SIMT_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
-OZ_PRODUCTS = 36  # slice pairs p + q < 8 of the FP64 tensor-core Schur tiles
+OZ_PRODUCTS = 28  # slice pairs p + q < 7 of the FP64 tensor-core Schur tiles
 NOMINAL_TF32_OVER_BF16 = 1.1 / 2.25  # nominal dense TF32 / BF16 rates of a GB300
 
 
@@ -617,12 +617,12 @@ def main():
     achieved = d["flops"] / (d["ms"] * 1e-3) / 1e12
     traffic = ncu_traffic(dom, d["flops"] / max(d["timed"], 1))
     if dom == "schur128_oz":
-        # FP64 tiles on the bf16 tensor cores: 36 bf16 slice products per FP64 product
+        # FP64 tiles on the bf16 tensor cores: 28 bf16 slice products per FP64 product
         achieved *= OZ_PRODUCTS
         roof = {"bound": "tensor", "peak": peaks["bf16_tflops"],
                 "peak_source": f"bf16 tensor {peak_src} {peaks['bf16_tflops']} TFLOP/s; achieved "
                                f"= {OZ_PRODUCTS} bf16 slice products x the tiles' FP64 flops / "
-                               "time (FP64-equivalent rate = achieved / 36)"}
+                               f"time (FP64-equivalent rate = achieved / {OZ_PRODUCTS})"}
     elif dom == "schur128_tc":
         # FP32 tiles on the TF32 tensor cores: three TF32 products per FP32 product
         achieved *= 3

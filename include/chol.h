@@ -88,9 +88,9 @@ typedef struct chol_opts {
                          factor's pattern, export and flop count stay those of the exact L */
   int fp64_schur;     /* CHOL_FP64 factors: how the 128x128 Schur tiles are computed.
                          CHOL_SCHUR_OZAKI (default): on the bf16 tensor cores (tcgen05) by
-                         splitting every L21 row into 8 exact 7-bit slices scaled by a power
+                         splitting every L21 row into 7 exact 8-bit slices scaled by a power
                          of two; slice products accumulate exactly, so the tile carries FP64
-                         accuracy (representation error < 2^-57 of the row maximum).  Needs
+                         accuracy (representation error <= 2^-56 of the row scale).  Needs
                          W <= 64 (else DMMA).  CHOL_SCHUR_DMMA: FP64 mma.sync tiles. */
 } chol_opts;
 

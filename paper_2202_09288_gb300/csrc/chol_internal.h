@@ -25,13 +25,13 @@ constexpr int kMaxWidth = 128;   // hard limit on the width cap W (diagonal bloc
 // 8 bits,
 //   L21[r,k] 2^-e_r = sum_p s_p[r,k] 2^(-7-8p),  |s_p| <= 128,
 // each exact in bf16.  Slice products are accumulated exactly in FP32 (a partial sum of the
-// diagonal p+q = d is an integer of magnitude <= K (d+1) 2^14, at most 7 2^20 for K <= 64), and
+// diagonal p+q = d is an integer of magnitude <= K (d+1) 2^14, at most 7 2^21 for K <= 128), and
 //   U[i,k] = 2^(e_i+e_k) sum_{p+q < kOzSlices} 2^(-14-8(p+q)) sum_kk s_p[i,kk] s_q[k,kk].
 // The representation error is at most 2^-56 of the row maximum.
 constexpr int kOzSlices = 7;
 constexpr int kOzPlanes = 8;      // planes of a slice scratch (the TF32 parts of 128 columns take 8)
 constexpr int kTfPlanes64 = 4;    // planes of the TF32 parts of up to 64 columns
-constexpr int kOzRowBytes = 128;  // one slice row: 64 bf16 (K <= 64), 128-byte swizzled
+constexpr int kOzRowBytes = 128;  // one slice row: 64 bf16 (of 64 columns)
 constexpr int kOzInvRows = 64;    // slice rows of a diagonal-block inverse (n <= 64, zero-padded)
 enum SchurClass { kTile64 = 0, kTile32 = 1, kTile16 = 2, kTile128 = 3, kNumTileClasses = 4 };
 inline int tile_of_class(int c) {

@@ -10,9 +10,9 @@
 // GEMM of Listing 1) and subtracts it from the ancestor panels.  The lock becomes either
 // device atomics or an owner-pulls assembly in a fixed order.
 //
-// FP64 throughput on GB300 is ~1 TFLOP/s for both DFMA and the FP64 `mma.sync` (DMMA)
-// path, with DMMA a few percent ahead; the 32- and 64-wide Schur tiles here use m8n8k4
-// DMMA, the 128-wide ones the bf16 tensor cores (oz_kernels.cu).
+// FP64 throughput on GB300 is ~1 TFLOP/s for both FMA instructions and the FP64 `mma.sync` (DMMA);
+// the 64-, 32- and 16-wide Schur tiles here use m8n8k4 DMMA (an eighth of the instructions and of the
+// shared-memory loads), the 128-wide ones the bf16 tensor cores (oz_kernels.cu).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -204,9 +204,10 @@ __device__ int potrf_lookahead(T* A, int n, const uint16_t* tab, Accept accept) 
 enum PotrfInverse { kInvBlocks, kInvFull };  // its 16 x 16 diagonal blocks, all of it
 
 // ---- FP64 blocks up to 64 wide: 8 x 8 blocks on the FP64 matrix instruction -----------------------
-// An SM's FP64 unit takes one warp instruction per 19 cycles from all warps together, one per 65
-// from a single warp, but an m8n8k4 product (256 multiply-adds, eight instructions' worth) per
-// 73 from all and 292 from one: twice the rate.  So the block is cut into 8 x 8 blocks: warp 0
+// An SM's FP64 unit takes one FMA warp instruction per 16 to 19 cycles from all warps together and
+// holds a single warp 65 cycles for each; an m8n8k4 product (256 multiply-adds, eight instructions'
+// worth) takes 146 of the unit: no more arithmetic per cycle, but an eighth of the instructions and
+// operand loads.  So the block is cut into 8 x 8 blocks: warp 0
 // factors a diagonal block in registers, in the fewest dependent FP64 instructions, and everything
 // else is 8 x 8 x 8 products, dealt over the other warps.  Layout: A[c * kPld + r], L in the
 // lower triangle, Y in the blocks above it (Y[r, c] at A[r * kPld + c]), Y's diagonal 8 x 8

@@ -4,9 +4,10 @@
 // A row r with exponent e_r (every |x| < 2^e_r) is the integer x 2^(55-e_r) per entry, rounded to
 // nearest, cut into kOzSlices balanced digits of 8 bits (|s_p| <= 128),
 // x = 2^e_r sum_p s_p 2^(-7-8p) + (error <= 2^(e_r-56)),
-// each digit stored as bf16 (exact) in slice planes of 128-byte rows (64 entries, K <= 64)
-// whose 16-byte chunks are pre-swizzled for the tensor cores' 128-byte swizzle: the chunk of
-// columns 8c .. 8c+7 of slice row R sits at physical chunk c ^ (R & 7).
+// each digit stored as bf16 (exact).  The TRSM's operands have slice planes of 128-byte rows (64
+// entries) whose 16-byte chunks are pre-swizzled for the tensor cores' 128-byte swizzle: the chunk of
+// columns 8c .. 8c+7 of slice row R sits at physical chunk c ^ (R & 7).  The Schur tiles' have
+// two planes of 64-byte rows per slice (see k_oz_slice).
 #pragma once
 
 #include <cuda_runtime.h>

@@ -48,7 +48,7 @@ namespace {
 constexpr int kOzConsumers = 512;                          // 16 warps: drain + scatter
 constexpr int kOzMetaThreads = 128;                        // 4 warps: per-task metadata
 constexpr int kOzMmaWarp = kOzConsumers / 32;              // issues the MMAs (one thread)
-constexpr int kOzLoadWarp = kOzMmaWarp + 1;                // issues the bulk copies (one thread)
+constexpr int kOzLoadWarp = kOzMmaWarp + 1;                // issues the TMA copies (one thread)
 constexpr int kOzMetaBase = kOzConsumers + 64;             // first metadata thread
 constexpr int kOzThreads = kOzMetaBase + kOzMetaThreads;
 constexpr int kOzRing = 16;
@@ -493,7 +493,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
   const uint32_t tmem = tmem_base;
 
   if (warp == kOzLoadWarp) {
-    // ---------------- loads: task claims, ring, bulk copies; one thread ----------------
+    // ---------------- loads: task claims, ring, tiled copies; one thread ----------------
     if (lane == 0) {
       int st = 0;                            // steps issued (B buffer st % kOzBBufs)
       // the A buffers: the unit in each (slice row, half) and the last step that reads it
@@ -1080,9 +1080,10 @@ size_t oy_scratch_bytes(int64_t oy_rows) {
   return oz_scratch_bytes(oy_rows) + (size_t)oy_rows * sizeof(int32_t);
 }
 
-// The slices as units for tiled copies: dimensions {8 rows of a unit (512 bytes, as FP64 elements), groups
-// of 8 rows, halves of K, slices}, boxes of `rows` rows and all slices.  One copy per unit: with bulk copies
-// (one per slice and unit, 144 a tile at K = 128) the load thread's issuing bounded the kernel.
+// The slices as units for tiled copies: dimensions {8 rows of a unit (512 bytes, as FP64 elements),
+// groups of 8 rows, halves of K, slices}, boxes of `rows` rows and all slices.  One copy per unit: with
+// bulk copies (one per slice and unit, 144 a tile at K = 128) the load thread issued for 22,000 of a
+// tile's 28,800 cycles.
 static decltype(&cuTensorMapEncodeTiled) tensor_map_encode() {
   static const auto fn = [] {
     void* p = nullptr;

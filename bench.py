@@ -665,7 +665,7 @@ def main():
         "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms_step,
         "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
         "dtype": "f32+f64" if mixed else (
-            "f64 (Schur tiles: exact bf16x8 splits on tensor cores)"
+            "f64 (Schur tiles: exact bf16x7 splits on tensor cores)"
             if args.fp64_schur == "ozaki" and args.width <= 64 else "f64"),
         "data": "synthetic",
         "config": dict(workload_config(args, sym.info["l_storage"]), n=n, nnz_a=A.nnz_lower,

@@ -33,6 +33,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 
 #include "chol_internal.h"
@@ -938,46 +939,46 @@ __global__ void __launch_bounds__(kOzThreads, 1)
 // (A21 S^-1)(Y S)^T is a product of row-sliced operands of exactly the Schur tiles' form,
 // L21[i, j] = 2^(e_i + e_j) sum_{p+q<7} 2^(-14-8(p+q)) sum_k a_p[i,k] y_q[j,k], K = n <= 64, so
 // every diagonal's partial sums are exact in FP32 and the combination is
-// the same integer one.  One CTA per task (128 rows of A21): one thread bulk-copies the task's
-// 7 A slices (112 KB) and Y's 7 slices (64 rows each, 56 KB), then issues, per K step and A
+// the same integer one.  A task is 128 rows of A21.  A CTA per SM takes consecutive tasks: a load and
+// MMA thread (its own warp) bulk-copies a task's 7 A slices (112 KB) and, for another supernode than
+// before, Y's 7 slices (64 rows each, 56 KB), then issues, per K step and A
 // slice p, the MMAs of A_p against Y slices 0 .. 6-p in one go (N = (7-p) 64, at most 256 per
 // MMA): diagonal p + q lands at TMEM columns (p + q) 64.
-// Eight warps then read the accumulators (warp w: TMEM lanes 32 (w & 3) .., columns
-// 32 (w >> 2) ..), combine them exactly, round once to FP64 and store L21 into the panel.
+// Eight warps read the accumulators (warp w: TMEM lanes 32 (w & 3) .., columns
+// 32 (w >> 2) ..), combine them exactly, round once to FP64 and store L21 into the panel, while the
+// next task's slices are on their way.  A CTA per task did these one after another, each at its
+// latency: per 80^3 27-point factorization 47.3 -> 29.9 ms, 48^3 6.4 -> 4.6 ms.
 // (Forming the slices inside this kernel as well was measured slower: one CTA per SM then
 // serializes the slicing, the copies and the tensor work, which separate launches overlap.)
 // Waits are bounded as in the Schur tiles; a timeout is recorded in err[3] and nothing stored.
-constexpr int kToThreads = 256;
+constexpr int kToWarps = 8;                       // of the epilogue
+constexpr int kToThreads = 32 * (kToWarps + 1);
 constexpr uint32_t kToBSlice = kOzInvRows * kOzRowBytes;  // 8 KB: one slice of Y's rows
 constexpr uint32_t kToBBytes = kOzSlices * kToBSlice;      // 56 KB
 constexpr size_t kToSmem = 1024 + kOzABytes + kToBBytes;   // + alignment slack
 constexpr uint32_t kToTmemCols = 512;                      // 7 diagonals of 64 columns
 
 __global__ void __launch_bounds__(kToThreads, 1)
-    k_trsm_oz(const int4* __restrict__ tasks, const SnDev* __restrict__ sns,
+    k_trsm_oz(const int4* __restrict__ tasks, int ntasks, const SnDev* __restrict__ sns,
               const MatDev* __restrict__ mats, const uint8_t* __restrict__ oz, int64_t oz_rows,
               const uint8_t* __restrict__ oy, int64_t oy_rows) {
   extern __shared__ __align__(1024) unsigned char to_sm[];
   unsigned char* A =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(to_sm) + 1023) & ~uintptr_t(1023));
   unsigned char* B = A + kOzABytes;
-  __shared__ __align__(8) uint64_t full, done;
+  __shared__ __align__(8) uint64_t full, done, drained;
   __shared__ uint32_t tmem_base;
   __shared__ int s_fail;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int4 tk = tasks[blockIdx.x];
+  const int e0 = (int)((long long)ntasks * blockIdx.x / gridDim.x);
+  const int e1 = (int)((long long)ntasks * (blockIdx.x + 1) / gridDim.x);
   pdl_wait();
-  if (tk.w < 0) return;  // the supernode keeps the FP64 TRSM
-  const SnDev d = sns[tk.x];
-  unsigned long long* err = mats[d.mat].err;
+  unsigned long long* err = mats[sns[tasks[e0].x].mat].err;
   // a launch of this factorization already gave up on a wait: skip (before any set-up)
   if (*(volatile unsigned long long*)(err + 3) != 0) return;
-  const int n = d.n, m = d.m, u = m - n, r0 = tk.y;
-  const int rb = min(kOzM, u - r0);
   const size_t sa = (size_t)oz_rows * kOzRowBytes, sb = (size_t)oy_rows * kOzRowBytes;
   const int32_t* ea = reinterpret_cast<const int32_t*>(oz + kOzSlices * sa);
   const int32_t* ey = reinterpret_cast<const int32_t*>(oy + kOzSlices * sb);
-  const int64_t arow = (int64_t)tk.z + r0, yrow = tk.w;
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(&tmem_base)),
@@ -988,72 +989,112 @@ __global__ void __launch_bounds__(kToThreads, 1)
     s_fail = 0;
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&full)));
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&done)));
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&drained)), "r"(kToWarps));
     asm volatile("fence.mbarrier_init.release.cluster;");
   }
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = tmem_base;
-  if (tid == 0) {
-    const uint32_t fb = smem_u32(&full);
-    oz_expect(fb, kOzABytes + kToBBytes);
-    for (int p = 0; p < kOzSlices; p++)
-      oz_bulk_load(smem_u32(A + p * kOzASlice), oz + p * sa + (size_t)arow * kOzRowBytes,
-                   kOzASlice, fb);
-    for (int p = 0; p < kOzSlices; p++)
-      oz_bulk_load(smem_u32(B + p * kToBSlice), oy + p * sb + (size_t)yrow * kOzRowBytes,
-                   kToBSlice, fb);
-    if (oz_wait(fb, 0)) {
-      asm volatile("tcgen05.fence::after_thread_sync;");
-      const uint64_t da = oz_desc(smem_u32(A)), db = oz_desc(smem_u32(B));
-      const int ks = (n + 15) >> 4;
-      // K step outer, A slice inner (consecutive MMAs start at different diagonals); the
-      // first K step of slice 0 writes every diagonal, everything after accumulates
-      for (int k = 0; k < ks; k++)
+  if (warp == kToWarps) {
+    if (lane == 0) {
+      const uint32_t fb = smem_u32(&full), db = smem_u32(&done);
+      const uint64_t ad = oz_desc(smem_u32(A)), bd = oz_desc(smem_u32(B));
+      bool ok = true;
+      int it = 0, yrow = -1;  // tasks issued; the supernode whose Y is in B
+      for (int e = e0; e < e1 && ok; e++) {
+        const int4 tk = tasks[e];
+        if (tk.w < 0) continue;  // the supernode keeps the FP64 TRSM
+        // the MMAs of the task before have read A and B
+        if (it > 0 && !oz_wait(db, (uint32_t)((it - 1) & 1))) {
+          ok = false;
+          break;
+        }
+        const bool newy = tk.w != yrow;
+        yrow = tk.w;
+        oz_expect(fb, newy ? kOzABytes + kToBBytes : kOzABytes);
+        const uint8_t* arow = oz + (size_t)((int64_t)tk.z + tk.y) * kOzRowBytes;
         for (int p = 0; p < kOzSlices; p++)
-          for (int q0 = 0; q0 < kOzSlices - p; q0 += 4) {
-            const int nq = min(4, kOzSlices - p - q0);
-            oz_mma(tmem + (uint32_t)((p + q0) * kOzInvRows),
-                   da + (uint64_t)((p * kOzASlice) >> 4) + 2 * k,
-                   db + (uint64_t)((q0 * kToBSlice) >> 4) + 2 * k, oz_idesc(nq * kOzInvRows),
-                   (p > 0 || k > 0) ? 1u : 0u);
-          }
-      oz_commit(smem_u32(&done));
-    } else {
-      s_fail = 1;
-      oz_arrive(smem_u32(&done));
-      oz_wait(fb, 0);  // bounded: the copies in flight
+          oz_bulk_load(smem_u32(A + p * kOzASlice), arow + p * sa, kOzASlice, fb);
+        if (newy)
+          for (int p = 0; p < kOzSlices; p++)
+            oz_bulk_load(smem_u32(B + p * kToBSlice), oy + p * sb + (size_t)yrow * kOzRowBytes,
+                         kToBSlice, fb);
+        const int ks = (sns[tk.x].n + 15) >> 4;
+        ok = oz_wait(fb, (uint32_t)(it & 1));
+        if (!ok) {
+          oz_wait(fb, (uint32_t)(it & 1));  // bounded: the copies in flight
+          break;
+        }
+        if (it > 0 && !oz_wait(smem_u32(&drained), (uint32_t)((it - 1) & 1))) {
+          ok = false;
+          break;
+        }
+        asm volatile("tcgen05.fence::after_thread_sync;");
+        // K step outer, A slice inner (consecutive MMAs start at different diagonals); the
+        // first K step of slice 0 writes every diagonal, everything after accumulates
+        for (int k = 0; k < ks; k++)
+          for (int p = 0; p < kOzSlices; p++)
+            for (int q0 = 0; q0 < kOzSlices - p; q0 += 4) {
+              const int nq = min(4, kOzSlices - p - q0);
+              oz_mma(tmem + (uint32_t)((p + q0) * kOzInvRows),
+                     ad + (uint64_t)((p * kOzASlice) >> 4) + 2 * k,
+                     bd + (uint64_t)((q0 * kToBSlice) >> 4) + 2 * k, oz_idesc(nq * kOzInvRows),
+                     (p > 0 || k > 0) ? 1u : 0u);
+            }
+        oz_commit(db);
+        it++;
+      }
+      if (!ok) s_fail = 1;
+      if (it > 0) oz_wait(db, (uint32_t)((it - 1) & 1));  // bounded: the MMAs in flight
     }
-  }
-  if (!oz_wait(smem_u32(&done), 0)) s_fail = 1;
-  asm volatile("tcgen05.fence::after_thread_sync;");
-  __syncthreads();
-  if (!s_fail) {  // uniform: the warps' TMEM loads are collective
+    __syncwarp();
+  } else {
     const int lq = warp & 3, ch = warp >> 2;
-    const int i = 32 * lq + lane;  // this thread's row of the task
-    const int eA = i < rb ? ea[arow + i] - 55 : 0;
-    double* out = reinterpret_cast<double*>(d.L) + n + r0 + i;
-    for (int c8 = 0; c8 < 4; c8++) {
-      const int col0 = 32 * ch + 8 * c8;
-      uint32_t v[kOzSlices][8];
+    const int i = 32 * lq + lane;  // this thread's row of a task
+    int it = 0;
+    for (int e = e0; e < e1; e++) {
+      const int4 tk = tasks[e];
+      if (tk.w < 0) continue;
+      const SnDev d = sns[tk.x];
+      const int n = d.n, m = d.m, r0 = tk.y, rb = min(kOzM, m - n - r0);
+      const int eA = i < rb ? ea[(int64_t)tk.z + r0 + i] - 55 : 0;
+      const int eY = ey[tk.w + 32 * ch + lane];  // of column 32 ch + lane
+      double* out = reinterpret_cast<double*>(d.L) + n + r0 + i;
+      if (!__all_sync(0xffffffffu, oz_wait(smem_u32(&done), (uint32_t)(it & 1)))) {
+        s_fail = 1;
+        break;
+      }
+      it++;
+      asm volatile("tcgen05.fence::after_thread_sync;");
+      for (int c8 = 0; c8 < 4; c8++) {
+        const int col0 = 32 * ch + 8 * c8;
+        uint32_t v[kOzSlices][8];
 #pragma unroll
-      for (int dd = 0; dd < kOzSlices; dd++)
-        oz_tmem_load8(tmem + ((uint32_t)(32 * lq) << 16) + (uint32_t)(dd * kOzInvRows + col0), v[dd]);
-      oz_tmem_wait();
+        for (int dd = 0; dd < kOzSlices; dd++)
+          oz_tmem_load8(tmem + ((uint32_t)(32 * lq) << 16) + (uint32_t)(dd * kOzInvRows + col0), v[dd]);
+        oz_tmem_wait();
+        if (c8 == 3) {  // the warp's last reads
+          asm volatile("tcgen05.fence::before_thread_sync;");
+          __syncwarp();
+          if (lane == 0) oz_arrive(smem_u32(&drained));
+        }
 #pragma unroll
-      for (int j = 0; j < 8; j++) {
-        const int col = col0 + j;
-        if (i < rb && col < n) {
-          const long long lo = oz_low(oz_int(v[4][j]), oz_int(v[5][j]), oz_int(v[6][j]));
-          const long long W =
-              oz_high(lo, oz_fbits(v[0][j]), oz_fbits(v[1][j]), oz_int(v[2][j]), oz_int(v[3][j]));
-          out[(int64_t)col * m] = oz_to_double<false>(W, eA + ey[yrow + col]);
+        for (int j = 0; j < 8; j++) {
+          const int col = col0 + j;
+          const int E = eA + __shfl_sync(0xffffffffu, eY, 8 * c8 + j);
+          if (i < rb && col < n) {
+            const long long lo = oz_low(oz_int(v[4][j]), oz_int(v[5][j]), oz_int(v[6][j]));
+            const long long W =
+                oz_high(lo, oz_fbits(v[0][j]), oz_fbits(v[1][j]), oz_int(v[2][j]), oz_int(v[3][j]));
+            out[(int64_t)col * m] = oz_to_double<false>(W, E);
+          }
         }
       }
     }
-  } else if (tid == 0) {
-    atomicAdd(err + 3, 1ull);
   }
+  __syncthreads();
+  if (s_fail && tid == 0) atomicAdd(err + 3, 1ull);
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   if (warp == 0)
@@ -1061,11 +1102,18 @@ __global__ void __launch_bounds__(kToThreads, 1)
                  "r"(kToTmemCols));
 }
 
+static int oz_sms() {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return sms;
+}
+
 void launch_trsm_oz(const int4* tasks, int ntasks, const SnDev* sns, const MatDev* mats,
                     const void* oz, int64_t oz_rows, const void* oy, int64_t oy_rows,
                     cudaStream_t st) {
   if (ntasks <= 0) return;
-  launch_pdl(k_trsm_oz, ntasks, kToThreads, kToSmem, st, tasks, sns, mats,
+  launch_pdl(k_trsm_oz, std::min(ntasks, oz_sms()), kToThreads, kToSmem, st, tasks, ntasks, sns, mats,
              static_cast<const uint8_t*>(oz), oz_rows, static_cast<const uint8_t*>(oy), oy_rows);
 }
 
@@ -1114,10 +1162,7 @@ int launch_schur_oz(const int4* segs, int nsegs, int ntasks, int* queue, const S
   CUtensorMap map_a, map_b;
   if (!oz_unit_map(&map_a, oz, oz_rows, kOzM) || !oz_unit_map(&map_b, oz, oz_rows, kOzQ))
     return CHOL_E_CUDA;
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int grid = ntasks < sms ? ntasks : sms;  // one resident CTA per SM, tasks by queue
+  const int grid = std::min(ntasks, oz_sms());  // one resident CTA per SM, tasks by queue
   const uint8_t* z = static_cast<const uint8_t*>(oz);
   const SchurSeg* sg = reinterpret_cast<const SchurSeg*>(segs);
   launch_pdl(owner ? k_schur_oz<true> : k_schur_oz<false>, grid, kOzThreads, kOzSmem, st, sg, nsegs, ntasks,

@@ -950,7 +950,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
 // latency: per 80^3 27-point factorization 47.3 -> 29.9 ms, 48^3 6.4 -> 4.6 ms.
 // (Forming the slices inside this kernel as well was measured slower: one CTA per SM then
 // serializes the slicing, the copies and the tensor work, which separate launches overlap.)
-// Waits are bounded as in the Schur tiles; a timeout is recorded in err[3] and nothing stored.
+// Waits are bounded as in the Schur tiles; a timeout is recorded in err[3] and ends the CTA.
 constexpr int kToWarps = 8;                       // of the epilogue
 constexpr int kToThreads = 32 * (kToWarps + 1);
 constexpr uint32_t kToBSlice = kOzInvRows * kOzRowBytes;  // 8 KB: one slice of Y's rows

@@ -29,6 +29,7 @@
 #include "device_common.cuh"
 #include "kernels.h"
 #include "launch_util.h"
+#include "solve_shape.h"
 
 namespace chol {
 
@@ -164,7 +165,6 @@ __device__ void stage_rows(P* X, const P* __restrict__ L21, int64_t m, int n, in
 // previous level still runs, fetch what no solve kernel writes (descriptors, row lists, Y and,
 // where staged, the panel block) and wait for the previous level only then.
 constexpr int kWideThreads = 4 * kSolveRows;
-enum SolveMode { kLeaf, kNarrow, kSplit };
 template <int MODE>
 __host__ __device__ constexpr int y_threads() { return MODE != kLeaf ? kWideThreads : kSolveThreads; }
 
@@ -606,7 +606,8 @@ __global__ void __launch_bounds__(y_threads<MODE>())
     P* red = xo + up4(n * NR);
     const int nq = (max(u, 1) + kSolveRows - 1) / kSolveRows;
     const int first = (int)blockIdx.x - tk.y / kSolveRows;
-    // one group: the supernode's own counter; several: its first task's, per group
+    // one group: the supernode's own counter; several: its first task's, per group (solve_shape
+    // launches several only where that many counters exist)
     int* counter = arrive + (gridDim.y == 1 ? tk.x : (int)(blockIdx.y * gridDim.x) + first);
     if (!last_arrival(counter, nq)) return;
     // kLeaf: Y over X, no longer read (kNarrow: X is free and holds the sums' parts)
@@ -847,38 +848,6 @@ void launch_scatter_perm(const double* w, const int32_t* perm, const double* sca
   k_scatter_perm<<<grid_for(n * nrhs), 256, 0, st>>>(w, perm, scale, n, nrhs, X, ldx);
 }
 
-// Form of a level of a factor that keeps Y (ntasks tasks of nsup supernodes), and right-hand
-// sides per CTA.  kNarrow while the tasks fit in one wave at one CTA per SM (its footprint is
-// ~115 KB at width 64) and, with several right-hand sides, do not fill every SM with FP64 work
-// (then the split form shares the product with Y); kSplit from two tasks per supernode on.
-// NR: the fewest per CTA with which the tasks times the groups still fit (an idle SM costs
-// nothing, the panel's further reads come from L2) -- for kNarrow's backward, as far as there are
-// arrival counters; otherwise the fewest groups of at most 16, evenly filled.
-constexpr int kWave = 152;
-constexpr int kNrList[] = {1, 2, 4, 8, 12, 16};
-struct SolveShape {
-  int mode, nr, groups;
-};
-static int even_nr(int nrhs) {
-  const int groups = (nrhs + 15) / 16, per = (nrhs + groups - 1) / groups;
-  for (int nr : kNrList)
-    if (nr >= per) return nr;
-  return 16;
-}
-static int fill_nr(int nrhs, int units, int64_t limit) {
-  for (int nr : kNrList)
-    if (nr >= nrhs || (int64_t)units * ((nrhs + nr - 1) / nr) <= limit) return nr;
-  return even_nr(nrhs);
-}
-static SolveShape solve_shape(int nrhs, int ntasks, int nsup, int64_t counters) {
-  const bool split = ntasks >= 2 * nsup && (ntasks > kWave || (int64_t)ntasks * nrhs > 4 * kWave);
-  const int mode = split ? kSplit : ntasks <= kWave ? kNarrow : kLeaf;
-  const int nr = mode == kSplit    ? fill_nr(nrhs, ntasks, 2 * kWave)
-                 : mode == kNarrow ? fill_nr(nrhs, ntasks, std::min<int64_t>(kWave, counters))
-                                   : even_nr(nrhs);
-  return {mode, nr, (nrhs + nr - 1) / nr};
-}
-
 struct FwdArgs {
   const int4 *tasks, *diag;
   int ntasks, nsup;
@@ -920,10 +889,11 @@ static void bwd_y_nr(const BwdArgs& a, const SolveShape& s) {
                bwd_y_elems<NR, M>(a.wl) * sizeof(P), a.st, a.tasks, a.sns, a.ldv, a.nrhs, cfirst, a.W,
                a.w, a.part, a.arrive);
   };
-  if (s.mode == kSplit) go(std::integral_constant<int, kSplit>(), s.groups, 0);
-  else if (s.mode == kNarrow) go(std::integral_constant<int, kNarrow>(), s.groups, 0);
-  else  // one counter per supernode: a launch per group
-    for (int p = 0; p < s.groups; p++) go(std::integral_constant<int, kLeaf>(), 1, p * NR);
+  for (int p = 0; p < s.groups; p += s.bwd_groups) {
+    if (s.mode == kSplit) go(std::integral_constant<int, kSplit>(), s.bwd_groups, p * NR);
+    else if (s.mode == kNarrow) go(std::integral_constant<int, kNarrow>(), s.bwd_groups, p * NR);
+    else go(std::integral_constant<int, kLeaf>(), s.bwd_groups, p * NR);
+  }
 }
 
 // f(integral constant NR) for the shape's NR

@@ -258,8 +258,9 @@ __device__ __forceinline__ double pivot_rcp(double p) {
 // right of column j; left of it the register of the eliminated column c holds M^-1 (M the unit
 // lower factor), whose row j gives u_c, and v_rj becomes -t.  The square roots come at the end,
 // all eight at once: L_rj = a_rj y_j and (L^-1)_rc = y_r (M^-1)_rc with y = p^{-1/2}.
-// Returns the first j whose pivot is not positive, else 8.
-__device__ __forceinline__ int potrf_diag8(double* A, double* Dv, int b) {
+// Returns the first j whose pivot is not positive, else 8; *lossy (shared memory): a pivot fell
+// below half of its diagonal entry (see refined_quotient).
+__device__ __forceinline__ int potrf_diag8(double* A, double* Dv, int b, int* lossy) {
   const int lane = threadIdx.x & 31, r = lane & 7, g = lane >> 3;
   constexpr unsigned full = 0xffffffffu;
   double v[2], raw[2] = {0.0, 0.0}, prow = 1.0;
@@ -268,6 +269,8 @@ __device__ __forceinline__ int potrf_diag8(double* A, double* Dv, int b) {
     const int c = g + 4 * s;
     v[s] = r >= c ? A[(b + c) * kPld + b + r] : A[(b + r) * kPld + b + c];
   }
+  const int dlo = __shfl_sync(full, __double2hiint(v[0]), 8 * (r & 3) + r);  // (r, r), r < 4
+  const int dhi = __shfl_sync(full, __double2hiint(v[1]), 8 * (r & 3) + r);
   int bad = 8;
 #pragma unroll
   for (int j = 0; j < 8; j++) {
@@ -319,6 +322,9 @@ __device__ __forceinline__ int potrf_diag8(double* A, double* Dv, int b) {
     if (c <= r) A[(b + c) * kPld + b + r] = l;
     Dv[r * 8 + c] = c < r ? w : c == r ? y : 0.0;
   }
+  // (high words: one exponent step is a factor of two)
+  const bool small = __any_sync(full, __double2hiint(prow) + 0x100000ll < (r < 4 ? dlo : dhi));
+  if (lane == 0) *lossy = small;
   return bad;
 }
 
@@ -347,6 +353,45 @@ __device__ __forceinline__ void block_product(double* C, int cr, int cn, const d
   c0[cn] = c[1];
 }
 
+// One warp: X <- X D^{-T}, X[r][c] at X[r + c * kPld], D a diagonal block of L and W its inverse, as
+// X0 = X W^T, R = X - X0 D^T, X0 + R W^T.  The product with the computed inverse alone leaves R of the
+// order of 2^-53 |X| |D| |W| instead of substitution's 2^-53 |X0| |D|: for 16 columns with pairs
+// dependent to 10^-5, |A - L L^T| was 5.5e-12 of the diagonal, 2.8e-16 by substitution, and is
+// 3.3e-16 refined.  Taken where a pivot fell below half of its diagonal entry;
+// otherwise the rows of D, scaled to unit length, have diagonals of at least 0.7 and the two
+// agree to a small factor.  (Ratios of the 2D, 3D and 27-point workloads: 0.74 and more, so that
+// their blocks never come here and their times are as before; diffusion with lognormal coefficients:
+// a few blocks in a thousand.)
+__device__ __noinline__ void refined_quotient(double* X, const double* W, const double* D) {
+  const int lane = threadIdx.x & 31, r = lane >> 2, k = lane & 3;
+  double* x = X + r + 2 * k * kPld;  // this lane's two entries of a product
+  double c[2] = {x[0], x[kPld]}, x0[2], a[2], b[2];
+  block_product<false, false>(X, 1, kPld, X, 1, kPld, W, 1, 8);
+  __syncwarp();
+#pragma unroll
+  for (int s = 0; s < 2; s++) {
+    x0[s] = x[s * kPld];
+    a[s] = -X[r + (4 * s + k) * kPld];
+    b[s] = r >= 4 * s + k ? D[(4 * s + k) * kPld + r] : 0.0;
+  }
+  __syncwarp();
+  dmma_884(c, a[0], b[0]);
+  dmma_884(c, a[1], b[1]);
+  x[0] = c[0];
+  x[kPld] = c[1];
+  __syncwarp();
+#pragma unroll
+  for (int s = 0; s < 2; s++) {
+    a[s] = X[r + (4 * s + k) * kPld];
+    b[s] = W[r * 8 + 4 * s + k];
+  }
+  __syncwarp();
+  dmma_884(x0, a[0], b[0]);
+  dmma_884(x0, a[1], b[1]);
+  x[0] = x0[0];
+  x[kPld] = x0[1];
+}
+
 // Cholesky of the n x n block (n <= 64, padded to whole 8 x 8 blocks with the identity, the
 // upper blocks zero) and Y.  Per block column p, one barrier of the CTA:
 //   warp 0: the block below the diagonal one, L_{p+1,p} = A_{p+1,p} D_p^{-T} (D_p the diagonal
@@ -363,35 +408,39 @@ __device__ __forceinline__ void block_product(double* C, int cr, int cn, const d
 // 15.6 ms; 64 x 64 2D Laplacian step 0.70 -> 0.62 ms.
 template <int INV, int WORKERS>
 __device__ int potrf_blocks(double* A, double* Dv, int n) {
-  __shared__ int s_bad;
+  __shared__ int s_bad, s_lossy[8];
   const int warp = threadIdx.x >> 5, nb = (n + 7) / 8;
   int bad = n;
   if (warp == 0) {
-    const int q = potrf_diag8(A, Dv, 0);
+    const int q = potrf_diag8(A, Dv, 0, s_lossy);
     if (q < 8) bad = min(n, q);
   }
   __syncthreads();
   for (int p = 0; p < nb; p++) {
     const int below = nb - 1 - p;
-    const double* D = Dv + 64 * p;
+    const double *D = Dv + 64 * p, *Lp = A + 8 * p * kPld + 8 * p;
+    const bool lossy = s_lossy[p];
     if (warp == 0) {
       if (below > 0) {
         const int b = 8 * (p + 1);
         double* X = A + 8 * p * kPld + b;
-        block_product<false, false>(X, 1, kPld, X, 1, kPld, D, 1, 8);
+        if (lossy) refined_quotient(X, D, Lp);
+        else block_product<false, false>(X, 1, kPld, X, 1, kPld, D, 1, 8);
         __threadfence_block();
         __syncwarp();
         asm volatile("bar.arrive 1, %0;" ::"n"(32 * (WORKERS + 1)) : "memory");
         block_product<true, true>(A + b * kPld + b, 1, kPld, X, 1, kPld, X, kPld, 1);
         __syncwarp();
-        const int q = potrf_diag8(A, Dv + 64 * (p + 1), b);
+        const int q = potrf_diag8(A, Dv + 64 * (p + 1), b, s_lossy + p + 1);
         if (q < 8 && bad == n) bad = min(n, b + q);
       }
     } else if (warp <= WORKERS) {
       const int c0 = INV == kInvFull ? 0 : p & ~1;  // first block column of Y's row p
       const int nx = below > 0 ? below - 1 : 0;
       for (int q = warp - 1; q < nx + p - c0; q += WORKERS) {
-        if (q < nx) {
+        if (lossy) {  // (D^{-1} S = (S^T D^{-T})^T: the same strides)
+          refined_quotient(A + 8 * p * kPld + 8 * (q < nx ? p + 2 + q : c0 + q - nx), D, Lp);
+        } else if (q < nx) {
           double* X = A + 8 * p * kPld + 8 * (p + 2 + q);
           block_product<false, false>(X, 1, kPld, X, 1, kPld, D, 1, 8);
         } else {

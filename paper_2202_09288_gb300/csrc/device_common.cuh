@@ -31,6 +31,15 @@ __device__ __forceinline__ void record_error(const MatDev& md, int col) {
   atomicMin(md.err, (unsigned long long)col + 1ull);
 }
 
+// Records a tensor-core wait that gave up with the factor of every supernode sn(0) .. sn(count - 1)
+// of the work it cuts short: the members of a batch share launches, and any of them may miss updates.
+// All threads of the CTA.
+template <typename F>
+__device__ __forceinline__ void record_timeout(int count, const SnDev* sns, const MatDev* mats, F sn) {
+  for (int i = threadIdx.x; i < count; i += blockDim.x)
+    atomicAdd(mats[sns[sn(i)].mat].err + 3, 1ull);
+}
+
 // Index of the target run of supernode d that holds its off-diagonal row position pos
 // (runs start at increasing positions, the first at 0).
 __device__ __forceinline__ int find_run(const MatDev& md, const SnDev& d, int pos) {

@@ -27,7 +27,7 @@
 // copies while the reductions fill the L2 (the rest).  In tiles of K = 64 with one chunk per task
 // the same work took 32,800.
 // Every wait is bounded in time (kOzWaitCycles SM clock cycles, about a second): then the
-// kernel records a timeout in err[3],
+// kernel records a timeout in err[3] of every factor with work in the launch,
 // waits (bounded) for its copies and MMAs in flight, frees its tensor memory and returns.
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -455,8 +455,12 @@ __global__ void __launch_bounds__(kOzThreads, 1)
   pdl_wait();
   // a launch of an earlier level of this factorization already gave up on a wait: its
   // updates are missing and the factorization is reported failed, so skip the work (before
-  // any barrier or tensor memory is set up); every thread reads the same word
-  if (*(volatile unsigned long long*)(mats[sns[segs[0].s].mat].err + 3) != 0) return;
+  // any barrier or tensor memory is set up); the whole CTA, or none of it: another CTA may be
+  // recording a timeout of this launch
+  if (__syncthreads_or(*(volatile unsigned long long*)(mats[sns[segs[0].s].mat].err + 3) != 0)) {
+    record_timeout(nsegs, sns, mats, [&](int i) { return segs[i].s; });
+    return;
+  }
   const size_t stride = (size_t)oz_rows * kOzRowBytes;
   const int32_t* exps = reinterpret_cast<const int32_t*>(oz + kOzSlices * stride);
 
@@ -924,7 +928,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
     }
   }
   __syncthreads();
-  if (s_fail && tid == 0) atomicAdd(mats[sns[segs[0].s].mat].err + 3, 1ull);
+  if (s_fail) record_timeout(nsegs, sns, mats, [&](int i) { return segs[i].s; });
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   if (warp == 0)
@@ -973,9 +977,11 @@ __global__ void __launch_bounds__(kToThreads, 1)
   const int e0 = (int)((long long)ntasks * blockIdx.x / gridDim.x);
   const int e1 = (int)((long long)ntasks * (blockIdx.x + 1) / gridDim.x);
   pdl_wait();
-  unsigned long long* err = mats[sns[tasks[e0].x].mat].err;
   // a launch of this factorization already gave up on a wait: skip (before any set-up)
-  if (*(volatile unsigned long long*)(err + 3) != 0) return;
+  if (__syncthreads_or(*(volatile unsigned long long*)(mats[sns[tasks[e0].x].mat].err + 3) != 0)) {
+    record_timeout(e1 - e0, sns, mats, [&](int i) { return tasks[e0 + i].x; });
+    return;
+  }
   const size_t sa = (size_t)oz_rows * kOzRowBytes, sb = (size_t)oy_rows * kOzRowBytes;
   const int32_t* ea = reinterpret_cast<const int32_t*>(oz + kOzSlices * sa);
   const int32_t* ey = reinterpret_cast<const int32_t*>(oy + kOzSlices * sb);
@@ -1094,7 +1100,7 @@ __global__ void __launch_bounds__(kToThreads, 1)
     }
   }
   __syncthreads();
-  if (s_fail && tid == 0) atomicAdd(err + 3, 1ull);
+  if (s_fail) record_timeout(e1 - e0, sns, mats, [&](int i) { return tasks[e0 + i].x; });
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   if (warp == 0)

@@ -21,7 +21,7 @@
 //                 different tasks overlap through mbarriers: stage full/empty, accumulator
 //                 full/empty, metadata full/empty, and the ring of the task sequence.
 // Every wait is bounded in time (kTfWaitCycles SM clock cycles, about a second): then the
-// thread records a timeout in err[3]
+// thread records a timeout in err[3] of every factor with work in the launch
 // and stops; its partners then time out as well, waits for copies and MMAs in flight are
 // bounded too, and the tensor memory is freed before the kernel returns.
 #include <cuda_runtime.h>
@@ -273,8 +273,12 @@ __global__ void __launch_bounds__(kTfThreads, 1)
   pdl_wait();
   // a launch of an earlier level of this factorization already gave up on a wait: its
   // updates are missing and the factorization is reported failed, so skip the work (before
-  // any barrier or tensor memory is set up); every thread reads the same word
-  if (*(volatile unsigned long long*)(mats[sns[segs[0].s].mat].err + 3) != 0) return;
+  // any barrier or tensor memory is set up); the whole CTA, or none of it: another CTA may be
+  // recording a timeout of this launch
+  if (__syncthreads_or(*(volatile unsigned long long*)(mats[sns[segs[0].s].mat].err + 3) != 0)) {
+    record_timeout(nsegs, sns, mats, [&](int i) { return segs[i].s; });
+    return;
+  }
   const size_t stride = (size_t)oz_rows * kOzRowBytes;
 
   if (warp == 0) {
@@ -569,7 +573,7 @@ __global__ void __launch_bounds__(kTfThreads, 1)
     }
   }
   __syncthreads();
-  if (s_fail && tid == 0) atomicAdd(mats[sns[segs[0].s].mat].err + 3, 1ull);
+  if (s_fail) record_timeout(nsegs, sns, mats, [&](int i) { return segs[i].s; });
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   if (warp == 0)

@@ -653,7 +653,7 @@ __device__ void slice_inverse(const double* A, const double* Dv, int n, const in
 // operand of its tensor-core TRSM.
 __global__ void __launch_bounds__(kPotrfThreads)
     k_potrf(const int4* __restrict__ tasks, const SnDev* __restrict__ sns,
-            const MatDev* __restrict__ mats, uint8_t* __restrict__ oy, int64_t oy_rows) {
+            const MatDev* __restrict__ mats, uint8_t* oy, int64_t oy_rows) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   double* A = reinterpret_cast<double*>(smem_raw);
   __shared__ int s_e[kOzInvRows], s_t[kOzInvRows];

@@ -24,6 +24,8 @@ inline int task_grid(K kernel, int threads, size_t smem, int ntasks) {
 // ordinary launch writes; for everything else it calls pdl_wait first, which returns when the
 // kernel before has ended and its writes are visible -- and with it every earlier one, since a
 // kernel that calls pdl_wait in all its CTAs cannot end before the one before it.
+// What an earlier kernel of such a chain writes is not read-only while k runs: k's parameters for it are
+// not __restrict__ (the compiler could take its loads through the read-only path, or before the wait).
 // Only kernels of a few CTAs, whose successor has something to fetch meanwhile, call
 // pdl_launch_dependents (the solves, POTRF and the blocked TRSM): from a kernel that fills the GPU the
 // next one's CTAs go to whichever SMs are free first, several to one FP64 unit (with the call

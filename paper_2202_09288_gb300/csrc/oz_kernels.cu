@@ -203,7 +203,7 @@ constexpr int kOzSliceLd = kOzM + 1;  // padded column stride of the staged bloc
 // over it, 80^3 27-point: the level's slicing 62 -> 67.5 ms, of 1,434).
 __global__ void __launch_bounds__(kOzSliceThreads)
     k_oz_slice(const int4* __restrict__ tasks, const SnDev* __restrict__ sns,
-               uint8_t* __restrict__ oz, int64_t oz_rows, const uint8_t* __restrict__ oy,
+               uint8_t* oz, int64_t oz_rows, const uint8_t* oy,
                int64_t oy_rows) {
   extern __shared__ __align__(16) double xs[];  // [n][kOzSliceLd]
   __shared__ int s_e[kOzM], s_t[kOzInvRows], s_f[kOzSliceThreads];
@@ -415,7 +415,7 @@ template <bool OWNER>
 __global__ void __launch_bounds__(kOzThreads, 1)
     k_schur_oz(const SchurSeg* __restrict__ segs, int nsegs, int ntasks, int* __restrict__ queue,
                const SnDev* __restrict__ sns, const MatDev* __restrict__ mats,
-               const uint8_t* __restrict__ oz, int64_t oz_rows, long long acc_wait,
+               const uint8_t* oz, int64_t oz_rows, long long acc_wait,
                const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b) {
   extern __shared__ __align__(512) unsigned char oz_sm[];
   unsigned char* A =
@@ -946,8 +946,8 @@ constexpr uint32_t kToTmemCols = 512;                      // 7 diagonals of 64 
 
 __global__ void __launch_bounds__(kToThreads, 1)
     k_trsm_oz(const int4* __restrict__ tasks, int ntasks, const SnDev* __restrict__ sns,
-              const MatDev* __restrict__ mats, const uint8_t* __restrict__ oz, int64_t oz_rows,
-              const uint8_t* __restrict__ oy, int64_t oy_rows) {
+              const MatDev* __restrict__ mats, const uint8_t* oz, int64_t oz_rows, const uint8_t* oy,
+              int64_t oy_rows) {
   extern __shared__ __align__(1024) unsigned char to_sm[];
   unsigned char* A =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(to_sm) + 1023) & ~uintptr_t(1023));

@@ -293,7 +293,7 @@ __host__ __device__ constexpr int diag_y_elems(int n) {
 template <typename P, int NR, int MODE>
 __global__ void __launch_bounds__(y_threads<MODE>())
     k_fwd_y(const int4* __restrict__ tasks, const SnDev* __restrict__ sns, int64_t ldv, int nrhs,
-            double* __restrict__ y, double* __restrict__ w, double* __restrict__ fstage) {
+            double* y, double* w, double* fstage) {
   constexpr int T = y_threads<MODE>();
   constexpr bool STAGED = MODE != kLeaf;
   // threads split the right-hand sides RS ways and the columns CS ways (staged)
@@ -411,7 +411,7 @@ __global__ void __launch_bounds__(y_threads<MODE>())
 template <typename P, int NR>
 __global__ void __launch_bounds__(kWideThreads)
     k_fwd_diag(const int4* __restrict__ tasks, const SnDev* __restrict__ sns, int64_t ldv, int nrhs,
-               const double* __restrict__ y, double* __restrict__ w) {
+               const double* y, double* w) {
   extern __shared__ __align__(16) double sm[];
   start_next_level(nrhs);
   const SnDev d = sns[tasks[blockIdx.x].x];
@@ -472,9 +472,8 @@ __device__ __forceinline__ bool last_arrival(int* counter, int nq) {
 // them); with fewer sums than threads QG threads share one, every QG-th task each, through hd
 // (T doubles), added in order.  The caller's next barrier publishes r.
 template <typename P, int NR, int T>
-__device__ void sum_partials(const SnDev& d, const double* __restrict__ w, int64_t ldv, int c0,
-                             int nr, const double* __restrict__ pp0, int64_t ps, int W, int nq,
-                             double* hd, P* r) {
+__device__ void sum_partials(const SnDev& d, const double* w, int64_t ldv, int c0, int nr,
+                             const double* pp0, int64_t ps, int W, int nq, double* hd, P* r) {
   const int n = d.n;
   constexpr int QG = 64 * NR >= T ? 1 : (T / (64 * NR) < 8 ? T / (64 * NR) : 8);
   const int items = n * NR;
@@ -525,8 +524,7 @@ __device__ void sum_partials(const SnDev& d, const double* __restrict__ w, int64
 template <typename P, int NR, int MODE>
 __global__ void __launch_bounds__(y_threads<MODE>())
     k_bwd_y(const int4* __restrict__ tasks, const SnDev* __restrict__ sns, int64_t ldv, int nrhs,
-            int cfirst, int W, double* __restrict__ w, double* __restrict__ part,
-            int* __restrict__ arrive) {
+            int cfirst, int W, double* w, double* part, int* arrive) {
   constexpr int T = y_threads<MODE>();
   constexpr int RS = MODE == kLeaf ? 1 : (NR >= 4 ? 4 : NR), RG = NR / RS, IL = NR == 1 ? 4 : 1;
   extern __shared__ __align__(16) double sm[];
@@ -630,7 +628,7 @@ __global__ void __launch_bounds__(y_threads<MODE>())
 template <typename P, int NR>
 __global__ void __launch_bounds__(kWideThreads)
     k_bwd_diag(const int4* __restrict__ tasks, const SnDev* __restrict__ sns, int64_t ldv, int nrhs,
-               int W, int64_t bwd0, double* __restrict__ w, const double* __restrict__ part) {
+               int W, int64_t bwd0, double* w, const double* part) {
   constexpr int T = kWideThreads;
   extern __shared__ __align__(16) double sm[];
   start_next_level(nrhs);

@@ -216,7 +216,7 @@ struct TfMeta {
 // and columns n .. are zero.
 __global__ void __launch_bounds__(256)
     k_tf32_split(const int4* __restrict__ tasks, const SnDev* __restrict__ sns,
-                 uint8_t* __restrict__ oz, int64_t oz_rows, int pp) {
+                 uint8_t* oz, int64_t oz_rows, int pp) {
   extern __shared__ __align__(16) float xf[];  // [n][kTfM]
   const int4 tk = tasks[blockIdx.x];
   pdl_wait();
@@ -255,7 +255,7 @@ template <bool OWNER>
 __global__ void __launch_bounds__(kTfThreads, 1)
     k_schur_tf32(const SchurSeg* __restrict__ segs, int nsegs, int ntasks, int* __restrict__ queue,
                  const SnDev* __restrict__ sns, const MatDev* __restrict__ mats,
-                 const uint8_t* __restrict__ oz, int64_t oz_rows, int pp, long long acc_wait) {
+                 const uint8_t* oz, int64_t oz_rows, int pp, long long acc_wait) {
   extern __shared__ __align__(1024) unsigned char tf_sm[];
   unsigned char* stage_base =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(tf_sm) + 1023) & ~uintptr_t(1023));

@@ -89,8 +89,13 @@ typedef struct chol_opts {
   int fp64_schur;     /* CHOL_FP64 factors: how the 128x128 Schur tiles are computed.
                          CHOL_SCHUR_OZAKI (default): on the bf16 tensor cores (tcgen05) by
                          splitting every L21 row into 7 exact 8-bit slices scaled by a power
-                         of two; slice products accumulate exactly, so the tile carries FP64
-                         accuracy (representation error <= 2^-56 of the row scale).  Needs
+                         of two, the row's scale: one for the columns of a supernode, or of
+                         the two that are updated together (K <= 128 columns).  The kept
+                         slice products accumulate exactly.  Against the exact product, in
+                         units of the two rows' scales, an entry is off by at most
+                         2^-56 per factor and column for the slices' rounding and
+                         about 6 K 2^-56 for the omitted products of low slices
+                         (typically 2^-53 in all for K = 128), then rounded to FP64.  Needs
                          W <= 64 (else DMMA).  CHOL_SCHUR_DMMA: FP64 mma.sync tiles. */
 } chol_opts;
 
@@ -257,7 +262,7 @@ int chol_refine_gmres(chol_ctx* ctx, chol_num* num, int64_t nrhs, const double* 
  * CHOL_E_SCRATCH before any work is enqueued.  The first call on a device looks up the
  * array's device address (with that device current); make that first call before any
  * stream capture.  All calls share the array and leave its contents behind; each call
- * clears the work-queue counters at its head (all that must start at zero).  Calls whose
+ * clears the arrival counters at its head (all that must start at zero).  Calls whose
  * device work overlaps (other streams or contexts on the same device) race on it and must
  * be ordered by the caller.  The array's address is kept for the life of the process: after
  * a cudaDeviceReset of a device (which destroys the context it was looked up in) the entry

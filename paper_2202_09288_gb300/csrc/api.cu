@@ -356,7 +356,7 @@ int enqueue_levels(chol_ctx* c, const TaskView& v, const SnDev* sns, const MatDe
     t = v.level(trsm_oz ? chol::kTaskTrsmRest : chol::kTaskTrsm, l, &cnt);
     if (cnt > 0) {
       prof_begin(c, kt);
-      chol::launch_trsm(t, cnt, q + 1, sns, v.max_width, f32, st);
+      chol::launch_trsm(t, cnt, q, sns, v.max_width, f32, st);
       prof_end(c, kt, v.flops[trsm_oz ? chol::kTaskTrsmRest : chol::kTaskTrsm][l], 0.0);
     }
     // the 128-tile supernodes' TRSM: slices of A21 S^-1, then L21 = A21 Y^T on the tensor
@@ -394,14 +394,14 @@ int enqueue_levels(chol_ctx* c, const TaskView& v, const SnDev* sns, const MatDe
       int nseg = 0;  // in int4
       if (tcc) t = v.level(segs, l, &nseg);
       if (tcc && f32)
-        chol::launch_schur_tc(t, nseg / 2, segtasks[l], q + 2 + cls, sns, mats, owner, v.max_width, oz,
+        chol::launch_schur_tc(t, nseg / 2, segtasks[l], q + 1 + cls, sns, mats, owner, v.max_width, oz,
                               oz_rows, c->acc_wait, st);
       else if (tcc) {
-        const int rc = chol::launch_schur_oz(t, nseg / 2, segtasks[l], q + 2 + cls, sns, mats, owner, oz,
+        const int rc = chol::launch_schur_oz(t, nseg / 2, segtasks[l], q + 1 + cls, sns, mats, owner, oz,
                                              oz_rows, c->acc_wait, st);
         if (rc != CHOL_OK) return rc;
       }
-      else chol::launch_schur(cls, t, cnt, q + 2 + cls, sns, mats, owner, f32, st);
+      else chol::launch_schur(cls, t, cnt, q + 1 + cls, sns, mats, owner, f32, st);
       prof_end(c, pk, v.flops[kind][l], 0.0);
     }
     if (owner) {
@@ -604,8 +604,8 @@ int enqueue_solve_seq(chol_ctx* c, const chol_num* f, int k, const double* B, in
     const int4* tb = task_ptr(sym, chol::kTaskBwd, l, &nb);
     const int4* dg = task_ptr(sym, chol::kTaskPotrf, l, &nsup);
     tr.begin(kProfBwd);
-    chol::launch_bwd(tb, nb, dg, nsup, S.task_off[chol::kTaskBwd][l], f->d_sn, n, k, W, S.lvl_maxw[l], bf.w, bf.part, bf.sq, counters, inv,
-                     f32, st);
+    chol::launch_bwd(tb, nb, dg, nsup, S.task_off[chol::kTaskBwd][l], f->d_sn, n, k, W, S.lvl_maxw[l],
+                     bf.w, bf.part, bf.sq, counters, inv, f32, st);
     tr.end(kProfBwd, S.lvl_panel_bytes[l] * (f32 ? 0.5 : 1.0));
   }
   tr.begin(kProfPerm);

@@ -10,8 +10,9 @@ namespace chol {
 
 void launch_assemble(const double* vals, const int64_t* amap, int64_t nnz, void* L, bool f32,
                      cudaStream_t st);
-// Task launches run one CTA per task (launch_util.h); a grid smaller than the task list would
-// take further tasks from the zero-initialized work-queue counter `queue` (one per launch).
+// Task launches run one CTA per task (launch_util.h).  Those with `queue`, a zero-initialized counter
+// of their own, could also run with fewer, which take further tasks from it (the tensor-core Schur
+// tiles do: one CTA per SM).
 // Widest supernode whose diagonal-block inverse the factor keeps (for the solves).
 constexpr int kDinvMaxWidth = 64;
 // Y = L11^-1 of every supernode of a POTRF task list whose descriptor has dinv set (the

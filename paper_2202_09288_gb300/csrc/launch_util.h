@@ -5,8 +5,8 @@
 
 namespace chol {
 
-// Grid of a task launch: one CTA per task.  Every task kernel also takes further tasks from
-// the launch's work queue when its grid is smaller than the task list, so any grid size is
+// Grid of a task launch: one CTA per task.  The kernels it is used for also take further tasks
+// from the launch's work queue when their grid is smaller than the task list, so any grid size is
 // correct; measured on GB300, one CTA per task (the hardware block scheduler refills SMs as
 // CTAs finish) balances the uneven task costs of a level better than a single resident wave
 // of CTAs taking tasks from the queue.

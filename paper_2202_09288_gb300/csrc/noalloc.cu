@@ -10,7 +10,7 @@
 //
 // The array lives in every GPU that loads the library until the process exits.  Every
 // call uses the same array and leaves its contents behind: the only part that must start
-// at zero, the work-queue counters of the solve's launches at its head, is cleared by each
+// at zero, the arrival counters of the solve at its head, is cleared by each
 // call; every other workspace entry is written before it is read.  Two calls whose device
 // work overlaps (different streams, or different contexts on one device) race on the
 // array, so the caller must order them.

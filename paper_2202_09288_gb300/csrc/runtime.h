@@ -107,7 +107,7 @@ struct chol_num {
   void* L = nullptr;           // panels (double, or float for CHOL_MIXED)
   SnDev* d_sn = nullptr;
   MatDev* d_mat = nullptr;
-  int* d_ctr = nullptr;        // work-queue counters: factor launches, then solve launches
+  int* d_ctr = nullptr;        // the factorization's work-queue counters, then the solves' arrival counters
   unsigned long long* d_err = nullptr;  // [0] failing column + 1, [1] map misses,
                                         // [2] FP64 pivot redos
   double* d_vals = nullptr;    // device copy of A's values (assembly and residual)
@@ -169,12 +169,12 @@ int enqueue_factor(chol_num* f);
 // Releases the device memory of every batch of c (called by chol_destroy).
 void detach_batches(chol_ctx* c);
 TaskView sym_view(const chol_sym* sym);
-// Work-queue counters (one int per task launch): 7 per level for a factorization (POTRF,
-// TRSM, four Schur tile classes, owner assembly).
-constexpr int kFactorCountersPerLevel = 3 + chol::kNumTileClasses;
+// Work-queue counters of a factorization, one int per launch whose kernel can take tasks from a queue:
+// TRSM and the four Schur tile classes of every level.
+constexpr int kFactorCountersPerLevel = 1 + chol::kNumTileClasses;
 inline size_t factor_counters(int32_t nlev) { return kFactorCountersPerLevel * (size_t)nlev + 8; }
-// Arrival counters of a solve's backward step, zeroed at its start: one per supernode and some
-// for levels whose right-hand sides are split over several CTAs.
+// Arrival counters of a solve's backward step, zeroed at its start: one per supernode, and some more
+// for levels that count tasks times groups of right-hand sides (where these fit: solve_shape).
 inline size_t solve_counters(const Sym& S) { return 3 * (size_t)S.nlev + 8 + (size_t)S.ns; }
 // oz / oz_rows: slice scratch of FP64 128-tiles on the bf16 tensor cores (null: those
 // tiles run as 64 x 64 DMMA tiles)

@@ -141,8 +141,8 @@ __device__ void stage_rows(P* X, const P* __restrict__ L21, int64_t m, int n, in
 // next to one another, V[row * NR + c], so that one or a few wide loads feed NR
 // multiply-adds; with them apart (V[c * n + row]) every multiply-add had a load of its own.
 // Measured, one solve: 48^3 27-point FP64, 1 right-hand side 11.0 -> 7.9 ms, 16 right-hand sides
-// 68.0 -> 39.1 ms (the FP64 unit's floor is 31 ms); 96^3 diffusion, three FP32 solves of 16
-// right-hand sides with their residuals 123.7 -> 35.6 ms.
+// 68.0 -> 38.2 ms (the FP64 unit's floor is 31 ms); 96^3 diffusion, three FP32 solves of 16
+// right-hand sides with their residuals 123.7 -> 38.4 ms.
 //  * kNarrow (levels whose tasks, times their groups of right-hand sides, fit in one wave):
 //    kWideThreads threads, the task's panel block and Y staged in shared memory with every
 //    copy in flight at once.  A task alone on its SM is bound by its FP64 work and the length of
@@ -170,9 +170,10 @@ __host__ __device__ constexpr int y_threads() { return MODE != kLeaf ? kWideThre
 
 // Lets the next level's CTAs start: on levels of one wave, and with a single right-hand side (with
 // more, a wide level's own work fills the SMs that the next one's waiting CTAs would take: 48^3,
-// 16 right-hand sides, 38.2 ms instead of 39.0; never: 8.8 instead of 7.9 ms for one).
+// 16 right-hand sides, 38.2 ms instead of 39.0, and the 96^3 FP32 refinement of 16 38.4 instead of
+// 39.7; never: 8.8 instead of 7.9 ms for one).
 __device__ __forceinline__ void start_next_level(int nrhs) {
-  if (nrhs == 1 || gridDim.x * gridDim.y <= 152) pdl_launch_dependents();
+  if (nrhs == 1 || gridDim.x * gridDim.y <= kWave) pdl_launch_dependents();
 }
 
 // NR consecutive shared-memory values by the widest loads their row alignment allows.

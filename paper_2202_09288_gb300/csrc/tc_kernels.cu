@@ -345,27 +345,27 @@ __global__ void __launch_bounds__(kTfThreads, 1)
         ord++;
         if (tq >= ntasks) break;
         for (int src = 0; src < t.g && ok; src++) {
-        // the group's earlier chunks' rows first, in their own slice rows; the last chunk's own
-        const int64_t row0 = src < t.g - 1 ? seg.w + (int64_t)src * t.gap : seg.oz;
-        const int nch = (int)(((t.widths >> (8 * src)) & 255u) + kTfChunk - 1) / kTfChunk;
-        const uint8_t* arow = oz + (size_t)(row0 + t.i0) * kOzRowBytes;
-        const uint8_t* brow = oz + (size_t)(row0 + t.k0) * kOzRowBytes;
-        for (int c = 0; c < nch && ok; c++, item++) {
-          const int s = (int)(item % kTfStages);
-          if (item >= kTfStages &&  // the stage's previous MMAs must have read it
-              !tf_wait(smem_u32(&st_empty[s]), (uint32_t)(((item / kTfStages) - 1) & 1))) {
-            ok = false;
-            break;
+          // the group's earlier chunks' rows first, in their own slice rows; the last chunk's own
+          const int64_t row0 = src < t.g - 1 ? seg.w + (int64_t)src * t.gap : seg.oz;
+          const int nch = (int)(((t.widths >> (8 * src)) & 255u) + kTfChunk - 1) / kTfChunk;
+          const uint8_t* arow = oz + (size_t)(row0 + t.i0) * kOzRowBytes;
+          const uint8_t* brow = oz + (size_t)(row0 + t.k0) * kOzRowBytes;
+          for (int c = 0; c < nch && ok; c++, item++) {
+            const int s = (int)(item % kTfStages);
+            if (item >= kTfStages &&  // the stage's previous MMAs must have read it
+                !tf_wait(smem_u32(&st_empty[s]), (uint32_t)(((item / kTfStages) - 1) & 1))) {
+              ok = false;
+              break;
+            }
+            unsigned char* sb = stage_base + (size_t)s * kTfStageBytes;
+            const uint32_t bar = smem_u32(&st_full[s]);
+            tf_expect(bar, kTfStageBytes);
+            tf_bulk_load(smem_u32(sb), arow + (size_t)c * stride, kTfPlane, bar);
+            tf_bulk_load(smem_u32(sb + kTfPlane), arow + (size_t)(pp + c) * stride, kTfPlane, bar);
+            tf_bulk_load(smem_u32(sb + 2 * kTfPlane), brow + (size_t)c * stride, kTfPlane, bar);
+            tf_bulk_load(smem_u32(sb + 3 * kTfPlane), brow + (size_t)(pp + c) * stride, kTfPlane,
+                         bar);
           }
-          unsigned char* sb = stage_base + (size_t)s * kTfStageBytes;
-          const uint32_t bar = smem_u32(&st_full[s]);
-          tf_expect(bar, kTfStageBytes);
-          tf_bulk_load(smem_u32(sb), arow + (size_t)c * stride, kTfPlane, bar);
-          tf_bulk_load(smem_u32(sb + kTfPlane), arow + (size_t)(pp + c) * stride, kTfPlane, bar);
-          tf_bulk_load(smem_u32(sb + 2 * kTfPlane), brow + (size_t)c * stride, kTfPlane, bar);
-          tf_bulk_load(smem_u32(sb + 3 * kTfPlane), brow + (size_t)(pp + c) * stride, kTfPlane,
-                       bar);
-        }
         }
         if (!ok) break;
         tq = gridDim.x >= ntasks ? ntasks : (int)gridDim.x + atomicAdd(queue, 1);
@@ -396,30 +396,30 @@ __global__ void __launch_bounds__(kTfThreads, 1)
         const uint32_t widths = ring[ord % kTfRing].widths;
         const int acc = ord % kTfSlots;
         for (int src = 0; src < g && ok; src++) {
-        const int n = (int)((widths >> (8 * src)) & 255u);
-        const int nch = (n + kTfChunk - 1) / kTfChunk;
-        for (int c = 0; c < nch; c++, done++) {
-          const int s = (int)(done % kTfStages);
-          if (!tf_wait(smem_u32(&st_full[s]), (uint32_t)((done / kTfStages) & 1)) ||
-              (src == 0 && c == 0 && ord >= kTfSlots &&  // wait for the drain of the slot
-               !tf_wait(smem_u32(&acc_empty[acc]), (uint32_t)(((ord / kTfSlots) - 1) & 1)))) {
-            ok = false;
-            break;
+          const int n = (int)((widths >> (8 * src)) & 255u);
+          const int nch = (n + kTfChunk - 1) / kTfChunk;
+          for (int c = 0; c < nch; c++, done++) {
+            const int s = (int)(done % kTfStages);
+            if (!tf_wait(smem_u32(&st_full[s]), (uint32_t)((done / kTfStages) & 1)) ||
+                (src == 0 && c == 0 && ord >= kTfSlots &&  // wait for the drain of the slot
+                 !tf_wait(smem_u32(&acc_empty[acc]), (uint32_t)(((ord / kTfSlots) - 1) & 1)))) {
+              ok = false;
+              break;
+            }
+            asm volatile("tcgen05.fence::after_thread_sync;");
+            const int kw = min(kTfChunk, n - kTfChunk * c);
+            const uint32_t sa = smem_u32(stage_base + (size_t)s * kTfStageBytes);
+            const uint64_t ahi = tf_desc(sa), alo = tf_desc(sa + kTfPlane);
+            const uint64_t bhi = tf_desc(sa + 2 * kTfPlane), blo = tf_desc(sa + 3 * kTfPlane);
+            const uint32_t dt = tmem + (uint32_t)(acc * kTfM);
+            for (int kk = 0; kk < (kw + 7) / 8; kk++) {  // K steps of 8 TF32 = 32 bytes
+              tf_mma(dt, ahi + 2 * kk, bhi + 2 * kk, idesc, (src > 0 || c > 0 || kk > 0) ? 1u : 0u);
+              tf_mma(dt, ahi + 2 * kk, blo + 2 * kk, idesc, 1u);
+              tf_mma(dt, alo + 2 * kk, bhi + 2 * kk, idesc, 1u);
+            }
+            tf_commit(smem_u32(&st_empty[s]));  // the stage is free once these MMAs are done
+            if (src + 1 == g && c + 1 == nch) tf_commit(smem_u32(&acc_full[acc]));
           }
-          asm volatile("tcgen05.fence::after_thread_sync;");
-          const int kw = min(kTfChunk, n - kTfChunk * c);
-          const uint32_t sa = smem_u32(stage_base + (size_t)s * kTfStageBytes);
-          const uint64_t ahi = tf_desc(sa), alo = tf_desc(sa + kTfPlane);
-          const uint64_t bhi = tf_desc(sa + 2 * kTfPlane), blo = tf_desc(sa + 3 * kTfPlane);
-          const uint32_t dt = tmem + (uint32_t)(acc * kTfM);
-          for (int kk = 0; kk < (kw + 7) / 8; kk++) {  // K steps of 8 TF32 = 32 bytes
-            tf_mma(dt, ahi + 2 * kk, bhi + 2 * kk, idesc, (src > 0 || c > 0 || kk > 0) ? 1u : 0u);
-            tf_mma(dt, ahi + 2 * kk, blo + 2 * kk, idesc, 1u);
-            tf_mma(dt, alo + 2 * kk, bhi + 2 * kk, idesc, 1u);
-          }
-          tf_commit(smem_u32(&st_empty[s]));  // the stage is free once these MMAs are done
-          if (src + 1 == g && c + 1 == nch) tf_commit(smem_u32(&acc_full[acc]));
-        }
         }
       }
       if (!ok) s_fail = 1;

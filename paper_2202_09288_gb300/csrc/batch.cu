@@ -164,7 +164,9 @@ int chol_batch_create(chol_ctx* c, int count, chol_num* const* nums, chol_batch*
   }
   // FP64 tensor-core Schur tiles: each member's slice rows of a level follow the previous
   // members' in one batch scratch
-  const bool oz = b->f32 || use_oz(c, nums[0]->sym);  // tensor-core 128-tiles need the scratch
+  // (if every member's supernodes fit the slices' rows of 64 columns: its tasks share the launches)
+  bool oz = true;
+  for (int i = 0; i < count; i++) oz = oz && (b->f32 || use_oz(c, nums[i]->sym));
   // FP64: the inverses' slices of the tensor-core TRSM follow the same pattern (every member
   // keeps its inverses when W <= kDinvMaxWidth, which the tensor-core tiles imply)
   bool oy = !b->f32 && oz;

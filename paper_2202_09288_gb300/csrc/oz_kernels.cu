@@ -435,14 +435,11 @@ __global__ void __launch_bounds__(kOzThreads, 1)
   __shared__ int s_fail;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   pdl_wait();
-  // a launch of an earlier level of this factorization already gave up on a wait: its
-  // updates are missing and the factorization is reported failed, so skip the work (before
-  // any barrier or tensor memory is set up); the whole CTA, or none of it: another CTA may be
-  // recording a timeout of this launch
-  if (__syncthreads_or(*(volatile unsigned long long*)(mats[sns[segs[0].s].mat].err + 3) != 0)) {
-    record_timeout(nsegs, sns, mats, [&](int i) { return segs[i].s; });
-    return;
-  }
+  // a launch of this factorization already gave up on a wait: its updates are missing and the
+  // factorization is reported failed, so skip the work below -- the whole CTA, or none of it
+  // (another CTA may be recording a timeout of this launch): decided at the set-up's barrier, which the
+  // loads' way there overlaps (a barrier of its own took 1 us a launch, 49.5 -> 49.75 ms at 48^3)
+  const bool gave_up = *(volatile unsigned long long*)(mats[sns[segs[0].s].mat].err + 3) != 0;
   const size_t stride = (size_t)oz_rows * kOzRowBytes;
   const int32_t* exps = reinterpret_cast<const int32_t*>(oz + kOzSlices * stride);
 
@@ -475,9 +472,17 @@ __global__ void __launch_bounds__(kOzThreads, 1)
     asm volatile("fence.mbarrier_init.release.cluster;");
   }
   asm volatile("tcgen05.fence::before_thread_sync;");
-  __syncthreads();
+  const bool skip = __syncthreads_or(gave_up);
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = tmem_base;
+  if (skip) {
+    record_timeout(nsegs, sns, mats, [&](int i) { return segs[i].s; });
+    __syncwarp();
+    if (warp == 0)
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                   "r"(kOzTmemCols));
+    return;
+  }
 
   if (warp == kOzLoadWarp) {
     // ---------------- loads: task claims, ring, tiled copies; one thread ----------------
@@ -959,11 +964,8 @@ __global__ void __launch_bounds__(kToThreads, 1)
   const int e0 = (int)((long long)ntasks * blockIdx.x / gridDim.x);
   const int e1 = (int)((long long)ntasks * (blockIdx.x + 1) / gridDim.x);
   pdl_wait();
-  // a launch of this factorization already gave up on a wait: skip (before any set-up)
-  if (__syncthreads_or(*(volatile unsigned long long*)(mats[sns[tasks[e0].x].mat].err + 3) != 0)) {
-    record_timeout(e1 - e0, sns, mats, [&](int i) { return tasks[e0 + i].x; });
-    return;
-  }
+  // a launch of this factorization already gave up on a wait: skip (as in k_schur_oz)
+  const bool gave_up = *(volatile unsigned long long*)(mats[sns[tasks[e0].x].mat].err + 3) != 0;
   const size_t sa = (size_t)oz_rows * kOzRowBytes, sb = (size_t)oy_rows * kOzRowBytes;
   const int32_t* ea = reinterpret_cast<const int32_t*>(oz + kOzSlices * sa);
   const int32_t* ey = reinterpret_cast<const int32_t*>(oy + kOzSlices * sb);
@@ -981,9 +983,17 @@ __global__ void __launch_bounds__(kToThreads, 1)
     asm volatile("fence.mbarrier_init.release.cluster;");
   }
   asm volatile("tcgen05.fence::before_thread_sync;");
-  __syncthreads();
+  const bool skip = __syncthreads_or(gave_up);
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = tmem_base;
+  if (skip) {
+    record_timeout(e1 - e0, sns, mats, [&](int i) { return tasks[e0 + i].x; });
+    __syncwarp();
+    if (warp == 0)
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                   "r"(kToTmemCols));
+    return;
+  }
   if (warp == kToWarps) {
     if (lane == 0) {
       const uint32_t fb = smem_u32(&full), db = smem_u32(&done);

@@ -110,7 +110,7 @@ class ClockSampler:
 KERNEL_SOURCES = ("factor_kernels.cu", "oz_kernels.cu", "tc_kernels.cu", "device_common.cuh",
                   "chol_internal.h")
 # the source files that define each traced kernel kind (its device code and shared helpers)
-KIND_SOURCES = {"schur128_oz": ("oz_kernels.cu", "device_common.cuh"),
+KIND_SOURCES = {"schur128_oz": ("oz_kernels.cu", "oz_combine.h", "device_common.cuh"),
                 "schur128_tc": ("tc_kernels.cu", "device_common.cuh")}
 
 

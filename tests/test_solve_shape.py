@@ -6,7 +6,6 @@ import ctypes
 import os
 import subprocess
 
-import numpy as np
 import pytest
 
 import paper_2202_09288_gb300 as P
